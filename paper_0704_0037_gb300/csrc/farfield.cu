@@ -1,0 +1,439 @@
+// Far-field sums of dda_scatter as exact integer matrix products on the
+// tensor cores (arXiv:0704.0037, Sec. 3.1: amplitudes in many directions).
+//
+//   S_c(n_d) = sum_j P_c,j exp(-i kd n_d . r_j)
+//
+// The phase factorises over the axes.  Along x the cells are folded about the
+// box centre, with S = P(x) + P(-x) and D = P(x) - P(-x):
+//   sum_x P e^{-i phi} = sum_{x > 0} (S cos phi - i D sin phi),
+// so a row of the lattice is a real product of [S.re | D.im] (real part) and
+// [S.im | -D.re] (imaginary part) with the columns [cos | sin] of the
+// directions: a matrix product whose rows are (lattice row, component, part),
+// whose columns are the directions and whose inner length is n_x.
+//
+// On this part the FP64 pipe does 2 fused multiply-adds per clock and SM, and
+// the direct sum (22 FP64 operations per dipole and direction) is bound by it.
+// So the product runs on the bf16 tensor cores without rounding (Ozaki's
+// error-free splitting of a matrix product): both factors are fixed-point
+// numbers of 55 bits, relative to the largest entry of their (lattice row,
+// component) and to 1, cut into seven signed 8-bit digits that bf16 holds
+// exactly; the products of digits i and j with i + j = g go to accumulator g
+// (28 of the 49 pairs, g <= 6: what is left out lies below 2^-53 of the
+// row's scale).  A product of two digits is at most 2^14 and accumulator g
+// adds at most (g + 1) K <= 7 * 144 of them, below 2^24: every FP32 sum of the
+// tensor cores is exact.  The seven accumulators are put together in 64-bit
+// integers; FP64 work is left only for the (y, z) phase of each row.
+//
+// One block holds the digits of 16 lattice rows (96 matrix rows, up to 144
+// inner columns: 193 KB) in shared memory, in the order the tensor-core
+// fragments are loaded, and runs all directions past them in tiles of 32,
+// whose digits stream through a three-stage ring.  12 warps: 6 tiles of 16
+// matrix rows (8 lattice rows, real and imaginary part, of one component)
+// times two halves of the directions; a warp reuses its 14 fragment loads for
+// 56 matrix instructions.
+//
+// 128^3 sphere, 1,152 directions: 65.4 ms with direct FP64 sums, 3.26 ms here (the
+// whole two-polarisation dda_scatter 131.6 -> 7.0 ms), error against 64-bit
+// sums 2.0e-15 before, 1.9e-15 now.
+#include <algorithm>
+
+#include "internal.h"
+
+#include <cuda_bf16.h>
+
+namespace dda {
+namespace {
+
+constexpr int kSl = 7;            // digits per number
+constexpr int kRows = 16;         // lattice rows per block
+constexpr int kDirs = 32;         // directions per tile
+constexpr int kJMax = 72;         // folded cells per chunk: 2 * 72 = 144 inner columns
+constexpr int kNT = 384;          // threads
+constexpr int kBBlk = kSl * 1024; // bytes of one 16-column step of a direction tile
+constexpr int kFix = 54;          // |value| <= 2^54 in fixed point
+
+// inner dimension: H = ceil(nx / 2) folded cells in nchunk chunks of J, each
+// ks steps of 16 columns (2 J padded with zeros)
+struct FfShape { int H, J, nchunk, ks; };
+
+// t = sum of dg[i] 256^(6 - i), -128 <= dg[i] <= 127 for i > 0
+__device__ __forceinline__ void digits(long long t, int (&dg)[kSl]) {
+#pragma unroll
+  for (int i = kSl - 1; i > 0; --i) {
+    const int d = (int)(signed char)(t & 0xff);
+    dg[i] = d;
+    t = (t - d) >> 8;
+  }
+  dg[0] = (int)t;
+}
+__device__ __forceinline__ unsigned pack2(int a, int b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn((float)a, (float)b);
+  return *reinterpret_cast<const unsigned*>(&v);
+}
+__device__ __forceinline__ double pow2(int e) {   // 2^e, -1022 <= e <= 1023
+  return __hiloint2double((e + 1023) << 20, 0);
+}
+
+// exp(-i kd n_mu r_mu) for the cells of x, then y, then z: tab[cell][n_dir]
+__global__ void k_ff_tab(const double* __restrict__ dirs, int n_dir, double kd, int nx, int ny,
+                         int nz, c128* __restrict__ tab) {
+  const int L = nx + ny + nz;
+  const long long total = (long long)n_dir * L;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    int k = (int)(i / n_dir);
+    const int d = (int)(i - (long long)k * n_dir);
+    int axis = 0, n = nx;
+    if (k >= nx) { k -= nx; axis = 1; n = ny; if (k >= ny) { k -= ny; axis = 2; n = nz; } }
+    const double r = 0.5 * (2 * k + 1 - n);
+    double s, c;
+    sincos(-kd * dirs[3 * d + axis] * r, &s, &c);
+    tab[i] = mk<double>(c, s);
+  }
+}
+
+// Digits of [cos | sin] in fragment order: block (chunk, tile, step) of kBBlk
+// bytes, then digit, half of the tile, lane, 8-direction group, k half
+__global__ void k_ff_pack(const c128* __restrict__ tab, int n_dir, int nx, FfShape sh, int ntiles,
+                          unsigned* __restrict__ B) {
+  const long long total = (long long)sh.nchunk * ntiles * sh.ks * 256;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    const int w = (int)(i & 255);
+    const long long blk = i >> 8;
+    const int s = (int)(blk % sh.ks);
+    const int tile = (int)((blk / sh.ks) % ntiles), ch = (int)(blk / ((long long)sh.ks * ntiles));
+    const int half = w >> 7, lane = (w >> 2) & 31, nt = (w >> 1) & 1, b = w & 1;
+    const int d = tile * kDirs + half * 16 + nt * 8 + (lane >> 2);
+    int dg[2][kSl];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int k = s * 16 + (lane & 3) * 2 + b * 8 + u;
+      const int j = ch * sh.J + (k < sh.J ? k : k - sh.J);
+      double v = 0.0;
+      if (k < 2 * sh.J && j < sh.H && d < n_dir) {
+        const c128 t = tab[(long long)(nx - sh.H + j) * n_dir + d];
+        v = k < sh.J ? t.x : -t.y;
+      }
+      digits(__double2ll_rn(v * pow2(kFix)), dg[u]);
+    }
+    unsigned* o = B + blk * (kBBlk / 4) + w;
+#pragma unroll
+    for (int q = 0; q < kSl; ++q) o[q * 256] = pack2(dg[0][q], dg[1][q]);
+  }
+}
+
+__device__ __forceinline__ void mma(float (&c)[4], const uint4& a, unsigned b0, unsigned b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+               "{%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void copy16(void* smem, const void* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+
+// shared memory behind the A digits: the gather stage of the build phase
+// (12 warps x 2 J cells), then ring (3 steps), row phases and the row-group
+// reduction of the product phase
+constexpr int kRing = 3 * kBBlk;
+constexpr int kWBytes = kRows * kDirs * 16;
+constexpr int kRedBytes = 3 * kDirs * 2 * 8;
+constexpr int kTail = kRing + kWBytes + kRedBytes;
+static_assert(12 * 2 * kJMax * 16 <= kTail, "the gather stage fits behind the digits");
+
+// Partial sums of the row blocks u = blockIdx.x, + gridDim.x, ... (of units =
+// row blocks x chunks) for the direction tiles of blockIdx.y:
+// part[blockIdx.x][n_dir][6] (components, re/im).  Rows are those of lat.arow
+// (or all nr rows).
+__global__ void __launch_bounds__(kNT, 1)
+    k_ff_mma(const c128* __restrict__ P, LatticeDev lat, const c128* __restrict__ tab,
+             const unsigned char* __restrict__ B, int n_dir, int nx, int ny, int nr, long long n_occ,
+             FfShape sh, int ntiles, int tiles_per_y, int units, double* __restrict__ part) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ double s_sc[kRows * 3];
+  __shared__ int s_iy[kRows], s_iz[kRows];
+  const int abytes = 6 * sh.ks * kSl * 512;
+  unsigned* A = reinterpret_cast<unsigned*>(smem);
+  unsigned char* tail = smem + abytes;
+  c128* s_w = reinterpret_cast<c128*>(tail + kRing);
+  double* s_red = reinterpret_cast<double*>(tail + kRing + kWBytes);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int mt = warp % 6, half = warp / 6, rg = mt / 3, comp = mt % 3;
+  const int g = lane >> 2;
+  const int t0 = blockIdx.y * tiles_per_y, t1 = min(ntiles, t0 + tiles_per_y);
+  const long long* off = lat.arow ? lat.aoff : lat.row_off;
+
+  for (int u = blockIdx.x; u < units; u += gridDim.x) {
+    const int rb = u / sh.nchunk, ch = u - rb * sh.nchunk, j0 = ch * sh.J;
+    __syncthreads();                         // the previous unit's reads of A, W and the ring
+    // ---- digits of the 16 rows: a warp per (row, component)
+    c128* stage = reinterpret_cast<c128*>(tail) + warp * 2 * kJMax;
+    for (int p = warp; p < 3 * kRows; p += kNT / 32) {
+      const int r = p / 3, c = p - 3 * r, ri = rb * kRows + r;
+      for (int k = lane; k < 2 * sh.J; k += 32) stage[k] = mk<double>(0.0, 0.0);
+      __syncwarp();
+      if (ri < nr) {
+        const long long s1 = off[ri + 1];
+        for (long long i = off[ri] + lane; i < s1; i += 32) {
+          const int x = lat.xi[i], hi = x - (nx - sh.H);
+          const int j = (hi >= 0 ? hi : (nx & 1) - 1 - hi) - j0;
+          if (j >= 0 && j < sh.J) stage[hi >= 0 ? j : sh.J + j] = P[c * n_occ + i];
+        }
+      }
+      if (c == 0 && lane == 0) {
+        const int row = ri < nr ? (lat.arow ? lat.arow[ri] : ri) : 0;
+        s_iy[r] = row % ny;
+        s_iz[r] = row / ny;
+      }
+      __syncwarp();
+      double m = 0.0;
+      bool bad = false;
+      for (int k = lane; k < sh.J; k += 32) {
+        const c128 h = stage[k], l = stage[sh.J + k];
+        const c128 s = h + l, d = h - l;
+        const double a = fmax(fmax(fabs(s.x), fabs(s.y)), fmax(fabs(d.x), fabs(d.y)));
+        bad |= !(isfinite(s.x) && isfinite(s.y) && isfinite(d.x) && isfinite(d.y));
+        m = fmax(m, a);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+      bad = __any_sync(0xffffffffu, bad);
+      // |values| <= m < 2^e (e no smaller than -900: below that the row counts as tiny)
+      const int e = max(((__double2hiint(m) >> 20) & 0x7ff) - 1022, -900);
+      const double scale = (m > 0.0 && !bad) ? pow2(kFix - e) : 0.0;
+      if (lane == 0) s_sc[p] = bad ? nan("") : pow2(e - 56);
+      const int pmt = (r >> 3) * 3 + c, pg = r & 7;
+      for (int kp = lane; kp < sh.ks * 8; kp += 32) {
+        int dr[2][kSl], di[2][kSl];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int k = 2 * kp + q;
+          double re = 0.0, im = 0.0;
+          if (k < sh.J) {
+            const c128 s = stage[k] + stage[sh.J + k];
+            re = s.x; im = s.y;
+          } else if (k < 2 * sh.J) {
+            const c128 d = stage[k - sh.J] - stage[k];
+            re = d.y; im = -d.x;
+          }
+          if (bad) re = im = 0.0;
+          digits(__double2ll_rn(re * scale), dr[q]);
+          digits(__double2ll_rn(im * scale), di[q]);
+        }
+        const int s = kp >> 3, kin = (2 * kp) & 15;
+        uint2* o = reinterpret_cast<uint2*>(A + ((pmt * sh.ks + s) * kSl) * 128 +
+                                            (pg * 4 + ((kin & 7) >> 1)) * 4 + (kin >= 8 ? 2 : 0));
+#pragma unroll
+        for (int q = 0; q < kSl; ++q) o[q * 64] = make_uint2(pack2(dr[0][q], dr[1][q]), pack2(di[0][q], di[1][q]));
+      }
+      __syncwarp();
+    }
+    __syncthreads();
+    // ---- the product with tiles t0 .. t1 - 1, one step of 16 columns at a time
+    const double sc = s_sc[(rg * 8 + g) * 3 + comp];
+    const int q0 = (ch * ntiles + t0) * sh.ks, q1 = (ch * ntiles + t1) * sh.ks;
+    auto fetch = [&](int q) {
+      if (q < q1) {
+        const unsigned char* src = B + (size_t)q * kBBlk;
+        unsigned char* dst = tail + ((q - q0) % 3) * kBBlk;
+        for (int i = threadIdx.x; i < kBBlk / 16; i += kNT) copy16(dst + 16 * i, src + 16 * i);
+      }
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    fetch(q0);
+    fetch(q0 + 1);
+    int q = q0;
+    for (int tile = t0; tile < t1; ++tile) {
+      for (int i = threadIdx.x; i < kRows * kDirs; i += kNT) {
+        const int r = i / kDirs, d = tile * kDirs + i % kDirs;
+        c128 w = mk<double>(0.0, 0.0);
+        if (rb * kRows + r < nr && d < n_dir)
+          w = tab[(long long)(nx + s_iy[r]) * n_dir + d] * tab[(long long)(nx + ny + s_iz[r]) * n_dir + d];
+        s_w[i] = w;
+      }
+      float acc[2][kSl][4];
+#pragma unroll
+      for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int k = 0; k < kSl; ++k)
+#pragma unroll
+          for (int v = 0; v < 4; ++v) acc[n][k][v] = 0.0f;
+      for (int s = 0; s < sh.ks; ++s, ++q) {
+        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        __syncthreads();
+        fetch(q + 2);
+        const uint4* a4 = reinterpret_cast<const uint4*>(A) + (mt * sh.ks + s) * kSl * 32 + lane;
+        const uint4* b4 = reinterpret_cast<const uint4*>(tail + ((q - q0) % 3) * kBBlk) + half * 32 + lane;
+        uint4 af[kSl], bf[kSl];
+#pragma unroll
+        for (int k = 0; k < kSl; ++k) { af[k] = a4[k * 32]; bf[k] = b4[k * 64]; }
+#pragma unroll
+        for (int i = 0; i < kSl; ++i)
+#pragma unroll
+          for (int j = 0; j < kSl - i; ++j) {
+            mma(acc[0][i + j], af[i], bf[j].x, bf[j].y);
+            mma(acc[1][i + j], af[i], bf[j].z, bf[j].w);
+          }
+      }
+      // ---- 64-bit sums, row phases, sum over the 8 rows of the tile
+      double v[2][2][2];                     // [direction group][column][re, im]
+#pragma unroll
+      for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int col = 0; col < 2; ++col) {
+          double z[2];
+#pragma unroll
+          for (int im = 0; im < 2; ++im) {
+            long long t = __float2int_rn(acc[n][0][2 * im + col]);
+#pragma unroll
+            for (int k = 1; k < kSl - 1; ++k) t = t * 256 + __float2int_rn(acc[n][k][2 * im + col]);
+            t = t * 16 + (__float2int_rn(acc[n][kSl - 1][2 * im + col]) >> 4);
+            z[im] = (double)t * sc;
+          }
+          const c128 w = s_w[(rg * 8 + g) * kDirs + half * 16 + n * 8 + (lane & 3) * 2 + col];
+          v[n][col][0] = z[0] * w.x - z[1] * w.y;
+          v[n][col][1] = z[0] * w.y + z[1] * w.x;
+        }
+      // lane bit 4 keeps a direction group, bit 3 a column, bit 2 a part
+      double a4v[2][2], a2v[2], a1;
+      const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+#pragma unroll
+      for (int col = 0; col < 2; ++col)
+#pragma unroll
+        for (int im = 0; im < 2; ++im) {
+          const double keep = b4 ? v[1][col][im] : v[0][col][im];
+          const double send = b4 ? v[0][col][im] : v[1][col][im];
+          a4v[col][im] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+        }
+#pragma unroll
+      for (int im = 0; im < 2; ++im) {
+        const double keep = b3 ? a4v[1][im] : a4v[0][im];
+        const double send = b3 ? a4v[0][im] : a4v[1][im];
+        a2v[im] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+      }
+      a1 = (b2 ? a2v[1] : a2v[0]) + __shfl_xor_sync(0xffffffffu, b2 ? a2v[0] : a2v[1], 4);
+      const int dl = half * 16 + (b4 ? 8 : 0) + (lane & 3) * 2 + (b3 ? 1 : 0);
+      const int slot = (comp * kDirs + dl) * 2 + (b2 ? 1 : 0);
+      if (rg == 1) s_red[slot] = a1;
+      __syncthreads();
+      const int d = tile * kDirs + dl;
+      if (rg == 0 && d < n_dir) {
+        a1 += s_red[slot];
+        double* o = part + ((long long)blockIdx.x * n_dir + d) * 6 + 2 * comp + (b2 ? 1 : 0);
+        *o = u == (int)blockIdx.x ? a1 : *o + a1;
+      }
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  }
+}
+
+// F(n_d) from the nb partials (fixed order), then the transverse projection:
+// 8 directions per block, 8 strided sums per value
+__global__ void __launch_bounds__(384) k_ff_fin(const double* __restrict__ part, int nb, int n_dir,
+                                                const double* __restrict__ dirs, double kd,
+                                                double* __restrict__ F) {
+  __shared__ double sh[8][48];
+  const int t = threadIdx.x % 48, q = threadIdx.x / 48, d0 = blockIdx.x * 8;
+  const long long n6 = 6LL * n_dir;
+  double s = 0.0;
+  if (6 * d0 + t < n6)
+    for (int b = q; b < nb; b += 8) s += part[b * n6 + 6 * d0 + t];
+  sh[q][t] = s;
+  __syncthreads();
+  if (threadIdx.x < 48) {
+    for (int b = 1; b < 8; ++b) s += sh[b][t];
+    sh[0][t] = s;
+  }
+  __syncthreads();
+  const int d = d0 + threadIdx.x;
+  if (threadIdx.x >= 8 || d >= n_dir) return;
+  const double* a = &sh[0][6 * threadIdx.x];
+  const double nx = dirs[3 * d], ny = dirs[3 * d + 1], nz = dirs[3 * d + 2];
+  const double dr = nx * a[0] + ny * a[2] + nz * a[4];
+  const double di = nx * a[1] + ny * a[3] + nz * a[5];
+  const double n3[3] = {nx, ny, nz};
+  const double k3 = kd * kd * kd;
+  for (int c = 0; c < 3; ++c) {
+    const double tr = a[2 * c] - n3[c] * dr;
+    const double ti = a[2 * c + 1] - n3[c] * di;
+    // -i k3 (tr + i ti) = k3 ti - i k3 tr
+    F[6 * d + 2 * c] = k3 * ti;
+    F[6 * d + 2 * c + 1] = -k3 * tr;
+  }
+}
+
+FfShape ff_shape(int nx) {
+  FfShape s;
+  s.H = (nx + 1) / 2;
+  s.nchunk = (s.H + kJMax - 1) / kJMax;
+  s.J = (s.H + s.nchunk - 1) / s.nchunk;
+  s.ks = (2 * s.J + 15) / 16;
+  return s;
+}
+
+// row blocks in flight: one block per SM, no more than there are units, and
+// partial sums of at most 64 MB
+int ff_groups(int units, int n_dir) {
+  const long long fit = std::max(1LL, (64LL << 20) / (48LL * n_dir));
+  return (int)std::min<long long>(std::min(units, num_sms()), fit);
+}
+
+size_t up256(size_t b) { return (b + 255) / 256 * 256; }
+
+}  // namespace
+
+FarfieldPlan farfield_plan(int n_dir, int nx, int ny, int nz, int nr) {
+  const FfShape s = ff_shape(nx);
+  const int nt = (n_dir + kDirs - 1) / kDirs;
+  const int units = ((nr + kRows - 1) / kRows) * s.nchunk;
+  FarfieldPlan p;
+  p.tab = up256((size_t)n_dir * (nx + ny + nz) * sizeof(c128));
+  p.pack = (size_t)s.nchunk * nt * s.ks * kBBlk;
+  p.part = up256((size_t)ff_groups(units, n_dir) * n_dir * 6 * sizeof(double));
+  return p;
+}
+
+cudaError_t farfield_tables(void* ws, const double* dirs, int n_dir, double kd, int nx, int ny, int nz,
+                            const FarfieldPlan& p, cudaStream_t st) {
+  const FfShape s = ff_shape(nx);
+  const int nt = (n_dir + kDirs - 1) / kDirs;
+  c128* tab = (c128*)ws;
+  unsigned* pack = (unsigned*)((unsigned char*)ws + p.tab);
+  const long long tt = (long long)n_dir * (nx + ny + nz), tp = (long long)s.nchunk * nt * s.ks * 256;
+  k_ff_tab<<<(int)std::min<long long>((tt + 255) / 256, 8192), 256, 0, st>>>(dirs, n_dir, kd, nx, ny, nz, tab);
+  count_launch();
+  k_ff_pack<<<(int)std::min<long long>((tp + 255) / 256, 8192), 256, 0, st>>>(tab, n_dir, nx, s, nt, pack);
+  count_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t farfield_sums(void* ws, const c128* P, const LatticeDev& lat, const double* dirs, int n_dir,
+                          double kd, int nx, int ny, int nr, long long n_occ, const FarfieldPlan& p,
+                          double* F, cudaStream_t st) {
+  const FfShape s = ff_shape(nx);
+  const int nt = (n_dir + kDirs - 1) / kDirs;
+  const int units = ((nr + kRows - 1) / kRows) * s.nchunk;
+  const int G = ff_groups(units, n_dir);
+  const c128* tab = (const c128*)ws;
+  const unsigned char* pack = (const unsigned char*)ws + p.tab;
+  double* part = (double*)((unsigned char*)ws + p.tab + p.pack);
+  // direction tiles split over blockIdx.y: enough blocks for every SM and,
+  // where the row blocks do not divide evenly over the SMs, finer pieces (of
+  // 8 tiles at least, over which the digits of a row block are made once)
+  const int want = G < num_sms() ? (num_sms() + G - 1) / G : 4;
+  const int ny_ = std::max(1, std::min(want, G < num_sms() ? nt : (nt + 7) / 8));
+  const int per = (nt + ny_ - 1) / ny_;
+  const size_t sm = (size_t)6 * s.ks * kSl * 512 + kTail;
+  cudaError_t e = ensure_smem((const void*)k_ff_mma, sm);
+  if (e != cudaSuccess) return e;
+  k_ff_mma<<<dim3(G, (nt + per - 1) / per), kNT, sm, st>>>(P, lat, tab, pack, n_dir, nx, ny, nr, n_occ, s,
+                                                          nt, per, units, part);
+  count_launch();
+  k_ff_fin<<<(n_dir + 7) / 8, 384, 0, st>>>(part, G, n_dir, dirs, kd, F);
+  count_launch();
+  return cudaGetLastError();
+}
+
+}  // namespace dda

@@ -252,7 +252,22 @@ long long launch_total();
 }  // namespace dda
 
 namespace dda {
-// Far-field kernels (scatter.cu), shared with the allocation-free entry point.
+// Far-field sums of dda_scatter (farfield.cu): workspace of one call for n_dir
+// directions on a lattice of nx x ny x nz cells with nr rows (phase tables,
+// their digits, partial sums), the direction tables, and the amplitudes F
+// [n_dir][6] of one polarization P from them.
+struct FarfieldPlan {
+  size_t tab, pack, part;
+  size_t bytes() const { return tab + pack + part; }
+};
+FarfieldPlan farfield_plan(int n_dir, int nx, int ny, int nz, int nr);
+cudaError_t farfield_tables(void* ws, const double* dirs, int n_dir, double kd, int nx, int ny, int nz,
+                            const FarfieldPlan& p, cudaStream_t st);
+cudaError_t farfield_sums(void* ws, const c128* P, const LatticeDev& lat, const double* dirs, int n_dir,
+                          double kd, int nx, int ny, int nr, long long n_occ, const FarfieldPlan& p,
+                          double* F, cudaStream_t st);
+
+// Direct far-field kernels (scatter.cu) of the allocation-free entry point.
 constexpr int kFarfieldDB = 4;   // directions per block of k_farfield
 __global__ void k_phase_tab(const double* dirs, int n_dir, double kd, int nx, int ny, int nz,
                             c128* tab);

@@ -165,6 +165,7 @@ __global__ void k_collapse_fin(const c128* __restrict__ part, int G, long long n
 struct Wave2 { double a[3]; double e[6]; };
 
 constexpr int kCollapseG = 8;   // y groups of the collapse (partials per (x, z))
+constexpr int kDirBlock = 8192; // directions whose phase tables are held at once
 
 // per-row-chunk partials of sum Im(E_inc^* . P) and sum w |P|^2.  ptab holds
 // exp(-i kd a_mu r_mu) along x, then y, then z (k_phase_tab for the incidence
@@ -184,22 +185,29 @@ __global__ void __launch_bounds__(256) k_qsums(const c128* __restrict__ P, Latti
     wab[i] = al.y / (al.x * al.x + al.y * al.y) - (2.0 / 3.0) * k3;
   }
   __syncthreads();
-  // E = e exp(i phi); E^* . P = conj(e) exp(-i phi) P
+  // E = e exp(i phi); E^* . P = conj(e) exp(-i phi) P.  The (y, z) phase of a
+  // row multiplies its sum once, and a real e (linear polarisation) takes half
+  // the products: the sweep is bound by the FP64 pipe
   const c128 e0 = mk<double>(w.e[0], -w.e[1]), e1 = mk<double>(w.e[2], -w.e[3]),
              e2 = mk<double>(w.e[4], -w.e[5]);
+  const bool real_e = w.e[1] == 0.0 && w.e[3] == 0.0 && w.e[5] == 0.0;
   double se = 0.0, sa = 0.0;
   for (int row = blockIdx.x * 8 + wid; row < nrows; row += nwarps) {
     const int iy = row % ny, iz = row / ny;
-    const c128 pyz = ptab[nx + iy] * ptab[nx + ny + iz];
+    c128 sr = mk<double>(0.0, 0.0);
     for (long long i = lat.row_off[row] + lane; i < lat.row_off[row + 1]; i += 32) {
-      const c128 ph = ptab[lat.xi[i]] * pyz;
+      const c128 ph = ptab[lat.xi[i]];
       const int m = lat.mat[i];
       const c128 p0 = P[i], p1 = P[n_occ + i], p2 = P[2 * n_occ + i];
-      const c128 t = (e0 * p0 + e1 * p1 + e2 * p2) * ph;
-      se += t.y;
+      const c128 ep = real_e ? fmas<double>(p2, e2.x, fmas<double>(p1, e1.x, scale<double>(p0, e0.x)))
+                             : e0 * p0 + e1 * p1 + e2 * p2;
+      sr.x += ep.x * ph.x - ep.y * ph.y;
+      sr.y += ep.x * ph.y + ep.y * ph.x;
       sa += wab[3 * m] * (p0.x * p0.x + p0.y * p0.y) + wab[3 * m + 1] * (p1.x * p1.x + p1.y * p1.y) +
             wab[3 * m + 2] * (p2.x * p2.x + p2.y * p2.y);
     }
+    const c128 pyz = ptab[nx + iy] * ptab[nx + ny + iz];
+    se += sr.x * pyz.y + sr.y * pyz.x;
   }
   __shared__ double sh[2][8];
   se = wsum(se); sa = wsum(sa);
@@ -263,20 +271,17 @@ int dda_scatter_internal(dda_t h, int presc, const void* P_dev, int nrhs, const 
     flat.yr = nullptr;
     flat.nact = 0;
   }
-  const int L = fnx + fny + fnz;
   const int qblocks = (int)std::min<long long>((g.nrows + 7) / 8, 1024);
-  int n_chunks = 1, rows_per_chunk = fnrows;
-  if (n_dir > 0) {
-    const int dblocks = (n_dir + kDB - 1) / kDB;
-    n_chunks = std::max(1, std::min((4 * num_sms() + dblocks - 1) / dblocks, (fnrows + 31) / 32));
-    rows_per_chunk = (fnrows + n_chunks - 1) / n_chunks;
-    n_chunks = (fnrows + rows_per_chunk - 1) / rows_per_chunk;
-  }
   const int Lq = g.nx + g.ny + g.nz;   // incidence phase table of the Q sums
-  const size_t tab_b = (size_t)std::max(n_dir, 1) * L * sizeof(c128) + (size_t)Lq * sizeof(c128) +
-                       (size_t)(std::max(n_dir, 1) + 1) * 3 * sizeof(double);
-  const size_t fp_b = std::max((size_t)n_chunks * std::max(n_dir, 1) * 6, (size_t)2 * qblocks) * sizeof(double) +
-                      (size_t)std::max(n_dir, 1) * 6 * sizeof(double);
+  // rows of the far-field lattice that can hold dipoles, and its directions
+  // in blocks of at most kDirBlock (bounded phase tables)
+  const int fnr = flat.arow ? flat.nact : fnrows;
+  const int nblk = n_dir > 0 ? (n_dir + kDirBlock - 1) / kDirBlock : 0;
+  FarfieldPlan plan{};
+  if (n_dir > 0) plan = farfield_plan(std::min(n_dir, kDirBlock), fnx, fny, fnz, fnr);
+  const size_t tab_b = plan.bytes() + (size_t)Lq * sizeof(c128);
+  const size_t fp_b = (size_t)2 * qblocks * sizeof(double) + (size_t)n_dir * 9 * sizeof(double) +
+                      3 * sizeof(double);
   if (h->tab_bytes < tab_b) {
     dev_free(h->d_tab, h->stream); h->d_tab = nullptr; h->tab_bytes = 0;
     if (dev_malloc(&h->d_tab, tab_b) != cudaSuccess) { cudaGetLastError(); return dda_fail(h, DDA_ERR_OOM, "scatter tables"); }
@@ -287,24 +292,26 @@ int dda_scatter_internal(dda_t h, int presc, const void* P_dev, int nrhs, const 
     if (dev_malloc(&h->d_fpart, fp_b) != cudaSuccess) { cudaGetLastError(); return dda_fail(h, DDA_ERR_OOM, "scatter partials"); }
     h->fpart_bytes = fp_b;
   }
-  c128* tab = (c128*)h->d_tab;
-  c128* qtab = tab + (size_t)std::max(n_dir, 1) * L;
-  double* d_dirs = (double*)(qtab + Lq);
-  double* d_qdir = d_dirs + (size_t)std::max(n_dir, 1) * 3;
+  void* ws = h->d_tab;
+  c128* qtab = (c128*)((unsigned char*)ws + plan.bytes());
   double* part = h->d_fpart;
-  double* d_F = part + std::max((size_t)n_chunks * std::max(n_dir, 1) * 6, (size_t)2 * qblocks);
+  double* d_F = part + 2 * qblocks;
+  double* d_dirs = d_F + 6 * (size_t)n_dir;
+  double* d_qdir = d_dirs + 3 * (size_t)n_dir;
+  auto tables = [&](int b) -> cudaError_t {
+    const int d0 = b * kDirBlock, nd = std::min(n_dir - d0, kDirBlock);
+    return farfield_tables(ws, d_dirs + 3 * (size_t)d0, nd, h->kd, fnx, fny, fnz,
+                           farfield_plan(nd, fnx, fny, fnz, fnr), st);
+  };
   if (n_dir > 0) {
     DDA_CK(h, cudaMemcpyAsync(d_dirs, dirs, (size_t)n_dir * 3 * sizeof(double), cudaMemcpyHostToDevice, st));
-    const long long tt = (long long)n_dir * L;
-    k_phase_tab<<<(int)std::min<long long>((tt + 255) / 256, 4096), 256, 0, st>>>(d_dirs, n_dir, h->kd, fnx, fny, fnz, tab); count_launch();
-    DDA_CK(h, cudaGetLastError());
+    if (nblk == 1) DDA_CK(h, tables(0));
   }
   std::vector<double> qp(2 * qblocks);
   for (int r = 0; r < nrhs; ++r) {
     const c128* P = (const c128*)P_dev + (size_t)r * n;
     const c128* beta = h->w64.beta + (long long)r * h->n_mat * 3;
     if (n_dir > 0) {
-      dim3 grid((n_dir + kDB - 1) / kDB, n_chunks);
       tr_begin(g.tr, st);
       const c128* Pf = P;
       if (collapse) {
@@ -315,11 +322,13 @@ int dda_scatter_internal(dda_t h, int presc, const void* P_dev, int nrhs, const 
         k_collapse_fin<<<(int)std::min<long long>((3 * fnocc + 255) / 256, 2048), 256, 0, st>>>(Qpart, G, fnocc, Qc); count_launch();
         Pf = Qc;
       }
-      k_farfield<<<grid, 256, 0, st>>>(Pf, flat, tab, n_dir, fnx, fny, fnz, fnrows, fnocc,
-                                       rows_per_chunk, part); count_launch();
+      for (int b = 0; b < nblk; ++b) {
+        const int d0 = b * kDirBlock, nd = std::min(n_dir - d0, kDirBlock);
+        if (nblk > 1) DDA_CK(h, tables(b));
+        DDA_CK(h, farfield_sums(ws, Pf, flat, d_dirs + 3 * (size_t)d0, nd, h->kd, fnx, fny, fnr, fnocc,
+                                farfield_plan(nd, fnx, fny, fnz, fnr), d_F + 6 * (size_t)d0, st));
+      }
       tr_end(g.tr, st, TR_FARFIELD);
-      k_farfield_fin<<<(n_dir + 127) / 128, 128, 0, st>>>(part, n_chunks, n_dir, d_dirs, h->kd, d_F); count_launch();
-      DDA_CK(h, cudaGetLastError());
       DDA_CK(h, cudaMemcpyAsync(F_out + (size_t)r * n_dir * 6, d_F, (size_t)n_dir * 6 * sizeof(double),
                                 cudaMemcpyDeviceToHost, st));
     }

@@ -1,0 +1,58 @@
+"""GPU parity of the far-field sums (exact digit products on the tensor cores)
+with the oracle's direct sum, at the edges of their tiles: folded rows of one
+cell, odd and even lengths, one and several inner chunks (72 folded cells
+each), row blocks of 16 that are partly filled, and direction tiles of 32.
+
+Tolerance: both sides evaluate the phases in FP64 (|phase| <= kd n: relative
+error of a sum a few 1e-16 times kd n) and sum at FP64 accuracy: 1e-13 of the
+largest amplitude leaves a factor of 20 at the largest case (kd n = 60)."""
+import numpy as np
+import pytest
+
+from oracle import lattice, observables
+from paper_0704_0037_gb300 import inputs
+
+from gpu_util import need_gpu
+
+pytestmark = pytest.mark.gpu
+
+CASES = [  # nx, ny, nz, fill (0: full box), directions
+    (1, 1, 1, 0, 1), (2, 1, 3, 0, 31), (5, 4, 4, 0, 32), (16, 3, 6, 0.4, 33), (15, 7, 5, 0.5, 64),
+    (143, 3, 2, 0.7, 40), (144, 2, 3, 0, 5), (145, 3, 3, 0.3, 70), (300, 2, 2, 0.6, 45),
+    (9, 33, 17, 0.2, 130),
+]
+
+
+@pytest.mark.parametrize("nx,ny,nz,fill,n_dir", CASES)
+def test_farfield_matches_direct_sum(nx, ny, nz, fill, n_dir):
+    torch, dda = need_gpu()
+    occ = inputs.random_occupancy(nx, ny, nz, fill, seed=nx) if fill else inputs.cube(nx, ny, nz)
+    occ[nz // 2, ny // 2, nx // 2] = 1
+    pos = lattice.positions(occ > 0)
+    prop, pol = [[0.0, 0.0, 1.0]] * 2, [[1.0, 0.0, 0.0], [0.0, 1.0, 0.0]]
+    dirs = inputs.random_unit_vectors(n_dir, n_dir)
+    if n_dir % 2:                       # the y-collapsed lattice of in-plane directions
+        dirs[:, 1] = 0.0
+    with dda.Particle(occ, [1.4 + 0.05j], 0.2) as p:
+        x = inputs.random_vectors(3, 2, p.n_occ)
+        x[1, 1] = 0.0                   # a component without any field
+        x[1, 2] *= 10.0 ** np.linspace(-30, 0, p.n_occ)
+        P = torch.from_numpy(x).cuda()
+        F, _ = dda.dda_scatter(p.h, dda.DDA_LDR, P, prop, pol, dirs)
+        again, _ = dda.dda_scatter(p.h, dda.DDA_LDR, P, prop, pol, dirs)
+        assert np.array_equal(F, again)
+        for r in range(2):
+            ref = observables.farfield(x[r], pos, p.kd, dirs)
+            assert np.abs(F[r] - ref).max() <= 1e-13 * np.abs(ref).max()
+
+
+def test_farfield_nonfinite_input_stays_nonfinite():
+    torch, dda = need_gpu()
+    occ = inputs.cube(6, 5, 4)
+    with dda.Particle(occ, [1.4], 0.2) as p:
+        x = inputs.random_vectors(3, 1, p.n_occ)
+        x[0, 0, 7] = np.nan
+        x[0, 1, 9] = np.inf
+        F, q = dda.dda_scatter(p.h, dda.DDA_LDR, torch.from_numpy(x).cuda(), [[0.0, 0.0, 1.0]],
+                               [[1.0, 0.0, 0.0]], inputs.random_unit_vectors(1, 9))
+        assert not np.isfinite(F).any() and not np.isfinite(q[0, 0])
