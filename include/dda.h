@@ -98,9 +98,10 @@ enum dda_prec { DDA_FP64 = 0, DDA_FP32_REFINED = 1, DDA_FP64_PAIR = 2 };
  *   DDA_ERR_CUDA / DDA_ERR_OOM.  Copies what it needs from the host arrays.
  * The FFT passes use register-resident kernels for padded lengths with a
  * compiled split (32, 40, 48, 64, 80, 96, 128, 256, 270; for complex64 also
- * 512 and 1080) and shared-memory Stockham kernels otherwise;
- * dda_set_fft_engine selects the latter for every length.  An axis is padded
- * to the smallest compiled length >= 2n - 1 when that is within 1.35x of the
+ * 512, 1080 and the 7-smooth lengths 135-189 and 280-378 but 343) and
+ * shared-memory Stockham kernels otherwise; dda_set_fft_engine selects the
+ * latter for every length.  An axis is padded to the smallest of the lengths
+ * 32, ..., 270, 512, 1080 that is >= 2n - 1 when it is within 1.35x of the
  * smallest 7-smooth one, else to the 7-smooth one.
  */
 int dda_init_lattice(dda_t* out, int nx, int ny, int nz, const uint8_t* occ_host,

@@ -36,5 +36,32 @@ cudaError_t run_pass(int pass, const FastArgs& a) {
   return cudaErrorNotSupported;
 }
 
+// The product passes alone, default tiles only (lengths without whole-line
+// passes and tile variants)
+template <typename R, int M1, int M2>
+cudaError_t run_product_pass(int pass, const FastArgs& a) {
+  using P = Passes<R, M1, M2>;
+  const cpx<R>* tw = (const cpx<R>*)a.tw;
+  switch (pass) {
+    case FP_XFWD:
+      return P::xfwd((const typename P::V*)a.in, (cpx<R>*)a.out, a.lat, (const cpx<R>*)a.beta, a.n_occ,
+                     a.nrows, tw, a.adj, a.nrhs, a.bstride, a.skip, a.st, a.pdl);
+    case FP_YFWD:
+      return P::template yfwd_t<P::T>((const cpx<R>*)a.in, (cpx<R>*)a.out, a.ny, a.nz, a.Mx, tw, a.nrhs,
+                                      a.skip, a.st, a.pdl, a.lat.yr);
+    case FP_ZCONV:
+      return P::template zconv_t<P::TZ>((cpx<R>*)a.out, (const cpx<R>*)a.D, a.nz, a.Mx, a.My, tw, a.nrhs,
+                                        a.skip, a.st, a.pdl);
+    case FP_YINV:
+      return P::template yinv_t<P::T>((const cpx<R>*)a.in, (cpx<R>*)a.out, a.ny, a.nz, a.Mx, tw, a.nrhs,
+                                      a.skip, a.st, a.pdl);
+    case FP_XINV:
+      return P::xinv((const cpx<R>*)a.in, (const typename P::V*)a.x, (typename P::V*)a.out, a.lat,
+                     (const cpx<R>*)a.beta, a.n_occ, a.nrows, tw, a.adj, a.dotp, a.nrhs, a.bstride,
+                     a.skip, a.st, a.pdl);
+  }
+  return cudaErrorNotSupported;
+}
+
 }  // namespace fast
 }  // namespace dda

@@ -337,9 +337,19 @@ inline int fast_xinv_blocks(int nrows, bool fp32, int Mx) {
 // size of the buffers that receive them)
 inline int fast_xinv_blocks_max(int nrows) { return 3 * ((nrows + 3) / 4); }
 bool fast_supported(int M);          // complex64, complex128 and double-float passes
-bool fast_supported_c64(int M);      // complex64 passes (also 512 and 1080)
+bool fast_supported_c64(int M);      // complex64 passes (also 512, 1080 and the 7-smooth
+                                     // lengths of fast_small.cu's table)
+bool fast_tile_variants(int M);      // lengths whose passes have both tile variants
 cudaError_t fast_pass_512_c64(int pass, const FastArgs& a);
 cudaError_t fast_pass_1080_c64(int pass, const FastArgs& a);
+cudaError_t fast_pass_c64_a(int M, int pass, const FastArgs& a);
+cudaError_t fast_pass_c64_b(int M, int pass, const FastArgs& a);
+cudaError_t fast_pass_c64_c(int M, int pass, const FastArgs& a);
+cudaError_t fast_pass_c64_d(int M, int pass, const FastArgs& a);
+cudaError_t fast_pass_c64_e(int M, int pass, const FastArgs& a);
+cudaError_t fast_pass_c64_f(int M, int pass, const FastArgs& a);
+cudaError_t fast_pass_c64_g(int M, int pass, const FastArgs& a);
+cudaError_t fast_pass_c64_h(int M, int pass, const FastArgs& a);
 template <typename R> cudaError_t fast_pass(int M, int pass, const FastArgs& a);
 template <typename R> cudaError_t fast_pass_270(int pass, const FastArgs& a);
 template <typename R> cudaError_t fast_pass_256(int pass, const FastArgs& a);

@@ -497,7 +497,7 @@ cudaError_t tune_tiles(Geom& g, const LatticeDev& lat, Work<R>& w, cudaStream_t 
   const int kind = std::is_same<R, float>::value ? 0 : std::is_same<R, double>::value ? 1 : 2;
   int* tl = g.tiles[kind];
   if (tl[0] >= 0 && tl[1] >= 0 && tl[2] >= 0) return cudaSuccess;
-  auto has = [](int M) { return std::is_same<R, float>::value ? fast_supported_c64(M) : fast_supported(M); };
+  auto has = [](int M) { return std::is_same<R, float>::value ? fast_tile_variants(M) : fast_supported(M); };
   if (g.engine != 0 || !w.B1 || !w.B2 || !w.D || !w.tw) return cudaSuccess;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -524,7 +524,7 @@ cudaError_t tune_tiles(Geom& g, const LatticeDev& lat, Work<R>& w, cudaStream_t 
   if ((e = cudaEventCreate(&e1)) != cudaSuccess) { cudaEventDestroy(e0); return e; }
   std::array<int, 3> best{0, 0, 0};
   for (int pass = 0; pass < 3 && e == cudaSuccess; ++pass) {
-    if (!has(pass == 1 ? g.Mz : g.My)) continue;       // that axis runs the Stockham passes
+    if (!has(pass == 1 ? g.Mz : g.My)) continue;       // one variant, or the Stockham passes
     float tbest = 0.f;
     for (int var = 0; var < 2 && e == cudaSuccess; ++var) {
       FastArgs a = fa;
