@@ -24,17 +24,19 @@
 // tensor cores is exact.  The seven accumulators are put together in 64-bit
 // integers; FP64 work is left only for the (y, z) phase of each row.
 //
-// One block holds the digits of 16 lattice rows (96 matrix rows, up to 144
-// inner columns: 193 KB) in shared memory, in the order the tensor-core
+// One block holds the digits of 8 lattice rows (48 matrix rows, up to 144
+// inner columns: 97 KB) in shared memory, in the order the tensor-core
 // fragments are loaded, and runs all directions past them in tiles of 32,
-// whose digits stream through a three-stage ring.  12 warps: 6 tiles of 16
-// matrix rows (8 lattice rows, real and imaginary part, of one component)
-// times two halves of the directions; a warp reuses its 14 fragment loads for
-// 56 matrix instructions.
+// whose digits stream through a two-stage ring.  Each of 4 warps takes 8
+// directions against the three tiles of 16 matrix rows (8 lattice rows, real
+// and imaginary part, of one component): 84 matrix instructions for 28
+// fragment loads.  Two blocks share an SM, so that one's sums (FP64 pipe)
+// overlap the other's products (tensor pipe).
 //
-// 128^3 sphere, 1,152 directions: 65.4 ms with direct FP64 sums, 3.26 ms here (the
-// whole two-polarisation dda_scatter 131.6 -> 7.0 ms), error against 64-bit
-// sums 2.0e-15 before, 1.9e-15 now.
+// 128^3 sphere, 1,152 directions, per right-hand side: direct FP64 sums 65.4 ms;
+// this product with 16 rows and 12 warps in one block per SM 3.26 ms, with two
+// blocks and integer scaling 2.58 ms (tensor pipe 42 %, FP64 pipe 43 % busy); error
+// against 64-bit sums 2.0e-15 before, 1.9e-15 now.
 #include <algorithm>
 
 #include "internal.h"
@@ -45,10 +47,10 @@ namespace dda {
 namespace {
 
 constexpr int kSl = 7;            // digits per number
-constexpr int kRows = 16;         // lattice rows per block
+constexpr int kRows = 8;          // lattice rows per block
 constexpr int kDirs = 32;         // directions per tile
 constexpr int kJMax = 72;         // folded cells per chunk: 2 * 72 = 144 inner columns
-constexpr int kNT = 384;          // threads
+constexpr int kNT = 128;          // threads
 constexpr int kBBlk = kSl * 1024; // bytes of one 16-column step of a direction tile
 constexpr int kFix = 54;          // |value| <= 2^54 in fixed point
 
@@ -93,7 +95,7 @@ __global__ void k_ff_tab(const double* __restrict__ dirs, int n_dir, double kd, 
 }
 
 // Digits of [cos | sin] in fragment order: block (chunk, tile, step) of kBBlk
-// bytes, then digit, half of the tile, lane, 8-direction group, k half
+// bytes, then digit, 8-direction group, lane, k half
 __global__ void k_ff_pack(const c128* __restrict__ tab, int n_dir, int nx, FfShape sh, int ntiles,
                           unsigned* __restrict__ B) {
   const long long total = (long long)sh.nchunk * ntiles * sh.ks * 256;
@@ -103,8 +105,8 @@ __global__ void k_ff_pack(const c128* __restrict__ tab, int n_dir, int nx, FfSha
     const long long blk = i >> 8;
     const int s = (int)(blk % sh.ks);
     const int tile = (int)((blk / sh.ks) % ntiles), ch = (int)(blk / ((long long)sh.ks * ntiles));
-    const int half = w >> 7, lane = (w >> 2) & 31, nt = (w >> 1) & 1, b = w & 1;
-    const int d = tile * kDirs + half * 16 + nt * 8 + (lane >> 2);
+    const int lane = (w >> 1) & 31, b = w & 1;
+    const int d = tile * kDirs + (w >> 6) * 8 + (lane >> 2);
     int dg[2][kSl];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
@@ -134,41 +136,46 @@ __device__ __forceinline__ void copy16(void* smem, const void* gmem) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 
-// shared memory behind the A digits: the gather stage of the build phase
-// (12 warps x 2 J cells), then ring (3 steps), row phases and the row-group
-// reduction of the product phase
-constexpr int kRing = 3 * kBBlk;
-constexpr int kWBytes = kRows * kDirs * 16;
-constexpr int kRedBytes = 3 * kDirs * 2 * 8;
-constexpr int kTail = kRing + kWBytes + kRedBytes;
-static_assert(12 * 2 * kJMax * 16 <= kTail, "the gather stage fits behind the digits");
+// t 2^e, rounded to nearest, put together in integer instructions: the FP64
+// pipe, which the row phases need, is left alone.  e keeps the result from
+// underflow; a result of 2^1024 and more becomes non-finite.
+__device__ __forceinline__ double scaled(long long t, int e) {
+  const unsigned long long m = t < 0 ? 0ull - (unsigned long long)t : (unsigned long long)t;
+  const int lz = __clzll((long long)m);
+  const unsigned long long u = m << lz;                       // bit 63 set
+  const unsigned long long v = (u >> 11) + ((u >> 10) & 1);   // 2^52 .. 2^53
+  const unsigned long long bits = ((unsigned long long)min(1085 - lz + e, 2046) << 52) + v;
+  return __longlong_as_double((long long)(t == 0 ? 0ull : bits | ((unsigned long long)t & (1ull << 63))));
+}
+
+// shared memory behind the A digits: ring (2 steps) and row phases; the
+// gather stage of the build phase (4 warps x 2 J cells) lies over the ring
+constexpr int kRing = 2 * kBBlk;
+constexpr int kTail = kRing + kRows * kDirs * 16;
+constexpr int kBad = 1 << 20;     // scale exponent of a row with NaN or infinity
+static_assert(kNT / 32 * 2 * kJMax * 16 <= kTail, "the gather stage fits behind the digits");
 
 // Partial sums of the row blocks u = blockIdx.x, + gridDim.x, ... (of units =
 // row blocks x chunks) for the direction tiles of blockIdx.y:
 // part[blockIdx.x][n_dir][6] (components, re/im).  Rows are those of lat.arow
 // (or all nr rows).
-__global__ void __launch_bounds__(kNT, 1)
+__global__ void __launch_bounds__(kNT, 2)
     k_ff_mma(const c128* __restrict__ P, LatticeDev lat, const c128* __restrict__ tab,
              const unsigned char* __restrict__ B, int n_dir, int nx, int ny, int nr, long long n_occ,
              FfShape sh, int ntiles, int tiles_per_y, int units, double* __restrict__ part) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double s_sc[kRows * 3];
-  __shared__ int s_iy[kRows], s_iz[kRows];
-  const int abytes = 6 * sh.ks * kSl * 512;
+  __shared__ int s_e[kRows * 3], s_iy[kRows], s_iz[kRows];
   unsigned* A = reinterpret_cast<unsigned*>(smem);
-  unsigned char* tail = smem + abytes;
+  unsigned char* tail = smem + 3 * sh.ks * kSl * 512;
   c128* s_w = reinterpret_cast<c128*>(tail + kRing);
-  double* s_red = reinterpret_cast<double*>(tail + kRing + kWBytes);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int mt = warp % 6, half = warp / 6, rg = mt / 3, comp = mt % 3;
-  const int g = lane >> 2;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2;
   const int t0 = blockIdx.y * tiles_per_y, t1 = min(ntiles, t0 + tiles_per_y);
   const long long* off = lat.arow ? lat.aoff : lat.row_off;
 
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
     const int rb = u / sh.nchunk, ch = u - rb * sh.nchunk, j0 = ch * sh.J;
     __syncthreads();                         // the previous unit's reads of A, W and the ring
-    // ---- digits of the 16 rows: a warp per (row, component)
+    // ---- digits of the 8 rows: a warp per (row, component)
     c128* stage = reinterpret_cast<c128*>(tail) + warp * 2 * kJMax;
     for (int p = warp; p < 3 * kRows; p += kNT / 32) {
       const int r = p / 3, c = p - 3 * r, ri = rb * kRows + r;
@@ -203,8 +210,7 @@ __global__ void __launch_bounds__(kNT, 1)
       // |values| <= m < 2^e (e no smaller than -900: below that the row counts as tiny)
       const int e = max(((__double2hiint(m) >> 20) & 0x7ff) - 1022, -900);
       const double scale = (m > 0.0 && !bad) ? pow2(kFix - e) : 0.0;
-      if (lane == 0) s_sc[p] = bad ? nan("") : pow2(e - 56);
-      const int pmt = (r >> 3) * 3 + c, pg = r & 7;
+      if (lane == 0) s_e[p] = bad ? kBad : e - 56;
       for (int kp = lane; kp < sh.ks * 8; kp += 32) {
         int dr[2][kSl], di[2][kSl];
 #pragma unroll
@@ -223,8 +229,8 @@ __global__ void __launch_bounds__(kNT, 1)
           digits(__double2ll_rn(im * scale), di[q]);
         }
         const int s = kp >> 3, kin = (2 * kp) & 15;
-        uint2* o = reinterpret_cast<uint2*>(A + ((pmt * sh.ks + s) * kSl) * 128 +
-                                            (pg * 4 + ((kin & 7) >> 1)) * 4 + (kin >= 8 ? 2 : 0));
+        uint2* o = reinterpret_cast<uint2*>(A + ((c * sh.ks + s) * kSl) * 128 +
+                                            (r * 4 + ((kin & 7) >> 1)) * 4 + (kin >= 8 ? 2 : 0));
 #pragma unroll
         for (int q = 0; q < kSl; ++q) o[q * 64] = make_uint2(pack2(dr[0][q], dr[1][q]), pack2(di[0][q], di[1][q]));
       }
@@ -232,18 +238,17 @@ __global__ void __launch_bounds__(kNT, 1)
     }
     __syncthreads();
     // ---- the product with tiles t0 .. t1 - 1, one step of 16 columns at a time
-    const double sc = s_sc[(rg * 8 + g) * 3 + comp];
+    const int e3[3] = {s_e[3 * g], s_e[3 * g + 1], s_e[3 * g + 2]};
     const int q0 = (ch * ntiles + t0) * sh.ks, q1 = (ch * ntiles + t1) * sh.ks;
     auto fetch = [&](int q) {
       if (q < q1) {
         const unsigned char* src = B + (size_t)q * kBBlk;
-        unsigned char* dst = tail + ((q - q0) % 3) * kBBlk;
+        unsigned char* dst = tail + ((q - q0) & 1) * kBBlk;
         for (int i = threadIdx.x; i < kBBlk / 16; i += kNT) copy16(dst + 16 * i, src + 16 * i);
       }
       asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
     fetch(q0);
-    fetch(q0 + 1);
     int q = q0;
     for (int tile = t0; tile < t1; ++tile) {
       for (int i = threadIdx.x; i < kRows * kDirs; i += kNT) {
@@ -253,79 +258,74 @@ __global__ void __launch_bounds__(kNT, 1)
           w = tab[(long long)(nx + s_iy[r]) * n_dir + d] * tab[(long long)(nx + ny + s_iz[r]) * n_dir + d];
         s_w[i] = w;
       }
-      float acc[2][kSl][4];
+      // after the reduction over rows a lane holds part (lane bit 4), column
+      // (bit 3) of its warp's 8 directions; the partial sums so far
+      const int dl = warp * 8 + (lane & 3) * 2 + ((lane >> 3) & 1), d = tile * kDirs + dl;
+      double* o = part + ((long long)blockIdx.x * n_dir + d) * 6 + (lane >> 4);
+      const bool mine = (lane & 4) == 0 && d < n_dir;
+      double old[3] = {0.0, 0.0, 0.0};
+      if (mine && u != (int)blockIdx.x) { old[0] = o[0]; old[1] = o[2]; old[2] = o[4]; }
+      float acc[3][kSl][4];
 #pragma unroll
-      for (int n = 0; n < 2; ++n)
+      for (int n = 0; n < 3; ++n)
 #pragma unroll
         for (int k = 0; k < kSl; ++k)
 #pragma unroll
           for (int v = 0; v < 4; ++v) acc[n][k][v] = 0.0f;
       for (int s = 0; s < sh.ks; ++s, ++q) {
-        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         __syncthreads();
-        fetch(q + 2);
-        const uint4* a4 = reinterpret_cast<const uint4*>(A) + (mt * sh.ks + s) * kSl * 32 + lane;
-        const uint4* b4 = reinterpret_cast<const uint4*>(tail + ((q - q0) % 3) * kBBlk) + half * 32 + lane;
-        uint4 af[kSl], bf[kSl];
+        fetch(q + 1);
+        const uint2* b2 = reinterpret_cast<const uint2*>(tail + ((q - q0) & 1) * kBBlk) + warp * 32 + lane;
+        uint2 bf[kSl];
 #pragma unroll
-        for (int k = 0; k < kSl; ++k) { af[k] = a4[k * 32]; bf[k] = b4[k * 64]; }
+        for (int k = 0; k < kSl; ++k) bf[k] = b2[k * 128];
 #pragma unroll
-        for (int i = 0; i < kSl; ++i)
+        for (int c = 0; c < 3; ++c) {
+          const uint4* a4 = reinterpret_cast<const uint4*>(A) + (c * sh.ks + s) * kSl * 32 + lane;
+          uint4 af[kSl];
 #pragma unroll
-          for (int j = 0; j < kSl - i; ++j) {
-            mma(acc[0][i + j], af[i], bf[j].x, bf[j].y);
-            mma(acc[1][i + j], af[i], bf[j].z, bf[j].w);
-          }
+          for (int k = 0; k < kSl; ++k) af[k] = a4[k * 32];
+#pragma unroll
+          for (int i = 0; i < kSl; ++i)
+#pragma unroll
+            for (int j = 0; j < kSl - i; ++j) mma(acc[c][i + j], af[i], bf[j].x, bf[j].y);
+        }
       }
-      // ---- 64-bit sums, row phases, sum over the 8 rows of the tile
-      double v[2][2][2];                     // [direction group][column][re, im]
+      // ---- 64-bit sums, row phases, sum over the 8 rows
+      double v[3][2][2];                     // [component][column][re, im]
 #pragma unroll
-      for (int n = 0; n < 2; ++n)
+      for (int col = 0; col < 2; ++col) {
+        const c128 w = s_w[g * kDirs + warp * 8 + (lane & 3) * 2 + col];
 #pragma unroll
-        for (int col = 0; col < 2; ++col) {
+        for (int c = 0; c < 3; ++c) {
           double z[2];
 #pragma unroll
           for (int im = 0; im < 2; ++im) {
-            long long t = __float2int_rn(acc[n][0][2 * im + col]);
+            long long t = __float2int_rn(acc[c][0][2 * im + col]);
 #pragma unroll
-            for (int k = 1; k < kSl - 1; ++k) t = t * 256 + __float2int_rn(acc[n][k][2 * im + col]);
-            t = t * 16 + (__float2int_rn(acc[n][kSl - 1][2 * im + col]) >> 4);
-            z[im] = (double)t * sc;
+            for (int k = 1; k < kSl - 1; ++k) t = t * 256 + __float2int_rn(acc[c][k][2 * im + col]);
+            t = t * 16 + (__float2int_rn(acc[c][kSl - 1][2 * im + col]) >> 4);
+            z[im] = e3[c] == kBad ? nan("") : scaled(t, e3[c]);
           }
-          const c128 w = s_w[(rg * 8 + g) * kDirs + half * 16 + n * 8 + (lane & 3) * 2 + col];
-          v[n][col][0] = z[0] * w.x - z[1] * w.y;
-          v[n][col][1] = z[0] * w.y + z[1] * w.x;
+          v[c][col][0] = z[0] * w.x - z[1] * w.y;
+          v[c][col][1] = z[0] * w.y + z[1] * w.x;
         }
-      // lane bit 4 keeps a direction group, bit 3 a column, bit 2 a part
-      double a4v[2][2], a2v[2], a1;
-      const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
-#pragma unroll
-      for (int col = 0; col < 2; ++col)
-#pragma unroll
-        for (int im = 0; im < 2; ++im) {
-          const double keep = b4 ? v[1][col][im] : v[0][col][im];
-          const double send = b4 ? v[0][col][im] : v[1][col][im];
-          a4v[col][im] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-        }
-#pragma unroll
-      for (int im = 0; im < 2; ++im) {
-        const double keep = b3 ? a4v[1][im] : a4v[0][im];
-        const double send = b3 ? a4v[0][im] : a4v[1][im];
-        a2v[im] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
       }
-      a1 = (b2 ? a2v[1] : a2v[0]) + __shfl_xor_sync(0xffffffffu, b2 ? a2v[0] : a2v[1], 4);
-      const int dl = half * 16 + (b4 ? 8 : 0) + (lane & 3) * 2 + (b3 ? 1 : 0);
-      const int slot = (comp * kDirs + dl) * 2 + (b2 ? 1 : 0);
-      if (rg == 1) s_red[slot] = a1;
-      __syncthreads();
-      const int d = tile * kDirs + dl;
-      if (rg == 0 && d < n_dir) {
-        a1 += s_red[slot];
-        double* o = part + ((long long)blockIdx.x * n_dir + d) * 6 + 2 * comp + (b2 ? 1 : 0);
-        *o = u == (int)blockIdx.x ? a1 : *o + a1;
+      const bool b4 = lane & 16, b3 = lane & 8;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        double p[2];
+#pragma unroll
+        for (int col = 0; col < 2; ++col)
+          p[col] = (b4 ? v[c][col][1] : v[c][col][0]) +
+                   __shfl_xor_sync(0xffffffffu, b4 ? v[c][col][0] : v[c][col][1], 16);
+        double a = (b3 ? p[1] : p[0]) + __shfl_xor_sync(0xffffffffu, b3 ? p[0] : p[1], 8);
+        a += __shfl_xor_sync(0xffffffffu, a, 4);
+        if (mine) o[2 * c] = old[c] + a;
       }
+      __syncthreads();                       // every read of the row phases
     }
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
   }
 }
 
@@ -373,11 +373,11 @@ FfShape ff_shape(int nx) {
   return s;
 }
 
-// row blocks in flight: one block per SM, no more than there are units, and
+// row blocks in flight: two blocks per SM, no more than there are units, and
 // partial sums of at most 64 MB
 int ff_groups(int units, int n_dir) {
   const long long fit = std::max(1LL, (64LL << 20) / (48LL * n_dir));
-  return (int)std::min<long long>(std::min(units, num_sms()), fit);
+  return (int)std::min<long long>(std::min(units, 2 * num_sms()), fit);
 }
 
 size_t up256(size_t b) { return (b + 255) / 256 * 256; }
@@ -422,11 +422,14 @@ cudaError_t farfield_sums(void* ws, const c128* P, const LatticeDev& lat, const 
   // direction tiles split over blockIdx.y: enough blocks for every SM and,
   // where the row blocks do not divide evenly over the SMs, finer pieces (of
   // 8 tiles at least, over which the digits of a row block are made once)
-  const int want = G < num_sms() ? (num_sms() + G - 1) / G : 4;
-  const int ny_ = std::max(1, std::min(want, G < num_sms() ? nt : (nt + 7) / 8));
+  const int slots = 2 * num_sms();
+  const int want = G < slots ? (slots + G - 1) / G : 4;
+  const int ny_ = std::max(1, std::min(want, G < slots ? nt : (nt + 7) / 8));
   const int per = (nt + ny_ - 1) / ny_;
-  const size_t sm = (size_t)6 * s.ks * kSl * 512 + kTail;
+  const size_t sm = (size_t)3 * s.ks * kSl * 512 + kTail;
   cudaError_t e = ensure_smem((const void*)k_ff_mma, sm);
+  if (e != cudaSuccess) return e;
+  e = ensure_carveout_max((const void*)k_ff_mma);
   if (e != cudaSuccess) return e;
   k_ff_mma<<<dim3(G, (nt + per - 1) / per), kNT, sm, st>>>(P, lat, tab, pack, n_dir, nx, ny, nr, n_occ, s,
                                                           nt, per, units, part);
