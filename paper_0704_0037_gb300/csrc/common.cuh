@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+
 namespace dda {
 
 // Programmatic dependent launch (sm_90 and later).  A kernel launched with
@@ -52,6 +54,16 @@ template <typename R, bool INV> __host__ __device__ __forceinline__ cpx<R> twidd
 // a * s + c for complex a, c and real s
 template <typename R> __host__ __device__ __forceinline__ cpx<R> fmas(cpx<R> a, R s, cpx<R> c) {
   return mk<R>(a.x * s + c.x, a.y * s + c.y);
+}
+
+// c + a b and c - a b: four fused multiply-adds in float and double (a product
+// and a sum take two instructions more, on the pipe that bounds the FP64
+// passes); double-float has no fused form
+template <typename R> __host__ __device__ __forceinline__ cpx<R> cmac(cpx<R> c, cpx<R> a, cpx<R> b) {
+  return mk<R>(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
+}
+template <typename R> __host__ __device__ __forceinline__ cpx<R> cnmac(cpx<R> c, cpx<R> a, cpx<R> b) {
+  return mk<R>(fma(-a.x, b.x, fma(a.y, b.y, c.x)), fma(-a.x, b.y, fma(-a.y, b.x, c.y)));
 }
 
 // Complex64 on sm_100-class devices: a complex number is one 64-bit register
@@ -287,6 +299,13 @@ template <> __host__ __device__ __forceinline__ cpx<df> fmas<df>(cpx<df> a, df s
 #else
   return mk<df>(a.x * s + c.x, a.y * s + c.y);
 #endif
+}
+
+template <> __host__ __device__ __forceinline__ cpx<df> cmac<df>(cpx<df> c, cpx<df> a, cpx<df> b) {
+  return c + a * b;
+}
+template <> __host__ __device__ __forceinline__ cpx<df> cnmac<df>(cpx<df> c, cpx<df> a, cpx<df> b) {
+  return c - a * b;
 }
 
 __host__ __device__ __forceinline__ double df_to_double(df a) { return (double)a.hi + (double)a.lo; }

@@ -195,6 +195,7 @@ struct dda_ctx {
   void* d_dscratch = nullptr;     // D-matrix build scratch kept between builds (small grids)
   size_t dscratch_bytes = 0;
   void* d_ptab = nullptr;         // incident-wave phase per axis (right-hand sides), complex128
+  size_t ptab_bytes = 0;
   int* d_arow = nullptr;          // rows within each plane's span of occupied rows
   long long* d_aoff = nullptr;    // their dipole offsets (+ n_occ)
   int* d_yr = nullptr;            // per z plane: first and last occupied row
@@ -223,10 +224,12 @@ int dda_solve_batch_internal(dda_t h, const dda_solve_opts* o, int nrhs, const d
                              const double* pol, void* P_dev, dda_solve_info* info);
 void batch_free(dda_t h);
 // incident plane wave of one right-hand side: propagation a, polarisation e
-// (complex, re/im pairs), and b = beta e exp(i kd a.r) on the handle's stream
+// (complex, re/im pairs); launch_rhs: b [nrhs][3 n_occ] = beta e exp(i kd a.r)
+// for nrhs of them (prop 3, pol 6 doubles each), on stream st
 namespace dda {
 struct Wave { double a[3]; double e[6]; };
-int launch_rhs(dda_t h, c128* b, const c128* beta, const Wave& wv, cudaStream_t st);
+int launch_rhs(dda_t h, c128* b, const c128* beta, int nrhs, const double* prop, const double* pol,
+               cudaStream_t st);
 }  // namespace dda
 // bytes of the host image of a batched QMR-CS solve (krylov.cu)
 long long dda_checkpoint_bytes_internal(dda_t h, int prec, int nrhs);

@@ -996,9 +996,6 @@ extern "C" int dda_solve_pc(dda_t h, dda_pcnet_t net, const dda_solve_opts* o, c
   c128 *s = buf + 6 * n, *t = buf + 7 * n, *ph = buf + 8 * n, *sh = buf + 9 * n;
   const int nbk = (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, 8LL * num_sms()));
   const c128 one = mk<double>(1.0, 0.0), zero = mk<double>(0.0, 0.0);
-  Wave wv;
-  for (int q = 0; q < 3; ++q) wv.a[q] = prop[q];
-  for (int q = 0; q < 6; ++q) wv.e[q] = pol[q];
   int status = DDA_NOT_CONVERGED, iters = 0, matvecs = 0, napps = 0, fallback = 0;
   double res_true = NAN, res_rec = NAN;
   std::vector<double> hv;
@@ -1009,7 +1006,7 @@ extern "C" int dda_solve_pc(dda_t h, dda_pcnet_t net, const dda_solve_opts* o, c
     return code;
   };
 #define PCK(call) do { const int rc_ = (call); if (rc_ != DDA_OK) return done(rc_); } while (0)
-  PCK(launch_rhs(h, b, h->w64.beta, wv, R.st));
+  PCK(launch_rhs(h, b, h->w64.beta, 1, prop, pol, R.st));
   DDA_CK(h, cudaMemsetAsync(x, 0, n * sizeof(c128), R.st));
   DDA_CK(h, cudaMemcpyAsync(r, b, n * sizeof(c128), cudaMemcpyDeviceToDevice, R.st));
   PCK(pc_dots(R, b, b));
