@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "pcconv.cuh"
 
 namespace dda {
 namespace pc {
@@ -40,157 +41,35 @@ constexpr int NL = 7;
 struct LayerSpec { int cin, cout, k, relu; };
 constexpr LayerSpec kSpec[NL] = {{7, 16, 3, 1},   {16, 32, 3, 1},  {32, 160, 3, 1}, {160, 160, 3, 1},
                                  {192, 32, 3, 1}, {48, 16, 3, 1},  {16, 6, 1, 0}};
-constexpr int kTX = 8, kTY = 8, kTZ = 4, kTV = kTX * kTY * kTZ;  // voxel tile of the conv kernels
-constexpr int kCO = 8;                                           // output channels per block
-
-struct Dims {
-  int x, y, z;
-  __host__ __device__ long long n() const { return (long long)x * y * z; }
-};
-inline Dims halved(Dims d) { return {(d.x + 1) / 2, (d.y + 1) / 2, (d.z + 1) / 2}; }
-
-// ---------------------------------------------------------------- conv kernels
-// out[co][v] = b[co] + sum_ci sum_k w[co][ci][k] in[ci][v + k - c]  (relu optional)
-// grid (tiles, Cout / kCO); 256 threads, one voxel each, kCO accumulators
-template <int K>
-__global__ void __launch_bounds__(kTV) k_conv_fwd(const float* __restrict__ in, int cin,
-                                                  const __nv_bfloat16* __restrict__ w,
-                                                  const float* __restrict__ bias,
-                                                  float* __restrict__ out, int cout, Dims d,
-                                                  int relu) {
-  constexpr int K3 = K * K * K, H = K / 2;
-  constexpr int HX = kTX + 2 * H, HY = kTY + 2 * H, HZ = kTZ + 2 * H;
-  __shared__ float s_in[HZ * HY * HX];
-  __shared__ float s_w[kCO * K3];
-  const int ntx = (d.x + kTX - 1) / kTX, nty = (d.y + kTY - 1) / kTY;
-  const int tile = blockIdx.x;
-  const int tx0 = (tile % ntx) * kTX, ty0 = ((tile / ntx) % nty) * kTY, tz0 = (tile / (ntx * nty)) * kTZ;
-  const int co0 = blockIdx.y * kCO;
-  const int lx = threadIdx.x % kTX, ly = (threadIdx.x / kTX) % kTY, lz = threadIdx.x / (kTX * kTY);
-  const int x = tx0 + lx, y = ty0 + ly, z = tz0 + lz;
-  const long long nv = d.n();
-  float acc[kCO];
-#pragma unroll
-  for (int c = 0; c < kCO; ++c) acc[c] = (bias && co0 + c < cout) ? bias[co0 + c] : 0.0f;
-  for (int ci = 0; ci < cin; ++ci) {
-    __syncthreads();
-    for (int k = threadIdx.x; k < HZ * HY * HX; k += kTV) {
-      const int hx = k % HX, hy = (k / HX) % HY, hz = k / (HX * HY);
-      const int gx = tx0 + hx - H, gy = ty0 + hy - H, gz = tz0 + hz - H;
-      const bool ok = gx >= 0 && gy >= 0 && gz >= 0 && gx < d.x && gy < d.y && gz < d.z;
-      s_in[k] = ok ? in[ci * nv + ((long long)gz * d.y + gy) * d.x + gx] : 0.0f;
+// Blocks below nb: g[co][ci][t] += sum over chunks of part[chunk][t][co][ci]
+// (fixed order; n = K3 nc sums of nc = cout cin); block nb + co: gb[co] +=
+// sum_v gout[co][v] (fixed-order reduction)
+__global__ void __launch_bounds__(256) k_sum_chunks(const float* __restrict__ part, int chunks, long long n,
+                                                    long long nc, float* __restrict__ g, int nb,
+                                                    const float* __restrict__ gout, long long nv,
+                                                    float* __restrict__ gb) {
+  if ((int)blockIdx.x < nb) {
+    for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += nb * 256LL) {
+      float s = 0.0f;
+#pragma unroll 8
+      for (int c = 0; c < chunks; ++c) s += part[c * n + i];
+      const long long t = i / nc;
+      g[(i - t * nc) * (n / nc) + t] += s;
     }
-    for (int k = threadIdx.x; k < kCO * K3; k += kTV) {
-      const int c = k / K3, t = k - c * K3;
-      s_w[k] = co0 + c < cout ? __bfloat162float(w[((long long)(co0 + c) * cin + ci) * K3 + t]) : 0.0f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int t = 0; t < K3; ++t) {
-      const int kx = t % K, ky = (t / K) % K, kz = t / (K * K);
-      const float v = s_in[((lz + kz) * HY + ly + ky) * HX + lx + kx];
-#pragma unroll
-      for (int c = 0; c < kCO; ++c) acc[c] = fmaf(s_w[c * K3 + t], v, acc[c]);
-    }
+    return;
   }
-  if (x < d.x && y < d.y && z < d.z) {
-    const long long v = ((long long)z * d.y + y) * d.x + x;
-#pragma unroll
-    for (int c = 0; c < kCO; ++c)
-      if (co0 + c < cout) out[(co0 + c) * nv + v] = relu ? fmaxf(acc[c], 0.0f) : acc[c];
-  }
-}
-
-// Partial weight gradients: part[chunk][co][ci][k] = sum over the voxels of
-// this chunk's tiles of gout[co][v] in[ci][v + k - c]; grid (chunks, Cout /
-// kCO, Cin), one thread per (co, k)
-template <int K>
-__global__ void __launch_bounds__(kCO * K * K * K) k_conv_wgrad(const float* __restrict__ in, int cin,
-                                                               const float* __restrict__ gout,
-                                                               int cout, Dims d,
-                                                               float* __restrict__ part,
-                                                               int tiles_per_chunk) {
-  constexpr int K3 = K * K * K, H = K / 2, NT = kCO * K3;
-  constexpr int HX = kTX + 2 * H, HY = kTY + 2 * H, HZ = kTZ + 2 * H;
-  __shared__ float s_in[HZ * HY * HX];
-  __shared__ float s_g[kCO * kTV];
-  const int ntx = (d.x + kTX - 1) / kTX, nty = (d.y + kTY - 1) / kTY, ntz = (d.z + kTZ - 1) / kTZ;
-  const int ntiles = ntx * nty * ntz;
-  const int co0 = blockIdx.y * kCO, ci = blockIdx.z;
-  const int c = threadIdx.x / K3, t = threadIdx.x - (threadIdx.x / K3) * K3;
-  const int kx = t % K, ky = (t / K) % K, kz = t / (K * K);
-  const long long nv = d.n();
-  float acc = 0.0f;
-  const int t0 = blockIdx.x * tiles_per_chunk, t1 = min(ntiles, t0 + tiles_per_chunk);
-  for (int tile = t0; tile < t1; ++tile) {
-    const int tx0 = (tile % ntx) * kTX, ty0 = ((tile / ntx) % nty) * kTY, tz0 = (tile / (ntx * nty)) * kTZ;
-    __syncthreads();
-    for (int k = threadIdx.x; k < HZ * HY * HX; k += NT) {
-      const int hx = k % HX, hy = (k / HX) % HY, hz = k / (HX * HY);
-      const int gx = tx0 + hx - H, gy = ty0 + hy - H, gz = tz0 + hz - H;
-      const bool ok = gx >= 0 && gy >= 0 && gz >= 0 && gx < d.x && gy < d.y && gz < d.z;
-      s_in[k] = ok ? in[ci * nv + ((long long)gz * d.y + gy) * d.x + gx] : 0.0f;
-    }
-    for (int k = threadIdx.x; k < kCO * kTV; k += NT) {
-      const int cc = k / kTV, u = k - cc * kTV;
-      const int gx = tx0 + u % kTX, gy = ty0 + (u / kTX) % kTY, gz = tz0 + u / (kTX * kTY);
-      const bool ok = co0 + cc < cout && gx < d.x && gy < d.y && gz < d.z;
-      s_g[k] = ok ? gout[(co0 + cc) * nv + ((long long)gz * d.y + gy) * d.x + gx] : 0.0f;
-    }
-    __syncthreads();
-    for (int u = 0; u < kTV; ++u) {
-      const int lx = u % kTX, ly = (u / kTX) % kTY, lz = u / (kTX * kTY);
-      acc = fmaf(s_g[c * kTV + u], s_in[((lz + kz) * HY + ly + ky) * HX + lx + kx], acc);
-    }
-  }
-  if (co0 + c < cout)
-    part[(((long long)blockIdx.x * cout + co0 + c) * cin + ci) * K3 + t] = acc;
-}
-
-// g[i] += sum over chunks of part[chunk][i] (fixed order)
-__global__ void k_sum_chunks(const float* __restrict__ part, int chunks, long long n,
-                             float* __restrict__ g) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    float s = 0.0f;
-    for (int c = 0; c < chunks; ++c) s += part[c * n + i];
-    g[i] += s;
-  }
-}
-
-// gb[co] += sum_v gout[co][v]: one block per channel, fixed-order reduction
-__global__ void k_bias_grad(const float* __restrict__ gout, long long nv, float* __restrict__ gb) {
+  const int co = blockIdx.x - nb;
   __shared__ float sh[256];
   float s = 0.0f;
-  for (long long v = threadIdx.x; v < nv; v += 256) s += gout[blockIdx.x * nv + v];
+#pragma unroll 8
+  for (long long v = threadIdx.x; v < nv; v += 256) s += gout[co * nv + v];
   sh[threadIdx.x] = s;
   __syncthreads();
   for (int o = 128; o > 0; o >>= 1) {
     if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
     __syncthreads();
   }
-  if (threadIdx.x == 0) gb[blockIdx.x] += sh[0];
-}
-
-// wT[ci][co][K3-1-t] = w[co][ci][t] (the transposed, flipped kernel of the
-// input gradient)
-__global__ void k_wtrans(const __nv_bfloat16* __restrict__ w, __nv_bfloat16* __restrict__ wt,
-                         int cin, int cout, int K3) {
-  const long long n = (long long)cin * cout * K3;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int t = (int)(i % K3);
-    const long long r = i / K3;
-    const int ci = (int)(r % cin), co = (int)(r / cin);
-    wt[((long long)ci * cout + co) * K3 + (K3 - 1 - t)] = w[i];
-  }
-}
-
-// g[c][v] *= (a[c][v] > 0)
-__global__ void k_relu_mask(float* __restrict__ g, const float* __restrict__ a, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    if (!(a[i] > 0.0f)) g[i] = 0.0f;
+  if (threadIdx.x == 0) gb[co] += sh[0];
 }
 
 // ---------------------------------------------------------------- pooling
@@ -217,9 +96,10 @@ __global__ void k_pool2(const float* __restrict__ in, Dims di, float* __restrict
     out[i] = s / (float)cnt;
   }
 }
-// gin[c][v] += gout[c][parent(v)] / children(parent)
+// gin[c][v] += gout[c][parent(v)] / children(parent), then zero where the
+// activation act[c][v] <= 0 (gradient behind its relu)
 __global__ void k_pool2_back(const float* __restrict__ gout, Dims dout, float* __restrict__ gin,
-                             Dims di, int ch) {
+                             Dims di, int ch, const float* __restrict__ act) {
   const long long n = di.n() * ch;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
@@ -228,24 +108,13 @@ __global__ void k_pool2_back(const float* __restrict__ gout, Dims dout, float* _
     const int x = (int)(v % di.x), y = (int)((v / di.x) % di.y), z = (int)(v / ((long long)di.x * di.y));
     const int X = x / 2, Y = y / 2, Z = z / 2;
     const int cnt = (min(2, di.x - 2 * X)) * (min(2, di.y - 2 * Y)) * (min(2, di.z - 2 * Z));
-    gin[i] += gout[c * dout.n() + ((long long)Z * dout.y + Y) * dout.x + X] / (float)cnt;
+    const float r = gin[i] + gout[c * dout.n() + ((long long)Z * dout.y + Y) * dout.x + X] / (float)cnt;
+    gin[i] = act[i] > 0.0f ? r : 0.0f;
   }
 }
-// out[c][v] = in[c][parent(v)] (nearest)
-__global__ void k_up2(const float* __restrict__ in, Dims dc, float* __restrict__ out, Dims df,
-                      int ch) {
-  const long long n = df.n() * ch;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(i / df.n());
-    const long long v = i - c * df.n();
-    const int x = (int)(v % df.x), y = (int)((v / df.x) % df.y), z = (int)(v / ((long long)df.x * df.y));
-    out[i] = in[c * dc.n() + ((long long)(z / 2) * dc.y + y / 2) * dc.x + x / 2];
-  }
-}
-// gin[c][p] = sum of gout[c][children of p]
+// gin[c][p] = sum of gout[c][children of p], zero where act[c][p] <= 0
 __global__ void k_up2_back(const float* __restrict__ gout, Dims df, float* __restrict__ gin,
-                           Dims dc, int ch) {
+                           Dims dc, int ch, const float* __restrict__ act) {
   const long long n = dc.n() * ch;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
@@ -259,7 +128,7 @@ __global__ void k_up2_back(const float* __restrict__ gout, Dims df, float* __res
           const int x = 2 * X + dx, y = 2 * Y + dy, z = 2 * Z + dz;
           if (x < df.x && y < df.y && z < df.z) s += gout[c * df.n() + ((long long)z * df.y + y) * df.x + x];
         }
-    gin[i] = s;
+    gin[i] = act[i] > 0.0f ? s : 0.0f;
   }
 }
 
@@ -273,32 +142,44 @@ __global__ void k_idx_map(LatticeDev lat, int nx, int ny, int nrows, int* __rest
       map[(long long)row * nx + lat.xi[i]] = (int)i;
 }
 // features at s0: channel 2c / 2c+1 = mean of Re / Im of v_c / rms over the
-// cell's children (void children count as zero), channel 6 = occupied fraction
-__global__ void k_feat_in(const c128* __restrict__ v, long long n_occ, const int* __restrict__ map,
-                          Dims dl, Dims d0, const double* __restrict__ scl, float* __restrict__ f) {
-  const double inv = scl[0] > 0.0 ? 1.0 / scl[0] : 0.0;
+// cell's children (void children count as zero), channel 6 = occupied
+// fraction; a thread per cell and component
+__global__ void __launch_bounds__(256) k_feat_in(const c128* __restrict__ v, long long n_occ,
+                                                 const int* __restrict__ map, Dims dl, Dims d0,
+                                                 const double* __restrict__ scl, float* __restrict__ f) {
+  const double inv = scl[5];
+  const int c = blockIdx.y;
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < d0.n();
        p += (long long)gridDim.x * blockDim.x) {
     const int X = (int)(p % d0.x), Y = (int)((p / d0.x) % d0.y), Z = (int)(p / ((long long)d0.x * d0.y));
-    double acc[6] = {0, 0, 0, 0, 0, 0};
+    int id[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int x = 2 * X + (k & 1), y = 2 * Y + ((k >> 1) & 1), z = 2 * Z + (k >> 2);
+      id[k] = x < dl.x && y < dl.y && z < dl.z ? map[((long long)z * dl.y + y) * dl.x + x] : -1;
+    }
+    double re = 0.0, im = 0.0;
     int occ = 0;
-    for (int dz = 0; dz < 2; ++dz)
-      for (int dy = 0; dy < 2; ++dy)
-        for (int dx = 0; dx < 2; ++dx) {
-          const int x = 2 * X + dx, y = 2 * Y + dy, z = 2 * Z + dz;
-          if (x >= dl.x || y >= dl.y || z >= dl.z) continue;
-          const int i = map[((long long)z * dl.y + y) * dl.x + x];
-          if (i < 0) continue;
-          ++occ;
-          for (int c = 0; c < 3; ++c) {
-            const c128 a = v[c * n_occ + i];
-            acc[2 * c] += a.x;
-            acc[2 * c + 1] += a.y;
-          }
-        }
-    for (int c = 0; c < 6; ++c) f[c * d0.n() + p] = (float)(acc[c] * inv * 0.125);
-    f[6 * d0.n() + p] = occ * 0.125f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (id[k] < 0) continue;               // FP64 additions only where there are dipoles
+      const c128 a = v[c * n_occ + id[k]];
+      ++occ;
+      re += a.x;
+      im += a.y;
+    }
+    f[(2 * c) * d0.n() + p] = (float)(re * inv * 0.125);
+    f[(2 * c + 1) * d0.n() + p] = (float)(im * inv * 0.125);
+    if (c == 0) f[6 * d0.n() + p] = occ * 0.125f;
   }
+}
+// (double)x in integer instructions (zero for subnormal x): the sweep below is
+// bound by the FP64 pipe, which also does the conversions
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+  if (m >= 0x7f800000u) return (double)x;                      // infinity, NaN
+  const unsigned hi = m < 0x00800000u ? 0u : (m >> 3) + 0x38000000u;
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), m < 0x00800000u ? 0 : (int)(u << 29));
 }
 // z_i = v_i + rms * out6[.][cell(i)] for every dipole (complex128): the
 // identity plus the learned correction
@@ -313,50 +194,57 @@ __global__ void k_feat_out(const float* __restrict__ o6, Dims d0, LatticeDev lat
     for (long long i = lat.row_off[row] + lane; i < lat.row_off[row + 1]; i += 32) {
       const long long p = ((long long)(zz / 2) * d0.y + y / 2) * d0.x + lat.xi[i] / 2;
       for (int c = 0; c < 3; ++c)
-        z[c * n_occ + i] = v[c * n_occ + i] +
-                           mk<double>(s * o6[(2 * c) * d0.n() + p], s * o6[(2 * c + 1) * d0.n() + p]);
+        z[c * n_occ + i] = fmas<double>(mk<double>(widen(o6[(2 * c) * d0.n() + p]), widen(o6[(2 * c + 1) * d0.n() + p])),
+                                        s, v[c * n_occ + i]);
     }
   }
 }
 // gradient of |z - e|^2 / |e|^2 with respect to out6 (z = rms * out6[cell]):
-// g6[ch][p] = rms * sum over the cell's dipoles of 2 (z - e)_ch / |e|^2
-__global__ void k_loss_grad(const c128* __restrict__ zz, const c128* __restrict__ e, long long n_occ,
-                            const int* __restrict__ map, Dims dl, Dims d0,
-                            const double* __restrict__ scl, float* __restrict__ g6) {
-  const double s = scl[0], inv_e = scl[1] > 0.0 ? 1.0 / scl[1] : 0.0;
+// g6[ch][p] = rms * sum over the cell's dipoles of 2 (z - e)_ch / |e|^2; a
+// thread per cell and component
+__global__ void __launch_bounds__(256) k_loss_grad(const c128* __restrict__ zz, const c128* __restrict__ e,
+                                                   long long n_occ, const int* __restrict__ map, Dims dl,
+                                                   Dims d0, const double* __restrict__ scl,
+                                                   float* __restrict__ g6) {
+  const double w = 2.0 * scl[0] * scl[6];
+  const int c = blockIdx.y;
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < d0.n();
        p += (long long)gridDim.x * blockDim.x) {
     const int X = (int)(p % d0.x), Y = (int)((p / d0.x) % d0.y), Z = (int)(p / ((long long)d0.x * d0.y));
-    double acc[6] = {0, 0, 0, 0, 0, 0};
-    for (int dz = 0; dz < 2; ++dz)
-      for (int dy = 0; dy < 2; ++dy)
-        for (int dx = 0; dx < 2; ++dx) {
-          const int x = 2 * X + dx, y = 2 * Y + dy, z = 2 * Z + dz;
-          if (x >= dl.x || y >= dl.y || z >= dl.z) continue;
-          const int i = map[((long long)z * dl.y + y) * dl.x + x];
-          if (i < 0) continue;
-          for (int c = 0; c < 3; ++c) {
-            const c128 d = zz[c * n_occ + i] - e[c * n_occ + i];
-            acc[2 * c] += d.x;
-            acc[2 * c + 1] += d.y;
-          }
-        }
-    for (int c = 0; c < 6; ++c) g6[c * d0.n() + p] = (float)(2.0 * s * inv_e * acc[c]);
+    int id[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int x = 2 * X + (k & 1), y = 2 * Y + ((k >> 1) & 1), z = 2 * Z + (k >> 2);
+      id[k] = x < dl.x && y < dl.y && z < dl.z ? map[((long long)z * dl.y + y) * dl.x + x] : -1;
+    }
+    double re = 0.0, im = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (id[k] < 0) continue;
+      const c128 d = zz[c * n_occ + id[k]] - e[c * n_occ + id[k]];
+      re += d.x;
+      im += d.y;
+    }
+    g6[(2 * c) * d0.n() + p] = (float)(w * re);
+    g6[(2 * c + 1) * d0.n() + p] = (float)(w * im);
   }
 }
 
 // per-block partial sums of |a|^2 (slot 0) and |a - b|^2 (slot 1; b may be
-// null), then one block adds them in order: out[0], out[1]
-__global__ void k_sq_part(const c128* __restrict__ a, const c128* __restrict__ b, long long n,
-                          double* __restrict__ part) {
+// null), four elements in flight per thread; k_sq_fin adds the kSqB blocks in
+// a fixed order
+constexpr int kSqB = 1024;
+__global__ void __launch_bounds__(256) k_sq_part(const c128* __restrict__ a, const c128* __restrict__ b,
+                                                 long long n, double* __restrict__ part) {
   __shared__ double sh[2][256];
   double s0 = 0.0, s1 = 0.0;
+#pragma unroll 4
   for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
     const c128 x = a[i];
-    s0 += x.x * x.x + x.y * x.y;
+    s0 = fma(x.x, x.x, fma(x.y, x.y, s0));
     if (b) {
       const c128 d = x - b[i];
-      s1 += d.x * d.x + d.y * d.y;
+      s1 = fma(d.x, d.x, fma(d.y, d.y, s1));
     }
   }
   sh[0][threadIdx.x] = s0;
@@ -374,17 +262,37 @@ __global__ void k_sq_part(const c128* __restrict__ a, const c128* __restrict__ b
     part[2 * blockIdx.x + 1] = sh[1][0];
   }
 }
-__global__ void k_sq_fin(const double* __restrict__ part, int nb, double* __restrict__ out, int mode) {
-  if (threadIdx.x != 0) return;
+// one block of 256 threads: the sums of slots 0 and 1 go to sc[0] as rms =
+// sqrt(s0 / n), sc[5] = 1 / rms (n > 0), or to sc[3] = s0, sc[4] = s1 and sc[6]
+// = 1 / s0 (n = 0); reciprocals of zero are 0
+__global__ void __launch_bounds__(256) k_sq_fin(const double* __restrict__ part, double* __restrict__ sc,
+                                                long long n) {
+  __shared__ double sh[2][256];
   double s0 = 0.0, s1 = 0.0;
-  for (int b = 0; b < nb; ++b) { s0 += part[2 * b]; s1 += part[2 * b + 1]; }
-  out[0] = s0;
-  out[1] = s1;
-  // mode 1: out[2] = rms = sqrt(s0 / n) is set by the caller's second launch
-  (void)mode;
-}
-__global__ void k_rms(double* __restrict__ sc, long long n) {
-  if (threadIdx.x == 0) sc[0] = n > 0 ? sqrt(sc[0] / (double)n) : 0.0;
+#pragma unroll
+  for (int b = threadIdx.x; b < kSqB; b += 256) { s0 += part[2 * b]; s1 += part[2 * b + 1]; }
+  sh[0][threadIdx.x] = s0;
+  sh[1][threadIdx.x] = s1;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) {
+      sh[0][threadIdx.x] += sh[0][threadIdx.x + o];
+      sh[1][threadIdx.x] += sh[1][threadIdx.x + o];
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x) return;
+  s0 = sh[0][0];
+  s1 = sh[1][0];
+  if (n > 0) {
+    const double rms = sqrt(s0 / (double)n);
+    sc[0] = rms;
+    sc[5] = rms > 0.0 ? 1.0 / rms : 0.0;
+  } else {
+    sc[3] = s0;
+    sc[4] = s1;
+    sc[6] = s0 > 0.0 ? 1.0 / s0 : 0.0;
+  }
 }
 
 // Adam (bias-corrected), then the BF16 copy used by the products
@@ -424,7 +332,9 @@ struct dda_pcnet {
   long long woff[NL] = {}, boff[NL] = {};
   float* w = nullptr;           // FP32 master weights and biases
   __nv_bfloat16* wb = nullptr;  // BF16 copy (weights and biases; products use the weights)
-  __nv_bfloat16* wt = nullptr;  // transposed, flipped kernels of the input gradients
+  uint2* wp = nullptr;          // BF16 weights in fragment order (forward products of apply)
+  float* wf = nullptr;          // FP32 copies for training: forward, then input gradients
+  PackList pack = {}, packf = {};   // their layouts: item L forward, item NL + L input gradient
   float* g = nullptr;           // gradients
   float* m1 = nullptr;
   float* m2 = nullptr;
@@ -437,7 +347,7 @@ struct dda_pcnet {
   int* map = nullptr;           // dipole index map of the current handle
   size_t map_bytes = 0;
   long long map_of = 0;         // uid of the handle the map was built for
-  double* scal = nullptr;       // [0] rms(v), [1] |e|^2, [2..] scratch
+  double* scal = nullptr;       // k_sq_fin: [0] rms(v), [3] |e|^2, [4] |e - z|^2, [5] 1 / [0], [6] 1 / [3]
   double* red = nullptr;        // reduction partials
   std::string err;
 };
@@ -452,12 +362,12 @@ int pc_fail(dda_pcnet_t n, int code, const std::string& m) {
 // Buffers of one forward/backward pass for lattice dims dl.
 struct Acts {
   Dims d0, d1, d2;
-  float *f0, *cat0, *a5, *o6, *p1, *cat1, *a4, *p2, *a2, *a3;
+  float *f0, *a0, *a5, *o6, *p1, *a1, *a4, *p2, *a2, *a3;
   float *g6, *ga5, *gcat0, *gcat1, *ga4, *ga3, *ga2, *gp2, *gp1;
 };
 
 size_t acts_floats(Dims d0, Dims d1, Dims d2) {
-  return (size_t)d0.n() * (7 + 48 + 16 + 6 + 6 + 16 + 48) + (size_t)d1.n() * (16 + 192 + 32 + 192 + 32 + 16) +
+  return (size_t)d0.n() * (7 + 16 + 16 + 6 + 6 + 16 + 48) + (size_t)d1.n() * (16 + 32 + 32 + 192 + 32 + 16) +
          (size_t)d2.n() * (32 + 160 + 160 + 160 + 160 + 32);
 }
 
@@ -480,14 +390,14 @@ int ensure_arena(dda_pcnet_t net, dda_t h, Acts& A) {
   float* p = (float*)net->arena;
   auto take = [&](long long n) { float* r = p; p += n; return r; };
   A.f0 = take(7 * A.d0.n());
-  A.cat0 = take(48 * A.d0.n());
+  A.a0 = take(16 * A.d0.n());
   A.a5 = take(16 * A.d0.n());
   A.o6 = take(6 * A.d0.n());
   A.g6 = take(6 * A.d0.n());
   A.ga5 = take(16 * A.d0.n());
   A.gcat0 = take(48 * A.d0.n());
   A.p1 = take(16 * A.d1.n());
-  A.cat1 = take(192 * A.d1.n());
+  A.a1 = take(32 * A.d1.n());
   A.a4 = take(32 * A.d1.n());
   A.gcat1 = take(192 * A.d1.n());
   A.ga4 = take(32 * A.d1.n());
@@ -522,40 +432,45 @@ int ensure_arena(dda_pcnet_t net, dda_t h, Acts& A) {
   return DDA_OK;
 }
 
-void conv_fwd(dda_pcnet_t net, int L, const float* in, float* out, Dims d, cudaStream_t st) {
-  const LayerSpec& s = kSpec[L];
-  const int tiles = ((d.x + kTX - 1) / kTX) * ((d.y + kTY - 1) / kTY) * ((d.z + kTZ - 1) / kTZ);
-  dim3 grid(tiles, (s.cout + kCO - 1) / kCO);
-  if (s.k == 3)
-    k_conv_fwd<3><<<grid, kTV, 0, st>>>(in, s.cin, net->wb + net->woff[L], net->w + net->boff[L], out,
-                                        s.cout, d, s.relu);
-  else
-    k_conv_fwd<1><<<grid, kTV, 0, st>>>(in, s.cin, net->wb + net->woff[L], net->w + net->boff[L], out,
-                                        s.cout, d, s.relu);
-  count_launch();
+// input of layer L: one array, or the upsampled coarse channels and the skip
+// connection of the decoder layers
+ConvIn layer_input(const Acts& A, int L) {
+  const Dims no{0, 0, 0};
+  switch (L) {
+    case 0: return {A.f0, 7, no, false, nullptr, 0};
+    case 1: return {A.p1, 16, no, false, nullptr, 0};
+    case 2: return {A.p2, 32, no, false, nullptr, 0};
+    case 3: return {A.a2, 160, no, false, nullptr, 0};
+    case 4: return {A.a3, 160, A.d2, true, A.a1, 32};
+    case 5: return {A.a4, 32, A.d1, true, A.a0, 16};
+    default: return {A.a5, 16, no, false, nullptr, 0};
+  }
 }
 
-// input gradient of layer L: gin = conv(gout, wT) (no bias, no relu)
-void conv_bwd_data(dda_pcnet_t net, int L, const float* gout, float* gin, Dims d, cudaStream_t st) {
+cudaError_t conv_fwd(dda_pcnet_t net, int L, const Acts& A, float* out, Dims d, bool train, cudaStream_t st) {
   const LayerSpec& s = kSpec[L];
-  const int K3 = s.k * s.k * s.k;
-  const long long nw = (long long)s.cin * s.cout * K3;
-  k_wtrans<<<gs(nw), 256, 0, st>>>(net->wb + net->woff[L], net->wt, s.cin, s.cout, K3);
-  count_launch();
-  const int tiles = ((d.x + kTX - 1) / kTX) * ((d.y + kTY - 1) / kTY) * ((d.z + kTZ - 1) / kTZ);
-  dim3 grid(tiles, (s.cin + kCO - 1) / kCO);
-  if (s.k == 3)
-    k_conv_fwd<3><<<grid, kTV, 0, st>>>(gout, s.cout, net->wt, nullptr, gin, s.cin, d, 0);
-  else
-    k_conv_fwd<1><<<grid, kTV, 0, st>>>(gout, s.cout, net->wt, nullptr, gin, s.cin, d, 0);
-  count_launch();
+  const float* bias = net->w + net->boff[L];
+  if (train)
+    return conv_f32(s.k, layer_input(A, L), net->wf + net->packf.item[L].at, bias, nullptr, out, s.cout, d,
+                    s.relu, st);
+  return conv_mma(s.k, layer_input(A, L), net->wp + net->pack.item[L].at, bias, nullptr, out, s.cout, d,
+                  s.relu, st);
 }
 
-int conv_bwd_weight(dda_pcnet_t net, int L, const float* in, const float* gout, Dims d,
-                    cudaStream_t st) {
+// input gradient of layer L: gin = conv(gout, wT) (no bias), zero where the
+// activation act <= 0 (act null: no relu in front)
+cudaError_t conv_bwd_data(dda_pcnet_t net, int L, const float* gout, float* gin, const float* act, Dims d,
+                          cudaStream_t st) {
+  const LayerSpec& s = kSpec[L];
+  const ConvIn in{gout, s.cout, {0, 0, 0}, false, nullptr, 0};
+  return conv_f32(s.k, in, net->wf + net->packf.item[NL + L].at, nullptr, act, gin, s.cin, d, 0, st);
+}
+
+int conv_bwd_weight(dda_pcnet_t net, int L, const Acts& A, const float* gout, Dims d, cudaStream_t st) {
   const LayerSpec& s = kSpec[L];
   const int K3 = s.k * s.k * s.k;
-  const int tiles = ((d.x + kTX - 1) / kTX) * ((d.y + kTY - 1) / kTY) * ((d.z + kTZ - 1) / kTZ);
+  // voxel tiles in up to 16 chunks (the order of the sums)
+  const int tiles = ((d.x + kWX - 1) / kWX) * ((d.y + kWY - 1) / kWY) * ((d.z + kWZ - 1) / kWZ);
   const int chunks = std::max(1, std::min(tiles, 16));
   const int per = (tiles + chunks - 1) / chunks;
   const long long nw = (long long)s.cout * s.cin * K3;
@@ -570,98 +485,96 @@ int conv_bwd_weight(dda_pcnet_t net, int L, const float* in, const float* gout, 
     }
     net->part_bytes = need;
   }
-  dim3 grid(chunks, (s.cout + kCO - 1) / kCO, s.cin);
   if (s.k == 3)
-    k_conv_wgrad<3><<<grid, kCO * 27, 0, st>>>(in, s.cin, gout, s.cout, d, net->part, per);
+    k_wgrad_f32<<<dim3(chunks, (s.cout + 7) / 8, (s.cin + 15) / 16), 216, 0, st>>>(layer_input(A, L), gout,
+                                                                                   s.cout, d, net->part, per);
   else
-    k_conv_wgrad<1><<<grid, kCO, 0, st>>>(in, s.cin, gout, s.cout, d, net->part, per);
+    k_wgrad1<<<chunks, 96, 0, st>>>(A.a5, s.cin, gout, s.cout, d, net->part, per);
   count_launch();
-  k_sum_chunks<<<gs(nw), 256, 0, st>>>(net->part, chunks, nw, net->g + net->woff[L]);
-  count_launch();
-  k_bias_grad<<<s.cout, 256, 0, st>>>(gout, d.n(), net->g + net->boff[L]);
+  const int nb = gs(nw);
+  k_sum_chunks<<<nb + s.cout, 256, 0, st>>>(net->part, chunks, nw, nw / K3, net->g + net->woff[L], nb, gout, d.n(),
+                                            net->g + net->boff[L]);
   count_launch();
   return DDA_OK;
 }
 
+// the copies of the weights the convolutions read, after every change of them
+// (the callers synchronise before they return, so any stream may read them)
+void pack_weights(dda_pcnet_t net, cudaStream_t st) {
+  auto size = [](const PackList& pl) { return pl.item[pl.count - 1].at + pl.item[pl.count - 1].n; };
+  k_pack_weights<<<gs(size(net->pack)), 256, 0, st>>>(net->wb, net->pack, net->wp, size(net->pack));
+  count_launch();
+  k_pack_f32<<<gs(size(net->packf)), 256, 0, st>>>(net->wb, net->packf, net->wf, size(net->packf));
+  count_launch();
+}
+
 // z = N(v) on the handle's lattice (v, z complex128 [3][N_occ]); leaves the
 // activations in A for a backward pass
-int forward(dda_pcnet_t net, dda_t h, const c128* v, c128* z, Acts& A) {
+int forward(dda_pcnet_t net, dda_t h, const c128* v, c128* z, Acts& A, bool train) {
   cudaStream_t st = h->stream;
   const long long n = 3 * h->g.n_occ;
   const Dims dl{h->g.nx, h->g.ny, h->g.nz};
-  // rms(v)
-  const int nb = 256;
-  k_sq_part<<<nb, 256, 0, st>>>(v, nullptr, n, net->red);
+  k_sq_part<<<kSqB, 256, 0, st>>>(v, nullptr, n, net->red);
   count_launch();
-  k_sq_fin<<<1, 32, 0, st>>>(net->red, nb, net->scal, 0);
+  k_sq_fin<<<1, 256, 0, st>>>(net->red, net->scal, n);     // rms(v)
   count_launch();
-  k_rms<<<1, 32, 0, st>>>(net->scal, n);
+  k_feat_in<<<dim3(gs(A.d0.n()), 3), 256, 0, st>>>(v, h->g.n_occ, net->map, dl, A.d0, net->scal, A.f0);
   count_launch();
-  k_feat_in<<<gs(A.d0.n()), 256, 0, st>>>(v, h->g.n_occ, net->map, dl, A.d0, net->scal, A.f0);
-  count_launch();
-  float* a0 = A.cat0 + 32 * A.d0.n();
-  float* a1 = A.cat1 + 160 * A.d1.n();
-  conv_fwd(net, 0, A.f0, a0, A.d0, st);
-  k_pool2<<<gs(16 * A.d1.n()), 256, 0, st>>>(a0, A.d0, A.p1, A.d1, 16); count_launch();
-  conv_fwd(net, 1, A.p1, a1, A.d1, st);
-  k_pool2<<<gs(32 * A.d2.n()), 256, 0, st>>>(a1, A.d1, A.p2, A.d2, 32); count_launch();
-  conv_fwd(net, 2, A.p2, A.a2, A.d2, st);
-  conv_fwd(net, 3, A.a2, A.a3, A.d2, st);
-  k_up2<<<gs(160 * A.d1.n()), 256, 0, st>>>(A.a3, A.d2, A.cat1, A.d1, 160); count_launch();
-  conv_fwd(net, 4, A.cat1, A.a4, A.d1, st);
-  k_up2<<<gs(32 * A.d0.n()), 256, 0, st>>>(A.a4, A.d1, A.cat0, A.d0, 32); count_launch();
-  conv_fwd(net, 5, A.cat0, A.a5, A.d0, st);
-  conv_fwd(net, 6, A.a5, A.o6, A.d0, st);
+  cudaError_t e = conv_fwd(net, 0, A, A.a0, A.d0, train, st);
+  k_pool2<<<gs(16 * A.d1.n()), 256, 0, st>>>(A.a0, A.d0, A.p1, A.d1, 16); count_launch();
+  if (e == cudaSuccess) e = conv_fwd(net, 1, A, A.a1, A.d1, train, st);
+  k_pool2<<<gs(32 * A.d2.n()), 256, 0, st>>>(A.a1, A.d1, A.p2, A.d2, 32); count_launch();
+  if (e == cudaSuccess) e = conv_fwd(net, 2, A, A.a2, A.d2, train, st);
+  if (e == cudaSuccess) e = conv_fwd(net, 3, A, A.a3, A.d2, train, st);
+  if (e == cudaSuccess) e = conv_fwd(net, 4, A, A.a4, A.d1, train, st);
+  if (e == cudaSuccess) e = conv_fwd(net, 5, A, A.a5, A.d0, train, st);
+  if (e == cudaSuccess) e = conv_fwd(net, 6, A, A.o6, A.d0, train, st);
   k_feat_out<<<std::min(4096, (h->g.nrows + 7) / 8), 256, 0, st>>>(A.o6, A.d0, h->lat(), h->g.nx, h->g.ny,
                                                                   h->g.nrows, h->g.n_occ, net->scal, v, z);
   count_launch();
-  const cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaGetLastError();
   return e == cudaSuccess ? DDA_OK : pc_fail(net, DDA_ERR_CUDA, cudaGetErrorString(e));
 }
 
 int backward(dda_pcnet_t net, dda_t h, const c128* z, const c128* e, Acts& A) {
   cudaStream_t st = h->stream;
   const Dims dl{h->g.nx, h->g.ny, h->g.nz};
-  float* a0 = A.cat0 + 32 * A.d0.n();
-  float* a1 = A.cat1 + 160 * A.d1.n();
   float* ga0 = A.gcat0 + 32 * A.d0.n();
   float* ga1 = A.gcat1 + 160 * A.d1.n();
-  k_loss_grad<<<gs(A.d0.n()), 256, 0, st>>>(z, e, h->g.n_occ, net->map, dl, A.d0, net->scal, A.g6);
+  k_loss_grad<<<dim3(gs(A.d0.n()), 3), 256, 0, st>>>(z, e, h->g.n_occ, net->map, dl, A.d0, net->scal, A.g6);
   count_launch();
   int rc;
+  cudaError_t er = cudaSuccess;
+  auto data = [&](int L, const float* gout, float* gin, const float* act, Dims d) {
+    if (er == cudaSuccess) er = conv_bwd_data(net, L, gout, gin, act, d, st);
+  };
   // L6 (conv1, linear)
-  if ((rc = conv_bwd_weight(net, 6, A.a5, A.g6, A.d0, st)) != DDA_OK) return rc;
-  conv_bwd_data(net, 6, A.g6, A.ga5, A.d0, st);
-  k_relu_mask<<<gs(16 * A.d0.n()), 256, 0, st>>>(A.ga5, A.a5, 16 * A.d0.n()); count_launch();
+  if ((rc = conv_bwd_weight(net, 6, A, A.g6, A.d0, st)) != DDA_OK) return rc;
+  data(6, A.g6, A.ga5, A.a5, A.d0);
   // L5
-  if ((rc = conv_bwd_weight(net, 5, A.cat0, A.ga5, A.d0, st)) != DDA_OK) return rc;
-  conv_bwd_data(net, 5, A.ga5, A.gcat0, A.d0, st);
+  if ((rc = conv_bwd_weight(net, 5, A, A.ga5, A.d0, st)) != DDA_OK) return rc;
+  data(5, A.ga5, A.gcat0, nullptr, A.d0);
   // up2 back to L4's output
-  k_up2_back<<<gs(32 * A.d1.n()), 256, 0, st>>>(A.gcat0, A.d0, A.ga4, A.d1, 32); count_launch();
-  k_relu_mask<<<gs(32 * A.d1.n()), 256, 0, st>>>(A.ga4, A.a4, 32 * A.d1.n()); count_launch();
+  k_up2_back<<<gs(32 * A.d1.n()), 256, 0, st>>>(A.gcat0, A.d0, A.ga4, A.d1, 32, A.a4); count_launch();
   // L4
-  if ((rc = conv_bwd_weight(net, 4, A.cat1, A.ga4, A.d1, st)) != DDA_OK) return rc;
-  conv_bwd_data(net, 4, A.ga4, A.gcat1, A.d1, st);
-  k_up2_back<<<gs(160 * A.d2.n()), 256, 0, st>>>(A.gcat1, A.d1, A.ga3, A.d2, 160); count_launch();
-  k_relu_mask<<<gs(160 * A.d2.n()), 256, 0, st>>>(A.ga3, A.a3, 160 * A.d2.n()); count_launch();
+  if ((rc = conv_bwd_weight(net, 4, A, A.ga4, A.d1, st)) != DDA_OK) return rc;
+  data(4, A.ga4, A.gcat1, nullptr, A.d1);
+  k_up2_back<<<gs(160 * A.d2.n()), 256, 0, st>>>(A.gcat1, A.d1, A.ga3, A.d2, 160, A.a3); count_launch();
   // L3
-  if ((rc = conv_bwd_weight(net, 3, A.a2, A.ga3, A.d2, st)) != DDA_OK) return rc;
-  conv_bwd_data(net, 3, A.ga3, A.ga2, A.d2, st);
-  k_relu_mask<<<gs(160 * A.d2.n()), 256, 0, st>>>(A.ga2, A.a2, 160 * A.d2.n()); count_launch();
+  if ((rc = conv_bwd_weight(net, 3, A, A.ga3, A.d2, st)) != DDA_OK) return rc;
+  data(3, A.ga3, A.ga2, A.a2, A.d2);
   // L2
-  if ((rc = conv_bwd_weight(net, 2, A.p2, A.ga2, A.d2, st)) != DDA_OK) return rc;
-  conv_bwd_data(net, 2, A.ga2, A.gp2, A.d2, st);
+  if ((rc = conv_bwd_weight(net, 2, A, A.ga2, A.d2, st)) != DDA_OK) return rc;
+  data(2, A.ga2, A.gp2, nullptr, A.d2);
   // pool back into L1's output (skip gradient already in gcat1[160..])
-  k_pool2_back<<<gs(32 * A.d1.n()), 256, 0, st>>>(A.gp2, A.d2, ga1, A.d1, 32); count_launch();
-  k_relu_mask<<<gs(32 * A.d1.n()), 256, 0, st>>>(ga1, a1, 32 * A.d1.n()); count_launch();
+  k_pool2_back<<<gs(32 * A.d1.n()), 256, 0, st>>>(A.gp2, A.d2, ga1, A.d1, 32, A.a1); count_launch();
   // L1
-  if ((rc = conv_bwd_weight(net, 1, A.p1, ga1, A.d1, st)) != DDA_OK) return rc;
-  conv_bwd_data(net, 1, ga1, A.gp1, A.d1, st);
-  k_pool2_back<<<gs(16 * A.d0.n()), 256, 0, st>>>(A.gp1, A.d1, ga0, A.d0, 16); count_launch();
-  k_relu_mask<<<gs(16 * A.d0.n()), 256, 0, st>>>(ga0, a0, 16 * A.d0.n()); count_launch();
+  if ((rc = conv_bwd_weight(net, 1, A, ga1, A.d1, st)) != DDA_OK) return rc;
+  data(1, ga1, A.gp1, nullptr, A.d1);
+  k_pool2_back<<<gs(16 * A.d0.n()), 256, 0, st>>>(A.gp1, A.d1, ga0, A.d0, 16, A.a0); count_launch();
   // L0 (no input gradient)
-  if ((rc = conv_bwd_weight(net, 0, A.f0, ga0, A.d0, st)) != DDA_OK) return rc;
-  const cudaError_t er = cudaGetLastError();
+  if ((rc = conv_bwd_weight(net, 0, A, ga0, A.d0, st)) != DDA_OK) return rc;
+  if (er == cudaSuccess) er = cudaGetLastError();
   return er == cudaSuccess ? DDA_OK : pc_fail(net, DDA_ERR_CUDA, cudaGetErrorString(er));
 }
 
@@ -688,9 +601,21 @@ extern "C" int dda_pcnet_create(dda_pcnet_t* out, unsigned long long seed) {
     off += kSpec[L].cout;
   }
   net->nparam = off;
-  size_t wtmax = 0;
-  for (int L = 0; L < NL; ++L)
-    wtmax = std::max(wtmax, (size_t)kSpec[L].cout * kSpec[L].cin * kSpec[L].k * kSpec[L].k * kSpec[L].k);
+  long long pat = 0, patf = 0;
+  net->pack.count = NL;
+  net->packf.count = 2 * NL;
+  for (int q = 0; q < 2 * NL; ++q) {
+    const LayerSpec& s = kSpec[q % NL];
+    const int flip = q >= NL, ni = flip ? s.cout : s.cin, no = flip ? s.cin : s.cout, k3 = s.k * s.k * s.k;
+    const long long n = (long long)((ni + 15) / 16) * k3 * ((no + 7) / 8) * 32;
+    const long long nf = (long long)ni * k3 * ((no + 7) / 8 * 8);
+    if (!flip) {
+      net->pack.item[q] = {net->woff[q], s.cin, s.cout, k3, 0, pat, n};
+      pat += n;
+    }
+    net->packf.item[q] = {net->woff[q % NL], s.cin, s.cout, k3, flip, patf, nf};
+    patf += nf;
+  }
   // He-normal weights from a seeded host generator, zero biases; the last
   // layer starts small so that the untrained network is close to zero
   std::vector<float> hw((size_t)off, 0.0f);
@@ -704,12 +629,13 @@ extern "C" int dda_pcnet_create(dda_pcnet_t* out, unsigned long long seed) {
   int rc = DDA_OK;
   if (dev_malloc(&net->w, off * sizeof(float)) != cudaSuccess ||
       dev_malloc(&net->wb, off * sizeof(__nv_bfloat16)) != cudaSuccess ||
-      dev_malloc(&net->wt, wtmax * sizeof(__nv_bfloat16)) != cudaSuccess ||
+      dev_malloc(&net->wp, pat * sizeof(uint2)) != cudaSuccess ||
+      dev_malloc(&net->wf, patf * sizeof(float)) != cudaSuccess ||
       dev_malloc(&net->g, off * sizeof(float)) != cudaSuccess ||
       dev_malloc(&net->m1, off * sizeof(float)) != cudaSuccess ||
       dev_malloc(&net->m2, off * sizeof(float)) != cudaSuccess ||
       dev_malloc(&net->scal, 8 * sizeof(double)) != cudaSuccess ||
-      dev_malloc(&net->red, 2 * 256 * sizeof(double)) != cudaSuccess) {
+      dev_malloc(&net->red, 2 * kSqB * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
     rc = DDA_ERR_OOM;
   } else if (cudaMemcpy(net->w, hw.data(), off * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
@@ -721,6 +647,7 @@ extern "C" int dda_pcnet_create(dda_pcnet_t* out, unsigned long long seed) {
   } else {
     k_to_bf16<<<gs(off), 256>>>(net->w, net->wb, off);
     count_launch();
+    pack_weights(net, 0);
     if (cudaDeviceSynchronize() != cudaSuccess) { cudaGetLastError(); rc = DDA_ERR_CUDA; }
   }
   if (rc != DDA_OK) {
@@ -735,7 +662,7 @@ extern "C" int dda_pcnet_free(dda_pcnet_t net) {
   if (!net) return DDA_OK;
   DeviceGuard dg(net->device);
   cudaDeviceSynchronize();
-  dev_free(net->w, 0); dev_free(net->wb, 0); dev_free(net->wt, 0); dev_free(net->g, 0);
+  dev_free(net->w, 0); dev_free(net->wb, 0); dev_free(net->wp, 0); dev_free(net->wf, 0); dev_free(net->g, 0);
   dev_free(net->m1, 0); dev_free(net->m2, 0); dev_free(net->arena, 0); dev_free(net->part, 0);
   dev_free(net->map, 0); dev_free(net->scal, 0); dev_free(net->red, 0);
   cudaGetLastError();
@@ -770,6 +697,7 @@ extern "C" int dda_pcnet_set_weights(dda_pcnet_t net, const float* host) {
   }
   k_to_bf16<<<gs(net->nparam), 256>>>(net->w, net->wb, net->nparam);
   count_launch();
+  pack_weights(net, 0);
   cudaMemset(net->m1, 0, net->nparam * sizeof(float));
   cudaMemset(net->m2, 0, net->nparam * sizeof(float));
   net->step = 0;
@@ -786,7 +714,7 @@ extern "C" int dda_pcnet_apply(dda_pcnet_t net, dda_t h, const void* v_dev, void
   DDA_ON_DEVICE(h);
   Acts A;
   int rc = ensure_arena(net, h, A);
-  if (rc == DDA_OK) rc = forward(net, h, (const c128*)v_dev, (c128*)z_dev, A);
+  if (rc == DDA_OK) rc = forward(net, h, (const c128*)v_dev, (c128*)z_dev, A, false);
   return rc;
 }
 
@@ -804,15 +732,13 @@ extern "C" int dda_pcnet_train_step(dda_pcnet_t net, dda_t h, const void* r_dev,
   const c128* r = (const c128*)r_dev;
   const c128* e = (const c128*)e_dev;
   c128* z = (c128*)z_dev;
-  if ((rc = forward(net, h, r, z, A)) != DDA_OK) return rc;
-  // |e|^2 into scal[1] (scal[0] keeps rms(r)), |z - e|^2 into scal[2]
+  if ((rc = forward(net, h, r, z, A, true)) != DDA_OK) return rc;
+  // |e|^2 into scal[3], |z - e|^2 into scal[4] (scal[0] keeps rms(r))
   const long long n = 3 * h->g.n_occ;
-  k_sq_part<<<256, 256, 0, st>>>(e, z, n, net->red);
+  k_sq_part<<<kSqB, 256, 0, st>>>(e, z, n, net->red);
   count_launch();
-  k_sq_fin<<<1, 32, 0, st>>>(net->red, 256, net->scal + 3, 0);   // scal[3] = |e|^2, scal[4] = |e - z|^2
+  k_sq_fin<<<1, 256, 0, st>>>(net->red, net->scal, 0);   // scal[3] = |e|^2, scal[4] = |e - z|^2
   count_launch();
-  if (cudaMemcpyAsync(net->scal + 1, net->scal + 3, sizeof(double), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-    return pc_fail(net, DDA_ERR_CUDA, "loss scalars");
   if (cudaMemsetAsync(net->g, 0, net->nparam * sizeof(float), st) != cudaSuccess)
     return pc_fail(net, DDA_ERR_CUDA, "gradient reset");
   if ((rc = backward(net, h, z, e, A)) != DDA_OK) return rc;
@@ -822,6 +748,7 @@ extern "C" int dda_pcnet_train_step(dda_pcnet_t net, dda_t h, const void* r_dev,
   k_adam<<<gs(net->nparam), 256, 0, st>>>(net->w, net->wb, net->g, net->m1, net->m2, net->nparam, lr,
                                          b1, b2, c1, c2, 1e-8f);
   count_launch();
+  pack_weights(net, st);
   double hs[2];
   if (cudaMemcpyAsync(hs, net->scal + 3, 2 * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess) {
