@@ -308,6 +308,31 @@ template <> __host__ __device__ __forceinline__ cpx<df> cnmac<df>(cpx<df> c, cpx
   return c - a * b;
 }
 
+// A real number that the compiler can know to be zero: after inlining the flag
+// is a constant, and sums with and products by a known zero disappear (an IEEE
+// addition of 0 does not fold, for the sign of -0).  Codelets instantiated on
+// cpx<pz<R>> skip the arithmetic of inputs that are padding.
+template <typename R> struct pz {
+  R v;
+  bool z;
+  __host__ __device__ constexpr pz() : v(0), z(true) {}
+  __host__ __device__ constexpr pz(R a, bool zero) : v(a), z(zero) {}
+  __host__ __device__ constexpr explicit pz(R a) : v(a), z(false) {}
+};
+template <typename R> __host__ __device__ __forceinline__ constexpr pz<R> operator-(pz<R> a) {
+  return a.z ? a : pz<R>(-a.v, false);
+}
+template <typename R> __host__ __device__ __forceinline__ constexpr pz<R> operator+(pz<R> a, pz<R> b) {
+  return a.z ? b : b.z ? a : pz<R>(a.v + b.v, false);
+}
+template <typename R> __host__ __device__ __forceinline__ constexpr pz<R> operator-(pz<R> a, pz<R> b) {
+  return b.z ? a : a.z ? pz<R>(-b.v, false) : pz<R>(a.v - b.v, false);
+}
+template <typename R> __host__ __device__ __forceinline__ constexpr pz<R> operator*(pz<R> a, pz<R> b) {
+  return a.z || b.z ? pz<R>() : pz<R>(a.v * b.v, false);
+}
+template <typename R> struct cpx<pz<R>> { pz<R> x, y; };
+
 __host__ __device__ __forceinline__ double df_to_double(df a) { return (double)a.hi + (double)a.lo; }
 __host__ __device__ __forceinline__ c128 to128(cdf a) {
   return mk<double>(df_to_double(a.x), df_to_double(a.y));

@@ -47,6 +47,28 @@ constexpr int kMinB(int nt, int want, long long smem_bytes) {
 template <typename R>
 __device__ __forceinline__ cpx<R> zero() { return mk<R>((R)0, (R)0); }
 
+// Forward M1-point transform of the first phase, whose inputs v[i], i >= KH,
+// are padding.  In complex128 their arithmetic is left out (the FP64 pipe
+// bounds those passes: 1.6 operations per clock and SM); the paired complex64
+// and the double-float codelets run whole.  With the fused products of the z
+// pass, 61 x 45 x 52 ellipsoid, FP64: product 777 -> 699 us, z pass 553 -> 486.
+template <typename R, int M1, int KH>
+__device__ __forceinline__ void dft_padded(cpx<R> (&v)[M1]) {
+  if constexpr (std::is_same<R, double>::value) {
+    cpx<pz<R>> t[M1];
+#pragma unroll
+    for (int i = 0; i < M1; ++i) {
+      t[i].x = i < KH ? pz<R>(v[i].x) : pz<R>();
+      t[i].y = i < KH ? pz<R>(v[i].y) : pz<R>();
+    }
+    cl::Dft<pz<R>, false, M1>::run(t);
+#pragma unroll
+    for (int i = 0; i < M1; ++i) v[i] = mk<R>(t[i].x.z ? (R)0 : t[i].x.v, t[i].y.z ? (R)0 : t[i].y.v);
+  } else {
+    cl::Dft<R, false, M1>::run(v);
+  }
+}
+
 // Element type of the product's input and output vectors: the arithmetic
 // type for complex64 and complex128, complex128 for the double-float passes
 // (their vectors are the FP64 refinement's).
@@ -126,7 +148,8 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>) fk_yfwd(const cpx<R>* __restri
         v[i] = w;
       }
     }
-    cl::Dft<R, false, M1>::run(v);
+    if constexpr (PRUNE) dft_padded<R, M1, kHalf<M1, M2>>(v);
+    else cl::Dft<R, false, M1>::run(v);
 #pragma unroll
     for (int k1 = 1; k1 < M1; ++k1) v[k1] = twiddle<R, false>(v[k1], s_tw[j * k1]);
 #pragma unroll
@@ -387,18 +410,17 @@ __device__ __forceinline__ void zc_product(cpx<R>* s, const cpx<R>* __restrict__
     {
       const int e = Z::at(a1, a2) * T + t2;
       const cpx<R> vx = s[e], vy = s[CS + e], vz = s[2 * CS + e];
-      s[e] = dxx * vx + dxy * vy + ez * vz;
-      s[CS + e] = dxy * vx + dyy * vy + fzz * vz;
-      s[2 * CS + e] = ez * vx + fzz * vy + dzz * vz;
+      s[e] = cmac(cmac(dxx * vx, dxy, vy), ez, vz);
+      s[CS + e] = cmac(cmac(dxy * vx, dyy, vy), fzz, vz);
+      s[2 * CS + e] = cmac(cmac(ez * vx, fzz, vy), dzz, vz);
     }
     if (fz != 0 && 2 * fz != M) {
-      // kz = M - fz: xz and yz change sign (odd in z); the negated terms are
-      // subtracted, which rounds exactly as adding the negated products
+      // kz = M - fz: xz and yz change sign (odd in z): their terms are subtracted
       const int e = Z::at(b1, b2) * T + t2;
       const cpx<R> vx = s[e], vy = s[CS + e], vz = s[2 * CS + e];
-      s[e] = dxx * vx + dxy * vy - ez * vz;
-      s[CS + e] = dxy * vx + dyy * vy - fzz * vz;
-      s[2 * CS + e] = dzz * vz - (ez * vx + fzz * vy);
+      s[e] = cnmac(cmac(dxx * vx, dxy, vy), ez, vz);
+      s[CS + e] = cnmac(cmac(dxy * vx, dyy, vy), fzz, vz);
+      s[2 * CS + e] = cnmac(cnmac(dzz * vz, ez, vx), fzz, vy);
     }
     a1 += S1;
     a2 += S2;
@@ -495,7 +517,7 @@ __device__ __forceinline__ void zc_forward_product_inva(cpx<R>* s, const cpx<R>*
     }
     __syncthreads();           // every read of the tile before the region is rewritten
     if (q < M2) {
-      cl::Dft<R, false, M1>::run(v);
+      dft_padded<R, M1, kZin>(v);
 #pragma unroll
       for (int k1 = 1; k1 < M1; ++k1) v[k1] = twiddle<R, false>(v[k1], s_tw[j * k1]);
 #pragma unroll
@@ -691,7 +713,7 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, 3, (M1 *
     cpx<R> v[M1];
 #pragma unroll
     for (int i = 0; i < M1; ++i) v[i] = i < kHalf<M1, M2> ? at[j + M2 * i] : zero<R>();
-    cl::Dft<R, false, M1>::run(v);
+    dft_padded<R, M1, kHalf<M1, M2>>(v);
 #pragma unroll
     for (int k1 = 1; k1 < M1; ++k1) v[k1] = twiddle<R, false>(v[k1], s_tw[j * k1]);
 #pragma unroll
@@ -846,7 +868,7 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, kXinvB<R
           const cpx<R> xv = vin<R>(k < kXS ? s_x[k] : xc[S0 + k]);
           cpx<R> v = xv;
           if (CONJ) v = conjg(v);
-          cpx<R> o = v - beta[mk_[u2] * 3 + c] * a[row_of<T>(s_off, S0 + k) * LD + xk[u2]];
+          cpx<R> o = cnmac(v, beta[mk_[u2] * 3 + c], a[row_of<T>(s_off, S0 + k) * LD + xk[u2]]);
           if (CONJ) o = conjg(o);
           yc[S0 + k] = vstore(o);
           if (dotp) {

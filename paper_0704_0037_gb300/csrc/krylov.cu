@@ -1246,11 +1246,14 @@ int dda_solve_internal(dda_t h, const dda_solve_opts* o, int nrhs, const double*
   Run ru;
   ru.h = h; ru.st = h->stream; ru.n = n;
   long long nb = (n + 4LL * kVT - 1) / (4LL * kVT);
+  // the FP64 sweeps are bound by the FP64 pipe: small vectors over every SM
+  // (QMR-CS keeps the blocks of the batched solve, whose bits it shares)
+  if (!refined && o->solver != DDA_QMR_CS)
+    nb = std::max(nb, std::min<long long>((n + kVT - 1) / kVT, num_sms()));
   ru.nb = (int)(nb < 1 ? 1 : (nb > kNB ? kNB : nb));
   ru.part = h->d_part;
   ru.ds = (Scal*)h->d_scal;
   ru.hs = (Scal*)h->h_scal;
-  const int rows_grid = (int)std::min<long long>((h->g.nrows + 7) / 8, 32LL * num_sms());
   int worst = DDA_OK;
   for (int r = 0; r < nrhs; ++r) {
     auto t0 = std::chrono::steady_clock::now();
@@ -1873,7 +1876,6 @@ int dda_solve_batch_internal(dda_t h, const dda_solve_opts* o, int nrhs, const d
   b.h = h; b.st = h->stream; b.n = n; b.nrhs = nrhs; b.m = m;
   long long nbl = (n + 4LL * kVT - 1) / (4LL * kVT);
   b.nb = (int)(nbl < 1 ? 1 : (nbl > kNB ? kNB : nbl));
-  const int rows_grid = (int)std::min<long long>((h->g.nrows + 7) / 8, 32LL * num_sms());
   cudaStream_t st = b.st;
   std::vector<int> status(nrhs, DDA_NOT_CONVERGED), iters(nrhs, 0), outer(nrhs, 0);
   std::vector<int> mv64(nrhs, 0);
