@@ -353,6 +353,12 @@ cudaError_t fast_pass_c64_e(int M, int pass, const FastArgs& a);
 cudaError_t fast_pass_c64_f(int M, int pass, const FastArgs& a);
 cudaError_t fast_pass_c64_g(int M, int pass, const FastArgs& a);
 cudaError_t fast_pass_c64_h(int M, int pass, const FastArgs& a);
+// x and y passes fused per z plane (fast_xy.cu, complex64): P1 and P2 (in: x,
+// out: B2), P4 and P5 (in: B2, x: x, out: y, dotp: nz partials per component);
+// tw: the twiddles of x followed by those of y
+bool fast_xy_supported(int Mx, int My);
+cudaError_t fast_xy_fwd_c64(const FastArgs& a);
+cudaError_t fast_yx_inv_c64(const FastArgs& a);
 template <typename R> cudaError_t fast_pass(int M, int pass, const FastArgs& a);
 template <typename R> cudaError_t fast_pass_270(int pass, const FastArgs& a);
 template <typename R> cudaError_t fast_pass_256(int pass, const FastArgs& a);

@@ -238,9 +238,9 @@ __global__ void __launch_bounds__(256) k_p3(cpx<R>* __restrict__ B2, const cpx<R
     if (ny_ ^ nz_) dyz = mk<R>(-dyz.x, -dyz.y);
     const int e = kz * ldm + t;
     const cpx<R> vx = cp[0][e], vy = cp[1][e], vz = cp[2][e];
-    cp[0][e] = dxx * vx + dxy * vy + dxz * vz;
-    cp[1][e] = dxy * vx + dyy * vy + dyz * vz;
-    cp[2][e] = dxz * vx + dyz * vy + dzz * vz;
+    cp[0][e] = cmac(cmac(dxx * vx, dxy, vy), dxz, vz);
+    cp[1][e] = cmac(cmac(dxy * vx, dyy, vy), dyz, vz);
+    cp[2][e] = cmac(cmac(dxz * vx, dyz, vy), dzz, vz);
   }
   __syncthreads();
   for (int c = 0; c < 3; ++c) {
@@ -343,7 +343,9 @@ cudaError_t launch_matvec(const Geom& g, const LatticeDev& lat, Work<R>& w, cons
     la.yr = nullptr;
     la.nact = 0;
   }
-  const int dnb = fast_xinv_blocks(la.arow ? la.nact : g.nrows, sizeof(R) == 4, g.Mx);
+  // small complex64 grids: x and y passes fused per z plane
+  const bool xy = sizeof(R) == 4 && g.engine == 0 && fast_xy_supported(g.Mx, g.My);
+  const int dnb = xy ? 3 * g.nz : fast_xinv_blocks(la.arow ? la.nact : g.nrows, sizeof(R) == 4, g.Mx);
   if (dotp && dot_nb && fx) *dot_nb = dnb;
   // right-hand sides in chunks of the work buffers' capacity, each chunk in
   // one launch per pass
@@ -367,7 +369,10 @@ cudaError_t launch_matvec(const Geom& g, const LatticeDev& lat, Work<R>& w, cons
     const int tb = sizeof(R) == 4 ? TR_P1_C64 : TR_P1_C128;
     // P1: x lines of the occupied rows, gather and beta -> B1 [rhs][3][nz][ny][Mx]
     tr_begin(g.tr, st);
-    if (fx) {
+    if (xy) {                      // P1 and P2 -> B2
+      fa.in = xr; fa.out = w.B2; fa.tw = twx;
+      if ((e = fast_xy_fwd_c64(fa)) != cudaSuccess) return e;
+    } else if (fx) {
       fa.in = xr; fa.out = w.B1; fa.tw = twx;
       if ((e = fast_pass<R>(g.Mx, FP_XFWD, fa)) != cudaSuccess) return e;
     } else if (adjoint) {
@@ -378,18 +383,20 @@ cudaError_t launch_matvec(const Geom& g, const LatticeDev& lat, Work<R>& w, cons
                                            bstride, sk); count_launch();
     }
     tr_end(g.tr, st, tb);
-    tr_begin(g.tr, st);
-    // P2: y lines of B1 [rhs][3][nz][ny][Mx] -> B2 [rhs][3][nz][My][Mx]
-    if (fy) {
-      fa.in = w.B1; fa.out = w.B2; fa.tw = twy;
-      e = fast_pass<R>(g.My, FP_YFWD, fa);
-    } else {
-      e = launch_lines<R>(g, w.B1, w.B2, g.py, twy, false, g.ny, g.My, g.Mx, g.nz, 3 * cnt, false,
-                          g.Mx, 1, (long long)g.ny * g.Mx, (long long)g.nz * g.ny * g.Mx,
-                          g.Mx, 1, (long long)g.My * g.Mx, (long long)g.nz * g.My * g.Mx, st, sk);
+    if (!xy) {
+      tr_begin(g.tr, st);
+      // P2: y lines of B1 [rhs][3][nz][ny][Mx] -> B2 [rhs][3][nz][My][Mx]
+      if (fy) {
+        fa.in = w.B1; fa.out = w.B2; fa.tw = twy;
+        e = fast_pass<R>(g.My, FP_YFWD, fa);
+      } else {
+        e = launch_lines<R>(g, w.B1, w.B2, g.py, twy, false, g.ny, g.My, g.Mx, g.nz, 3 * cnt, false,
+                            g.Mx, 1, (long long)g.ny * g.Mx, (long long)g.nz * g.ny * g.Mx,
+                            g.Mx, 1, (long long)g.My * g.Mx, (long long)g.nz * g.My * g.Mx, st, sk);
+      }
+      if (e != cudaSuccess) return e;
+      tr_end(g.tr, st, tb + 1);
     }
-    if (e != cudaSuccess) return e;
-    tr_end(g.tr, st, tb + 1);
     dim3 g3((g.Mx + (1 << lt3) - 1) >> lt3, g.My, cnt);
     tr_begin(g.tr, st);
     // P3: z lines, product with the octant of FFT(G), inverse z lines (in place)
@@ -400,6 +407,14 @@ cudaError_t launch_matvec(const Geom& g, const LatticeDev& lat, Work<R>& w, cons
       k_p3<R><<<g3, 256, sm3, st>>>(w.B2, w.D, g.nz, g.Mx, g.My, g.pz, twz, lt3, sk); count_launch();
     }
     tr_end(g.tr, st, tb + 2);
+    if (xy) {                      // P4 and P5 -> y
+      tr_begin(g.tr, st);
+      fa.in = w.B2; fa.x = xr; fa.out = yr; fa.tw = twx;
+      if (dotp && dot_nb) fa.dotp = dotp + (size_t)r0 * 2 * dnb;
+      if ((e = fast_yx_inv_c64(fa)) != cudaSuccess) return e;
+      tr_end(g.tr, st, tb + 4);
+      continue;
+    }
     tr_begin(g.tr, st);
     // P4: inverse y, keep y < ny
     if (fy) {
