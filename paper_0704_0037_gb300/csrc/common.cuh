@@ -14,7 +14,9 @@ namespace dda {
 // anything that kernel wrote (the wait returns once it has completed and its
 // writes are visible).  pdl_launch() lets the next such kernel be scheduled
 // as soon as every block of this one has called it.  Both are no-ops in an
-// ordinary launch.
+// ordinary launch.  Every kernel waits before it lets the next one in, so
+// what runs ahead of the wait may read anything older than the kernel just
+// before it: the product passes load twiddles and lattice tables there.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

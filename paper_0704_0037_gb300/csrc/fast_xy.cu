@@ -11,7 +11,8 @@
 // among codelets compiled into the one kernel (a switch per direction instead
 // of a kernel per pair of lengths); each line is computed with the arithmetic
 // of the separate passes (fastfft.cuh), so the products agree bit for bit.
-// 16^3 sphere: 13.4 -> 11.5 us a product.  With 16 right-hand sides on a
+// 16^3 sphere: 13.4 -> 11.5 us a product (9.9 with the tables loaded ahead of
+// the wait for the kernel before).  With 16 right-hand sides on a
 // 40 x 29 x 22 ellipsoid the two kernels take what the four took (43.6 against
 // 43.4 us), so the line lies at the lengths whose planes fit an SM twice.
 #include "fastfft.cuh"
@@ -190,13 +191,13 @@ __global__ void __launch_bounds__(kXYT) fk_xy_fwd(const c64* __restrict__ x, c64
                                                   const int* __restrict__ skip) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int z = blockIdx.x, cc = blockIdx.y, c = cc % 3;
-  pdl_wait();
-  pdl_launch();
-  if (skip && skip[cc / 3]) return;
   beta += (long long)(cc / 3) * bstride;
   const PlaneMem m = plane_mem(smem_raw, tw, lat, z, ny, Mx, My);
   for (int i = threadIdx.x; i < m.nrow * m.ld; i += kXYT) m.P[i] = zero<float>();
   __syncthreads();
+  pdl_wait();
+  pdl_launch();
+  if (skip && skip[cc / 3]) return;
   const c64* xc = x + (long long)cc * n_occ;
   const long long S0 = m.off[0];
   const int span = (int)(m.off[ny] - S0);
@@ -238,12 +239,12 @@ __global__ void __launch_bounds__(kXYT) fk_yx_inv(const c64* __restrict__ B2, co
                                                   const int* __restrict__ skip) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int z = blockIdx.x, cc = blockIdx.y, c = cc % 3;
-  pdl_wait();
-  pdl_launch();
-  if (skip && skip[cc / 3]) return;
   beta += (long long)(cc / 3) * bstride;
   const PlaneMem m = plane_mem(smem_raw, tw, lat, z, ny, Mx, My);
   __syncthreads();
+  pdl_wait();
+  pdl_launch();
+  if (skip && skip[cc / 3]) return;
   const c64* in = B2 + ((long long)cc * gridDim.x + z) * My * Mx;
 #define COLS(A, B) cols_inv<A, B>(in, m.P, m.Q, m.y0, m.nrow, m.ld, Mx, m.twy)
   DDA_XY_LENGTHS(My, COLS)

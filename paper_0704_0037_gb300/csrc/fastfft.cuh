@@ -107,9 +107,6 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>) fk_yfwd(const cpx<R>* __restri
                                                           int msign, const int* __restrict__ skip,
                                                           long long ostr, const int* __restrict__ yr) {
   constexpr int M = M1 * M2, NT = T * kQ<M1, M2>;
-  pdl_wait();
-  pdl_launch();
-  if (skip && skip[blockIdx.z / 3]) return;     // right-hand side already converged
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* s_tw = reinterpret_cast<cpx<R>*>(smem_raw);
   cpx<R>* s = s_tw + M;
@@ -124,6 +121,9 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>) fk_yfwd(const cpx<R>* __restri
   __shared__ int s_yr[2];
   if (threadIdx.x < 2) s_yr[threadIdx.x] = yr ? yr[2 * blockIdx.y + threadIdx.x] : (threadIdx.x ? ny - 1 : 0);
   load_tw(s_tw, tw, M, NT);
+  pdl_wait();
+  pdl_launch();
+  if (skip && skip[blockIdx.z / 3]) return;     // right-hand side already converged
   __syncthreads();
   const int ylo = s_yr[0], yhi = s_yr[1];
   if (q < M2) {
@@ -175,9 +175,6 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>) fk_yinv(const cpx<R>* __restri
                                                           int Mx, const cpx<R>* __restrict__ tw,
                                                           const int* __restrict__ skip) {
   constexpr int M = M1 * M2, NT = T * kQ<M1, M2>;
-  pdl_wait();
-  pdl_launch();
-  if (skip && skip[blockIdx.z / 3]) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* s_tw = reinterpret_cast<cpx<R>*>(smem_raw);
   cpx<R>* s = s_tw + M;
@@ -186,6 +183,9 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>) fk_yinv(const cpx<R>* __restri
   const long long ib = ((long long)blockIdx.z * nz + blockIdx.y) * M * Mx;
   const long long ob = ((long long)blockIdx.z * nz + blockIdx.y) * ny * Mx;
   load_tw(s_tw, tw, M, NT);
+  pdl_wait();
+  pdl_launch();
+  if (skip && skip[blockIdx.z / 3]) return;
   __syncthreads();
   if (q < M1) {
     const int k1 = q;
@@ -595,13 +595,14 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>,
     fk_zconv(cpx<R>* __restrict__ B2, const cpx<R>* __restrict__ D, int nz, int Mx, int My,
              const cpx<R>* __restrict__ tw, const int* __restrict__ skip) {
   constexpr int M = M1 * M2, NT = T * kQ<M1, M2>, CS = ZRows<R, M1, M2, T>::rows * T;
-  pdl_wait();
-  pdl_launch();
-  if (skip && skip[blockIdx.z]) return;
   B2 += (long long)blockIdx.z * 3 * nz * My * Mx;      // right-hand side blockIdx.z
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* s_tw = reinterpret_cast<cpx<R>*>(smem_raw);
   cpx<R>* s = s_tw + M;                      // [3][rows][T]
+  load_tw(s_tw, tw, M, NT);
+  pdl_wait();
+  pdl_launch();
+  if (skip && skip[blockIdx.z]) return;
   // complex64 (interleaved octant): mirrored rows together; the double-width
   // passes measured faster in natural order
   const int bx = blockIdx.x, ky = kOctInterleaved<R> ? ky_order(blockIdx.y, My) : (int)blockIdx.y;
@@ -611,7 +612,6 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>,
   const long long col = (long long)ky * Mx + kx;
   for (int c = 0; c < 3; ++c) zc_stage<R, T, NT>(s + c * CS, B2, c, nz, Mx, My, bx, ky);
   zc_prefetch<R, M, T, NT>(D, Mx, My, bx, ky);
-  load_tw(s_tw, tw, M, NT);
   zc_forward_product_inva<R, M1, M2, T, NT>(s, s_tw, D, nz, Mx, My, bx, ky);
 #pragma unroll 1
   for (int c = 0; c < 3; ++c) zc_inverse_b<R, M1, M2, T>(s + c * CS, B2 + c * comp, nz, Mx, plane, col, kx);
@@ -657,9 +657,6 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, 3, (M1 *
   cpx<R>* a = s_tw + M;                      // [T][LD]
   // blockIdx.y = 3 * (right-hand side) + component; vectors [rhs][3][n_occ]
   const int cc = blockIdx.y, c = cc % 3;
-  pdl_wait();
-  pdl_launch();
-  if (skip && skip[cc / 3]) return;
   beta += (long long)(cc / 3) * bstride;
   // the rows transformed: those within the planes' spans of occupied rows
   // when the lattice lists them, else every row
@@ -673,6 +670,9 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, 3, (M1 *
   }
   load_tw(s_tw, tw, M, NT);
   for (int i = threadIdx.x; i < T * LD; i += NT) a[i] = zero<R>();
+  pdl_wait();
+  pdl_launch();
+  if (skip && skip[cc / 3]) return;
   __syncthreads();
   {
     // all threads over the block's dipoles (contiguous in x: rows r0..r0+T-1),
@@ -778,6 +778,7 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, kXinvB<R
   cpx<R>* a = s_tw + M;                      // [T][LD]
   V* s_x = reinterpret_cast<V*>(a + T * LD); // [kXS]
   const int cc = blockIdx.y, c = cc % 3;     // 3 * (right-hand side) + component
+  load_tw(s_tw, tw, M, NT);
   pdl_wait();
   pdl_launch();
   if (skip && skip[cc / 3]) return;
@@ -811,7 +812,6 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, kXinvB<R
   for (int k = threadIdx.x; k < staged; k += NT) cp_async_elem<sizeof(V)>(s_x + k, xc + S0 + k, true);
   cp_async_commit();
   if (threadIdx.x <= T) s_off[threadIdx.x] = off[min(r0 + (int)threadIdx.x, nr)];
-  load_tw(s_tw, tw, M, NT);
   cp_async_wait<0>();
   __syncthreads();
   const int t = threadIdx.x % T, q = threadIdx.x / T;
