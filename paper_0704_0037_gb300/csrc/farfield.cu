@@ -26,16 +26,18 @@
 //
 // One block holds the digits of 8 lattice rows (48 matrix rows, up to 144
 // inner columns: 97 KB) in shared memory, in the order the tensor-core
-// fragments are loaded, and runs all directions past them in tiles of 32,
-// whose digits stream through a two-stage ring.  Each of 4 warps takes 8
-// directions against the three tiles of 16 matrix rows (8 lattice rows, real
-// and imaginary part, of one component): 84 matrix instructions for 28
-// fragment loads.  Two blocks share an SM, so that one's sums (FP64 pipe)
-// overlap the other's products (tensor pipe).
+// fragments are loaded, and runs all directions past them in tiles of 32.  Each
+// of 4 warps takes 8 directions, whose digits it streams from L2 in fragment
+// order, against the three tiles of 16 matrix rows (8 lattice rows, real and
+// imaginary part, of one component): 84 matrix instructions for 28 fragment
+// loads.  The warps meet only when the digits of the next rows are made, and
+// two blocks share an SM, so that one warp's sums (FP64 and integer pipes)
+// overlap another's products (tensor pipe).
 //
 // 128^3 sphere, 1,152 directions, per right-hand side: direct FP64 sums 65.4 ms;
 // this product with 16 rows and 12 warps in one block per SM 3.26 ms, with two
-// blocks and integer scaling 2.58 ms (tensor pipe 42 %, FP64 pipe 43 % busy); error
+// blocks and integer scaling 2.58 ms; digits made in integer instructions 2.31 ms;
+// warps that meet only once per row block 2.0 ms; error
 // against 64-bit sums 2.0e-15 before, 1.9e-15 now.
 #include <algorithm>
 
@@ -72,25 +74,36 @@ __device__ __forceinline__ unsigned pack2(int a, int b) {
   const __nv_bfloat162 v = __floats2bfloat162_rn((float)a, (float)b);
   return *reinterpret_cast<const unsigned*>(&v);
 }
-__device__ __forceinline__ double pow2(int e) {   // 2^e, -1022 <= e <= 1023
-  return __hiloint2double((e + 1023) << 20, 0);
+// v 2^(kFix - e) rounded to an integer, for |v| <= 2^e and e >= -900, in integer
+// instructions (the FP64 pipe is the busiest one): the mantissa shifted by the
+// difference of the exponents
+__device__ __forceinline__ long long to_fixed(double v, int e) {
+  const long long b = __double_as_longlong(v);
+  const int ev = (int)(b >> 52) & 0x7ff, k = 1022 + e - ev;      // v = m 2^(ev - 1075)
+  if (k > 55 || ev == 0) return 0;
+  const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | (1ull << 52);
+  const long long t = (long long)(k < 0 ? m << 2 : ((m << 1) + ((1ull << k) >> 1)) >> k);   // k = -1: |v| = 2^e
+  return b < 0 ? -t : t;
 }
 
-// exp(-i kd n_mu r_mu) for the cells of x, then y, then z: tab[cell][n_dir]
+// exp(-i kd n_mu r_mu) for the cells of x, then y, then z: tab[cell][n_dir].
+// Cells k and n - 1 - k of an axis lie at r and -r: one sincos for both (the
+// FP64 pipe bounds this table).
 __global__ void k_ff_tab(const double* __restrict__ dirs, int n_dir, double kd, int nx, int ny,
                          int nz, c128* __restrict__ tab) {
-  const int L = nx + ny + nz;
-  const long long total = (long long)n_dir * L;
+  const int hx = (nx + 1) / 2, hy = (ny + 1) / 2, hz = (nz + 1) / 2;
+  const long long total = (long long)n_dir * (hx + hy + hz);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
     int k = (int)(i / n_dir);
     const int d = (int)(i - (long long)k * n_dir);
-    int axis = 0, n = nx;
-    if (k >= nx) { k -= nx; axis = 1; n = ny; if (k >= ny) { k -= ny; axis = 2; n = nz; } }
+    int axis = 0, n = nx, base = 0;
+    if (k >= hx) { k -= hx; axis = 1; n = ny; base = nx; if (k >= hy) { k -= hy; axis = 2; n = nz; base = nx + ny; } }
     const double r = 0.5 * (2 * k + 1 - n);
     double s, c;
     sincos(-kd * dirs[3 * d + axis] * r, &s, &c);
-    tab[i] = mk<double>(c, s);
+    tab[(long long)(base + k) * n_dir + d] = mk<double>(c, s);
+    tab[(long long)(base + n - 1 - k) * n_dir + d] = mk<double>(c, -s);
   }
 }
 
@@ -117,7 +130,7 @@ __global__ void k_ff_pack(const c128* __restrict__ tab, int n_dir, int nx, FfSha
         const c128 t = tab[(long long)(nx - sh.H + j) * n_dir + d];
         v = k < sh.J ? t.x : -t.y;
       }
-      digits(__double2ll_rn(v * pow2(kFix)), dg[u]);
+      digits(to_fixed(v, 0), dg[u]);
     }
     unsigned* o = B + blk * (kBBlk / 4) + w;
 #pragma unroll
@@ -126,14 +139,10 @@ __global__ void k_ff_pack(const c128* __restrict__ tab, int n_dir, int nx, FfSha
 }
 
 __device__ __forceinline__ void mma(float (&c)[4], const uint4& a, unsigned b0, unsigned b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
                "{%8,%9}, {%0,%1,%2,%3};"
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void copy16(void* smem, const void* gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 
 // t 2^e, rounded to nearest, put together in integer instructions: the FP64
@@ -148,12 +157,11 @@ __device__ __forceinline__ double scaled(long long t, int e) {
   return __longlong_as_double((long long)(t == 0 ? 0ull : bits | ((unsigned long long)t & (1ull << 63))));
 }
 
-// shared memory behind the A digits: ring (2 steps) and row phases; the
-// gather stage of the build phase (4 warps x 2 J cells) lies over the ring
-constexpr int kRing = 2 * kBBlk;
-constexpr int kTail = kRing + kRows * kDirs * 16;
+// shared memory behind the A digits: the gather stage of the build phase (4
+// warps x 2 J cells), then the row phases of the directions of each warp
+constexpr int kTail = kNT / 32 * 2 * kJMax * 16;
 constexpr int kBad = 1 << 20;     // scale exponent of a row with NaN or infinity
-static_assert(kNT / 32 * 2 * kJMax * 16 <= kTail, "the gather stage fits behind the digits");
+static_assert(kRows * kDirs * 16 <= kTail, "the row phases fit in the gather stage");
 
 // Partial sums of the row blocks u = blockIdx.x, + gridDim.x, ... (of units =
 // row blocks x chunks) for the direction tiles of blockIdx.y:
@@ -167,14 +175,14 @@ __global__ void __launch_bounds__(kNT, 2)
   __shared__ int s_e[kRows * 3], s_iy[kRows], s_iz[kRows];
   unsigned* A = reinterpret_cast<unsigned*>(smem);
   unsigned char* tail = smem + 3 * sh.ks * kSl * 512;
-  c128* s_w = reinterpret_cast<c128*>(tail + kRing);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2;
+  c128* s_w = reinterpret_cast<c128*>(tail) + warp * kRows * 8;   // [row][direction] of this warp
   const int t0 = blockIdx.y * tiles_per_y, t1 = min(ntiles, t0 + tiles_per_y);
   const long long* off = lat.arow ? lat.aoff : lat.row_off;
 
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
     const int rb = u / sh.nchunk, ch = u - rb * sh.nchunk, j0 = ch * sh.J;
-    __syncthreads();                         // the previous unit's reads of A, W and the ring
+    __syncthreads();                         // the previous unit's reads of A and the row phases
     // ---- digits of the 8 rows: a warp per (row, component)
     c128* stage = reinterpret_cast<c128*>(tail) + warp * 2 * kJMax;
     for (int p = warp; p < 3 * kRows; p += kNT / 32) {
@@ -195,38 +203,36 @@ __global__ void __launch_bounds__(kNT, 2)
         s_iz[r] = row / ny;
       }
       __syncwarp();
-      double m = 0.0;
-      bool bad = false;
+      // S and D in place of P(x) and P(-x), and the largest exponent field of
+      // their parts (2047: infinity or NaN)
+      int m = 0;
       for (int k = lane; k < sh.J; k += 32) {
         const c128 h = stage[k], l = stage[sh.J + k];
         const c128 s = h + l, d = h - l;
-        const double a = fmax(fmax(fabs(s.x), fabs(s.y)), fmax(fabs(d.x), fabs(d.y)));
-        bad |= !(isfinite(s.x) && isfinite(s.y) && isfinite(d.x) && isfinite(d.y));
-        m = fmax(m, a);
+        stage[k] = s;
+        stage[sh.J + k] = d;
+        m = max(max(max(m, __double2hiint(s.x) & 0x7ff00000), __double2hiint(s.y) & 0x7ff00000),
+                max(__double2hiint(d.x) & 0x7ff00000, __double2hiint(d.y) & 0x7ff00000));
       }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-      bad = __any_sync(0xffffffffu, bad);
-      // |values| <= m < 2^e (e no smaller than -900: below that the row counts as tiny)
-      const int e = max(((__double2hiint(m) >> 20) & 0x7ff) - 1022, -900);
-      const double scale = (m > 0.0 && !bad) ? pow2(kFix - e) : 0.0;
+      m = __reduce_max_sync(0xffffffffu, m) >> 20;
+      const bool bad = m == 0x7ff;
+      // |values| < 2^e (e no smaller than -900: below that the row counts as tiny)
+      const int e = max(m - 1022, -900);
       if (lane == 0) s_e[p] = bad ? kBad : e - 56;
+      __syncwarp();
       for (int kp = lane; kp < sh.ks * 8; kp += 32) {
         int dr[2][kSl], di[2][kSl];
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           const int k = 2 * kp + q;
           double re = 0.0, im = 0.0;
-          if (k < sh.J) {
-            const c128 s = stage[k] + stage[sh.J + k];
-            re = s.x; im = s.y;
-          } else if (k < 2 * sh.J) {
-            const c128 d = stage[k - sh.J] - stage[k];
-            re = d.y; im = -d.x;
+          if (k < 2 * sh.J && !bad) {
+            const c128 v = stage[k];
+            re = k < sh.J ? v.x : v.y;         // S.re, S.im | D.im, -D.re
+            im = k < sh.J ? v.y : -v.x;
           }
-          if (bad) re = im = 0.0;
-          digits(__double2ll_rn(re * scale), dr[q]);
-          digits(__double2ll_rn(im * scale), di[q]);
+          digits(to_fixed(re, e), dr[q]);
+          digits(to_fixed(im, e), di[q]);
         }
         const int s = kp >> 3, kin = (2 * kp) & 15;
         uint2* o = reinterpret_cast<uint2*>(A + ((c * sh.ks + s) * kSl) * 128 +
@@ -239,20 +245,17 @@ __global__ void __launch_bounds__(kNT, 2)
     __syncthreads();
     // ---- the product with tiles t0 .. t1 - 1, one step of 16 columns at a time
     const int e3[3] = {s_e[3 * g], s_e[3 * g + 1], s_e[3 * g + 2]};
+    // (each warp on its own: it streams the digits of its 8 directions of every
+    // tile from L2 a step ahead, so one warp's sums overlap another's products)
     const int q0 = (ch * ntiles + t0) * sh.ks, q1 = (ch * ntiles + t1) * sh.ks;
-    auto fetch = [&](int q) {
-      if (q < q1) {
-        const unsigned char* src = B + (size_t)q * kBBlk;
-        unsigned char* dst = tail + ((q - q0) & 1) * kBBlk;
-        for (int i = threadIdx.x; i < kBBlk / 16; i += kNT) copy16(dst + 16 * i, src + 16 * i);
-      }
-      asm volatile("cp.async.commit_group;\n" ::: "memory");
-    };
-    fetch(q0);
+    const uint2* bp = reinterpret_cast<const uint2*>(B) + warp * 32 + lane;
+    uint2 bn[kSl];
+#pragma unroll
+    for (int k = 0; k < kSl; ++k) bn[k] = bp[(size_t)q0 * (kBBlk / 8) + k * 128];
     int q = q0;
     for (int tile = t0; tile < t1; ++tile) {
-      for (int i = threadIdx.x; i < kRows * kDirs; i += kNT) {
-        const int r = i / kDirs, d = tile * kDirs + i % kDirs;
+      for (int i = lane; i < kRows * 8; i += 32) {
+        const int r = i >> 3, d = tile * kDirs + warp * 8 + (i & 7);
         c128 w = mk<double>(0.0, 0.0);
         if (rb * kRows + r < nr && d < n_dir)
           w = tab[(long long)(nx + s_iy[r]) * n_dir + d] * tab[(long long)(nx + ny + s_iz[r]) * n_dir + d];
@@ -273,30 +276,32 @@ __global__ void __launch_bounds__(kNT, 2)
 #pragma unroll
           for (int v = 0; v < 4; ++v) acc[n][k][v] = 0.0f;
       for (int s = 0; s < sh.ks; ++s, ++q) {
-        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-        __syncthreads();
-        fetch(q + 1);
-        const uint2* b2 = reinterpret_cast<const uint2*>(tail + ((q - q0) & 1) * kBBlk) + warp * 32 + lane;
         uint2 bf[kSl];
 #pragma unroll
-        for (int k = 0; k < kSl; ++k) bf[k] = b2[k * 128];
+        for (int k = 0; k < kSl; ++k) bf[k] = bn[k];
+        if (q + 1 < q1) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const uint4* a4 = reinterpret_cast<const uint4*>(A) + (c * sh.ks + s) * kSl * 32 + lane;
-          uint4 af[kSl];
-#pragma unroll
-          for (int k = 0; k < kSl; ++k) af[k] = a4[k * 32];
-#pragma unroll
-          for (int i = 0; i < kSl; ++i)
-#pragma unroll
-            for (int j = 0; j < kSl - i; ++j) mma(acc[c][i + j], af[i], bf[j].x, bf[j].y);
+          for (int k = 0; k < kSl; ++k) bn[k] = bp[(size_t)(q + 1) * (kBBlk / 8) + k * 128];
         }
+        uint4 af[3][kSl];
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+          for (int k = 0; k < kSl; ++k)
+            af[c][k] = reinterpret_cast<const uint4*>(A)[((c * sh.ks + s) * kSl + k) * 32 + lane];
+#pragma unroll
+        for (int i = 0; i < kSl; ++i)
+#pragma unroll
+          for (int j = 0; j < kSl - i; ++j)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) mma(acc[c][i + j], af[c][i], bf[j].x, bf[j].y);
       }
       // ---- 64-bit sums, row phases, sum over the 8 rows
+      __syncwarp();
       double v[3][2][2];                     // [component][column][re, im]
 #pragma unroll
       for (int col = 0; col < 2; ++col) {
-        const c128 w = s_w[g * kDirs + warp * 8 + (lane & 3) * 2 + col];
+        const c128 w = s_w[g * 8 + (lane & 3) * 2 + col];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           double z[2];
@@ -324,7 +329,7 @@ __global__ void __launch_bounds__(kNT, 2)
         a += __shfl_xor_sync(0xffffffffu, a, 4);
         if (mine) o[2 * c] = old[c] + a;
       }
-      __syncthreads();                       // every read of the row phases
+      __syncwarp();                          // every read of the row phases
     }
   }
 }
@@ -401,7 +406,7 @@ cudaError_t farfield_tables(void* ws, const double* dirs, int n_dir, double kd, 
   const int nt = (n_dir + kDirs - 1) / kDirs;
   c128* tab = (c128*)ws;
   unsigned* pack = (unsigned*)((unsigned char*)ws + p.tab);
-  const long long tt = (long long)n_dir * (nx + ny + nz), tp = (long long)s.nchunk * nt * s.ks * 256;
+  const long long tt = (long long)n_dir * ((nx + 1) / 2 + (ny + 1) / 2 + (nz + 1) / 2), tp = (long long)s.nchunk * nt * s.ks * 256;
   k_ff_tab<<<(int)std::min<long long>((tt + 255) / 256, 8192), 256, 0, st>>>(dirs, n_dir, kd, nx, ny, nz, tab);
   count_launch();
   k_ff_pack<<<(int)std::min<long long>((tp + 255) / 256, 8192), 256, 0, st>>>(tab, n_dir, nx, s, nt, pack);
