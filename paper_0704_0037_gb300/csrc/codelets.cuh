@@ -70,7 +70,7 @@ __host__ __device__ __forceinline__ cpx<R> tw_mul(cpx<R> z) {
   if constexpr (m == 0) {
     return z;
   } else if constexpr (2 * m == N) {
-    return mk<R>(-z.x, -z.y);
+    return cneg<R>(z);
   } else if constexpr (4 * m == N) {
     return mul_mi<R, INV>(z);
   } else if constexpr (4 * m == 3 * N) {

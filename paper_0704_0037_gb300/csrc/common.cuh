@@ -237,7 +237,9 @@ __device__ __forceinline__ df2 dsub2(df2 a, df2 b) {
   const unsigned long long e = f2sub(f2sub(a.h, f2sub(s, bb)), f2add(b.h, bb));
   return df2{s, f2add(e, f2sub(a.l, b.l))};
 }
-__device__ __forceinline__ df2 dmul2(df2 a, df2 b) {
+// Product without the final renormalisation: (p, e), p the rounded product of
+// the high words and e its error plus the cross terms (within 2 ulp of p)
+__device__ __forceinline__ df2 dmul2_raw(df2 a, df2 b) {
   // The rounded product comes from an fma with a zero addend the compiler
   // cannot see through (a - a): a paired multiply followed by the paired add
   // below may otherwise be contracted into one fused operation, which adds
@@ -247,9 +249,13 @@ __device__ __forceinline__ df2 dmul2(df2 a, df2 b) {
   unsigned long long e = f2fma(a.h, b.h, f2sub(0ull, p));
   e = f2fma(a.h, b.l, e);
   e = f2fma(a.l, b.h, e);
-  const unsigned long long h = f2add(p, e);
-  return df2{h, f2sub(e, f2sub(h, p))};
+  return df2{p, e};
 }
+__device__ __forceinline__ df2 drenorm2(df2 a) {
+  const unsigned long long h = f2add(a.h, a.l);
+  return df2{h, f2sub(a.l, f2sub(h, a.h))};
+}
+__device__ __forceinline__ df2 dmul2(df2 a, df2 b) { return drenorm2(dmul2_raw(a, b)); }
 // the pair (v, v) of a double-float scalar
 __device__ __forceinline__ df2 dsplat(df v) { return df2{pk2(v.hi, v.hi), pk2(v.lo, v.lo)}; }
 // multiply the first part by -1 (exact)
@@ -257,13 +263,16 @@ __device__ __forceinline__ df2 dneg_re(df2 a) {
   const unsigned long long m = pk2(-1.0f, 1.0f);
   return df2{f2mul(a.h, m), f2mul(a.l, m)};
 }
-// (a + ib)(c + id) = (ac - bd) + i(ad + bc): (ac, ad) + (-bd, bc)
+// (a + ib)(c + id) = (ac - bd) + i(ad + bc): (ac, ad) + (-bd, bc), renormalised
+// once, after the sum (25 paired instructions; with both products
+// renormalised before it 28, at the same error bound: what the sum loses is
+// 2^-48 of the products)
 __device__ __forceinline__ cpx<df> dcmul(const cpx<df>& z, const cpx<df>& w) {
   const df2 wp = dpack(w);
   const df2 ws{pk2(w.y.hi, w.x.hi), pk2(w.y.lo, w.x.lo)};
-  const df2 p1 = dmul2(dsplat(z.x), wp);
-  const df2 p2 = dmul2(dsplat(z.y), ws);
-  return dunpack(dadd2(p1, dneg_re(p2)));
+  const df2 p1 = dmul2_raw(dsplat(z.x), wp);
+  const df2 p2 = dmul2_raw(dsplat(z.y), ws);
+  return dunpack(drenorm2(dadd2(p1, dneg_re(p2))));
 }
 #endif
 
@@ -310,30 +319,58 @@ template <> __host__ __device__ __forceinline__ cpx<df> cnmac<df>(cpx<df> c, cpx
   return c - a * b;
 }
 
-// A real number that the compiler can know to be zero: after inlining the flag
-// is a constant, and sums with and products by a known zero disappear (an IEEE
-// addition of 0 does not fold, for the sign of -0).  Codelets instantiated on
-// cpx<pz<R>> skip the arithmetic of inputs that are padding.
+// Complex numbers that the compiler can know to be zero: after inlining the
+// flag is a constant, and sums with and products by a known zero disappear (an
+// IEEE addition of 0 does not fold, for the sign of -0, and the paired
+// instructions fold nothing).  Codelets instantiated on pz<R> skip the
+// arithmetic of inputs that are padding.
 template <typename R> struct pz {
   R v;
-  bool z;
-  __host__ __device__ constexpr pz() : v(0), z(true) {}
-  __host__ __device__ constexpr pz(R a, bool zero) : v(a), z(zero) {}
-  __host__ __device__ constexpr explicit pz(R a) : v(a), z(false) {}
+  __host__ __device__ constexpr explicit pz(double a) : v((R)a) {}
 };
 template <typename R> __host__ __device__ __forceinline__ constexpr pz<R> operator-(pz<R> a) {
-  return a.z ? a : pz<R>(-a.v, false);
+  pz<R> r = a;
+  r.v = -a.v;
+  return r;
 }
-template <typename R> __host__ __device__ __forceinline__ constexpr pz<R> operator+(pz<R> a, pz<R> b) {
-  return a.z ? b : b.z ? a : pz<R>(a.v + b.v, false);
-}
-template <typename R> __host__ __device__ __forceinline__ constexpr pz<R> operator-(pz<R> a, pz<R> b) {
-  return b.z ? a : a.z ? pz<R>(-b.v, false) : pz<R>(a.v - b.v, false);
-}
-template <typename R> __host__ __device__ __forceinline__ constexpr pz<R> operator*(pz<R> a, pz<R> b) {
-  return a.z || b.z ? pz<R>() : pz<R>(a.v * b.v, false);
-}
-template <typename R> struct cpx<pz<R>> { pz<R> x, y; };
+template <typename R> struct cpx<pz<R>> {
+  cpx<R> v;
+  bool z;
+};
+// -a
+template <typename R> __host__ __device__ __forceinline__ cpx<R> cneg(cpx<R> a) { return mk<R>(-a.x, -a.y); }
+#define DDA_KNOWN_ZEROS(R)                                                                              \
+  template <> __host__ __device__ __forceinline__ cpx<pz<R>> mk<pz<R>>(pz<R> a, pz<R> b) {              \
+    return cpx<pz<R>>{mk<R>(a.v, b.v), false};                                                          \
+  }                                                                                                     \
+  template <> __host__ __device__ __forceinline__ cpx<pz<R>> cneg<pz<R>>(cpx<pz<R>> a) {                \
+    return a.z ? a : cpx<pz<R>>{cneg<R>(a.v), false};                                                   \
+  }                                                                                                     \
+  template <> __host__ __device__ __forceinline__ cpx<pz<R>> operator+<pz<R>>(cpx<pz<R>> a, cpx<pz<R>> b) { \
+    return a.z ? b : b.z ? a : cpx<pz<R>>{a.v + b.v, false};                                            \
+  }                                                                                                     \
+  template <> __host__ __device__ __forceinline__ cpx<pz<R>> operator-<pz<R>>(cpx<pz<R>> a, cpx<pz<R>> b) { \
+    return b.z ? a : a.z ? cneg<pz<R>>(b) : cpx<pz<R>>{a.v - b.v, false};                               \
+  }                                                                                                     \
+  template <> __host__ __device__ __forceinline__ cpx<pz<R>> operator*<pz<R>>(cpx<pz<R>> a, cpx<pz<R>> b) { \
+    return a.z ? a : b.z ? b : cpx<pz<R>>{a.v * b.v, false};                                            \
+  }                                                                                                     \
+  template <> __host__ __device__ __forceinline__ cpx<pz<R>> scale<pz<R>>(cpx<pz<R>> a, pz<R> s) {      \
+    return a.z ? a : cpx<pz<R>>{scale<R>(a.v, s.v), false};                                             \
+  }                                                                                                     \
+  template <> __host__ __device__ __forceinline__ cpx<pz<R>> fmas<pz<R>>(cpx<pz<R>> a, pz<R> s, cpx<pz<R>> c) { \
+    return a.z ? c : c.z ? scale<pz<R>>(a, s) : cpx<pz<R>>{fmas<R>(a.v, s.v, c.v), false};              \
+  }                                                                                                     \
+  template <> __host__ __device__ __forceinline__ cpx<pz<R>> mul_mi<pz<R>, false>(cpx<pz<R>> a) {       \
+    return a.z ? a : cpx<pz<R>>{mul_mi<R, false>(a.v), false};                                          \
+  }                                                                                                     \
+  template <> __host__ __device__ __forceinline__ cpx<pz<R>> mul_mi<pz<R>, true>(cpx<pz<R>> a) {        \
+    return a.z ? a : cpx<pz<R>>{mul_mi<R, true>(a.v), false};                                           \
+  }
+DDA_KNOWN_ZEROS(float)
+DDA_KNOWN_ZEROS(double)
+DDA_KNOWN_ZEROS(df)
+#undef DDA_KNOWN_ZEROS
 
 __host__ __device__ __forceinline__ double df_to_double(df a) { return (double)a.hi + (double)a.lo; }
 __host__ __device__ __forceinline__ c128 to128(cdf a) {

@@ -32,7 +32,7 @@ __device__ __forceinline__ void rows_fwd(c64* P, c64* Q, int nrow, int ld, const
     c64 v[M1];
 #pragma unroll
     for (int i = 0; i < M1; ++i) v[i] = i < kHalf<M1, M2> ? P[t * ld + j + M2 * i] : zero<float>();
-    cl::Dft<float, false, M1>::run(v);
+    dft_padded<float, M1, kHalf<M1, M2>>(v);
 #pragma unroll
     for (int k1 = 1; k1 < M1; ++k1) v[k1] = twiddle<float, false>(v[k1], tw[j * k1]);
 #pragma unroll
@@ -89,7 +89,7 @@ __device__ __forceinline__ void cols_fwd(const c64* P, c64* Q, int y0, int nrow,
       const int t = j + M2 * i - y0;
       v[i] = (i < kHalf<M1, M2> && t >= 0 && t < nrow) ? P[t * ld + kx] : zero<float>();
     }
-    cl::Dft<float, false, M1>::run(v);
+    dft_padded<float, M1, kHalf<M1, M2>>(v);
 #pragma unroll
     for (int k1 = 1; k1 < M1; ++k1) v[k1] = twiddle<float, false>(v[k1], tw[j * k1]);
 #pragma unroll

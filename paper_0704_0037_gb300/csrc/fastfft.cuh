@@ -48,25 +48,23 @@ template <typename R>
 __device__ __forceinline__ cpx<R> zero() { return mk<R>((R)0, (R)0); }
 
 // Forward M1-point transform of the first phase, whose inputs v[i], i >= KH,
-// are padding.  In complex128 their arithmetic is left out (the FP64 pipe
-// bounds those passes: 1.6 operations per clock and SM); the paired complex64
-// and the double-float codelets run whole.  With the fused products of the z
-// pass, 61 x 45 x 52 ellipsoid, FP64: product 777 -> 699 us, z pass 553 -> 486.
+// are padding: their arithmetic is left out.  The passes are bound by the
+// instructions of their transforms (FP64: 1.6 operations per clock and SM;
+// double-float: the FP32 pipe; complex64: issue and the shared-memory pipe).
+// Product, whole codelets -> this: FP64 61 x 45 x 52 ellipsoid 777 -> 699 us
+// (with the fused products of the z pass); double-float 16 pairs of 46^3 cubes
+// 1,968 -> 1,903; complex64 134^3 sphere 473 -> 471, 256^3 3,677 -> 3,639.
 template <typename R, int M1, int KH>
 __device__ __forceinline__ void dft_padded(cpx<R> (&v)[M1]) {
-  if constexpr (std::is_same<R, double>::value) {
-    cpx<pz<R>> t[M1];
+  cpx<pz<R>> t[M1];
 #pragma unroll
-    for (int i = 0; i < M1; ++i) {
-      t[i].x = i < KH ? pz<R>(v[i].x) : pz<R>();
-      t[i].y = i < KH ? pz<R>(v[i].y) : pz<R>();
-    }
-    cl::Dft<pz<R>, false, M1>::run(t);
-#pragma unroll
-    for (int i = 0; i < M1; ++i) v[i] = mk<R>(t[i].x.z ? (R)0 : t[i].x.v, t[i].y.z ? (R)0 : t[i].y.v);
-  } else {
-    cl::Dft<R, false, M1>::run(v);
+  for (int i = 0; i < M1; ++i) {
+    t[i].v = v[i];
+    t[i].z = i >= KH;
   }
+  cl::Dft<pz<R>, false, M1>::run(t);
+#pragma unroll
+  for (int i = 0; i < M1; ++i) v[i] = t[i].z ? zero<R>() : t[i].v;
 }
 
 // Element type of the product's input and output vectors: the arithmetic
