@@ -41,25 +41,31 @@ constexpr int NL = 7;
 struct LayerSpec { int cin, cout, k, relu; };
 constexpr LayerSpec kSpec[NL] = {{7, 16, 3, 1},   {16, 32, 3, 1},  {32, 160, 3, 1}, {160, 160, 3, 1},
                                  {192, 32, 3, 1}, {48, 16, 3, 1},  {16, 6, 1, 0}};
-// Blocks below nb: g[co][ci][t] += sum over chunks of part[chunk][t][co][ci]
-// (fixed order; n = K3 nc sums of nc = cout cin); block nb + co: gb[co] +=
-// sum_v gout[co][v] (fixed-order reduction)
-__global__ void __launch_bounds__(256) k_sum_chunks(const float* __restrict__ part, int chunks, long long n,
-                                                    long long nc, float* __restrict__ g, int nb,
+// Blocks below nb = cout ceil(cin / 8): g[co][ci][t] += sum over chunks of
+// part[chunk][t][co][ci] (fixed order) for one co and 8 ci, a thread per
+// weight, read along ci, turned in shared memory and written along t; block
+// nb + co: gb[co] += sum_v gout[co][v] (fixed-order reduction)
+__global__ void __launch_bounds__(256) k_sum_chunks(const float* __restrict__ part, int chunks, int k3,
+                                                    int cin, int cout, float* __restrict__ g, int nb,
                                                     const float* __restrict__ gout, long long nv,
                                                     float* __restrict__ gb) {
+  __shared__ float sh[256];
   if ((int)blockIdx.x < nb) {
-    for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += nb * 256LL) {
+    const int cb = (cin + 7) / 8, co = blockIdx.x / cb, c0 = (blockIdx.x % cb) * 8, nc = min(8, cin - c0);
+    const long long n = (long long)k3 * cout * cin;
+    const int t = threadIdx.x >> 3, ci = threadIdx.x & 7;
+    if (t < k3 && ci < nc) {
+      const float* p = part + ((long long)t * cout + co) * cin + c0 + ci;
       float s = 0.0f;
-#pragma unroll 8
-      for (int c = 0; c < chunks; ++c) s += part[c * n + i];
-      const long long t = i / nc;
-      g[(i - t * nc) * (n / nc) + t] += s;
+#pragma unroll 16
+      for (int c = 0; c < chunks; ++c) s += p[c * n];
+      sh[ci * k3 + t] = s;
     }
+    __syncthreads();
+    if ((int)threadIdx.x < nc * k3) g[((long long)co * cin + c0) * k3 + threadIdx.x] += sh[threadIdx.x];
     return;
   }
   const int co = blockIdx.x - nb;
-  __shared__ float sh[256];
   float s = 0.0f;
 #pragma unroll 8
   for (long long v = threadIdx.x; v < nv; v += 256) s += gout[co * nv + v];
@@ -147,7 +153,7 @@ __global__ void k_idx_map(LatticeDev lat, int nx, int ny, int nrows, int* __rest
 __global__ void __launch_bounds__(256) k_feat_in(const c128* __restrict__ v, long long n_occ,
                                                  const int* __restrict__ map, Dims dl, Dims d0,
                                                  const double* __restrict__ scl, float* __restrict__ f) {
-  const double inv = scl[5];
+  const double inv = scl[5] * 0.125;           // exact: a power of two
   const int c = blockIdx.y;
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < d0.n();
        p += (long long)gridDim.x * blockDim.x) {
@@ -168,8 +174,8 @@ __global__ void __launch_bounds__(256) k_feat_in(const c128* __restrict__ v, lon
       re += a.x;
       im += a.y;
     }
-    f[(2 * c) * d0.n() + p] = (float)(re * inv * 0.125);
-    f[(2 * c + 1) * d0.n() + p] = (float)(im * inv * 0.125);
+    f[(2 * c) * d0.n() + p] = (float)(re * inv);
+    f[(2 * c + 1) * d0.n() + p] = (float)(im * inv);
     if (c == 0) f[6 * d0.n() + p] = occ * 0.125f;
   }
 }
@@ -231,9 +237,10 @@ __global__ void __launch_bounds__(256) k_loss_grad(const c128* __restrict__ zz, 
 }
 
 // per-block partial sums of |a|^2 (slot 0) and |a - b|^2 (slot 1; b may be
-// null), four elements in flight per thread; k_sq_fin adds the kSqB blocks in
-// a fixed order
+// null), four elements in flight per thread; k_sq_fin adds the sq_blocks(n) of
+// them (at most kSqB) in a fixed order
 constexpr int kSqB = 1024;
+inline int sq_blocks(long long n) { return (int)std::max<long long>(1, std::min<long long>((n + 1023) / 1024, kSqB)); }
 __global__ void __launch_bounds__(256) k_sq_part(const c128* __restrict__ a, const c128* __restrict__ b,
                                                  long long n, double* __restrict__ part) {
   __shared__ double sh[2][256];
@@ -265,12 +272,11 @@ __global__ void __launch_bounds__(256) k_sq_part(const c128* __restrict__ a, con
 // one block of 256 threads: the sums of slots 0 and 1 go to sc[0] as rms =
 // sqrt(s0 / n), sc[5] = 1 / rms (n > 0), or to sc[3] = s0, sc[4] = s1 and sc[6]
 // = 1 / s0 (n = 0); reciprocals of zero are 0
-__global__ void __launch_bounds__(256) k_sq_fin(const double* __restrict__ part, double* __restrict__ sc,
-                                                long long n) {
+__global__ void __launch_bounds__(256) k_sq_fin(const double* __restrict__ part, int nb,
+                                                double* __restrict__ sc, long long n) {
   __shared__ double sh[2][256];
   double s0 = 0.0, s1 = 0.0;
-#pragma unroll
-  for (int b = threadIdx.x; b < kSqB; b += 256) { s0 += part[2 * b]; s1 += part[2 * b + 1]; }
+  for (int b = threadIdx.x; b < nb; b += 256) { s0 += part[2 * b]; s1 += part[2 * b + 1]; }
   sh[0][threadIdx.x] = s0;
   sh[1][threadIdx.x] = s1;
   __syncthreads();
@@ -485,15 +491,19 @@ int conv_bwd_weight(dda_pcnet_t net, int L, const Acts& A, const float* gout, Di
     }
     net->part_bytes = need;
   }
-  if (s.k == 3)
-    k_wgrad_f32<<<dim3(chunks, (s.cout + 7) / 8, (s.cin + 15) / 16), 216, 0, st>>>(layer_input(A, L), gout,
-                                                                                   s.cout, d, net->part, per);
-  else
+  if (s.k == 3) {
+    const size_t sm = (size_t)(per > 1 ? 2 : 1) * kWTile * sizeof(float);
+    cudaError_t e = ensure_smem((const void*)k_wgrad_f32, sm);
+    if (e == cudaSuccess) e = ensure_carveout_max((const void*)k_wgrad_f32);
+    if (e != cudaSuccess) return pc_fail(net, DDA_ERR_CUDA, cudaGetErrorString(e));
+    k_wgrad_f32<<<dim3(chunks, (s.cout + 7) / 8, (s.cin + 15) / 16), 216, sm, st>>>(layer_input(A, L), gout,
+                                                                                    s.cout, d, net->part, per);
+  } else
     k_wgrad1<<<chunks, 96, 0, st>>>(A.a5, s.cin, gout, s.cout, d, net->part, per);
   count_launch();
-  const int nb = gs(nw);
-  k_sum_chunks<<<nb + s.cout, 256, 0, st>>>(net->part, chunks, nw, nw / K3, net->g + net->woff[L], nb, gout, d.n(),
-                                            net->g + net->boff[L]);
+  const int nb = s.cout * ((s.cin + 7) / 8);
+  k_sum_chunks<<<nb + s.cout, 256, 0, st>>>(net->part, chunks, K3, s.cin, s.cout, net->g + net->woff[L], nb, gout,
+                                            d.n(), net->g + net->boff[L]);
   count_launch();
   return DDA_OK;
 }
@@ -514,9 +524,9 @@ int forward(dda_pcnet_t net, dda_t h, const c128* v, c128* z, Acts& A, bool trai
   cudaStream_t st = h->stream;
   const long long n = 3 * h->g.n_occ;
   const Dims dl{h->g.nx, h->g.ny, h->g.nz};
-  k_sq_part<<<kSqB, 256, 0, st>>>(v, nullptr, n, net->red);
+  k_sq_part<<<sq_blocks(n), 256, 0, st>>>(v, nullptr, n, net->red);
   count_launch();
-  k_sq_fin<<<1, 256, 0, st>>>(net->red, net->scal, n);     // rms(v)
+  k_sq_fin<<<1, 256, 0, st>>>(net->red, sq_blocks(n), net->scal, n);     // rms(v)
   count_launch();
   k_feat_in<<<dim3(gs(A.d0.n()), 3), 256, 0, st>>>(v, h->g.n_occ, net->map, dl, A.d0, net->scal, A.f0);
   count_launch();
@@ -601,19 +611,18 @@ extern "C" int dda_pcnet_create(dda_pcnet_t* out, unsigned long long seed) {
     off += kSpec[L].cout;
   }
   net->nparam = off;
-  long long pat = 0, patf = 0;
+  int pat = 0, patf = 0;
   net->pack.count = NL;
   net->packf.count = 2 * NL;
   for (int q = 0; q < 2 * NL; ++q) {
     const LayerSpec& s = kSpec[q % NL];
     const int flip = q >= NL, ni = flip ? s.cout : s.cin, no = flip ? s.cin : s.cout, k3 = s.k * s.k * s.k;
-    const long long n = (long long)((ni + 15) / 16) * k3 * ((no + 7) / 8) * 32;
-    const long long nf = (long long)ni * k3 * ((no + 7) / 8 * 8);
+    const int n = ((ni + 15) / 16) * k3 * ((no + 7) / 8) * 32, nf = ni * k3 * ((no + 7) / 8 * 8);
     if (!flip) {
-      net->pack.item[q] = {net->woff[q], s.cin, s.cout, k3, 0, pat, n};
+      net->pack.item[q] = {(int)net->woff[q], s.cin, s.cout, k3, 0, pat, n};
       pat += n;
     }
-    net->packf.item[q] = {net->woff[q % NL], s.cin, s.cout, k3, flip, patf, nf};
+    net->packf.item[q] = {(int)net->woff[q % NL], s.cin, s.cout, k3, flip, patf, nf};
     patf += nf;
   }
   // He-normal weights from a seeded host generator, zero biases; the last
@@ -735,9 +744,9 @@ extern "C" int dda_pcnet_train_step(dda_pcnet_t net, dda_t h, const void* r_dev,
   if ((rc = forward(net, h, r, z, A, true)) != DDA_OK) return rc;
   // |e|^2 into scal[3], |z - e|^2 into scal[4] (scal[0] keeps rms(r))
   const long long n = 3 * h->g.n_occ;
-  k_sq_part<<<kSqB, 256, 0, st>>>(e, z, n, net->red);
+  k_sq_part<<<sq_blocks(n), 256, 0, st>>>(e, z, n, net->red);
   count_launch();
-  k_sq_fin<<<1, 256, 0, st>>>(net->red, net->scal, 0);   // scal[3] = |e|^2, scal[4] = |e - z|^2
+  k_sq_fin<<<1, 256, 0, st>>>(net->red, sq_blocks(n), net->scal, 0);   // scal[3] = |e|^2, scal[4] = |e - z|^2
   count_launch();
   if (cudaMemsetAsync(net->g, 0, net->nparam * sizeof(float), st) != cudaSuccess)
     return pc_fail(net, DDA_ERR_CUDA, "gradient reset");

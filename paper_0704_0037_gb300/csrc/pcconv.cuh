@@ -21,7 +21,7 @@
 //
 // 128^3 sphere (31 GFLOP a pass): 2.09 ms of convolutions on the FP32 pipe
 // before, 0.39 ms now (48 to 16 channels at 64^3 voxels 435 -> 130 us); the
-// pass 2.36 -> 0.51 ms; error of N(r) against 64 bits 4.5e-7 before, 1.6e-7 now.
+// pass 2.36 -> 0.50 ms; error of N(r) against 64 bits 4.5e-7 before, 1.6e-7 now.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -59,13 +59,13 @@ __device__ __forceinline__ void cp4(void* smem, const float* gmem, bool ok) {
 __device__ __forceinline__ void ldm4(unsigned (&r)[4], const void* smem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(sa) : "memory");
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(sa));
 }
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-               "{%8,%9}, {%0,%1,%2,%3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 // x = hi + mid + lo, exact for every normal float whose parts stay normal
 __device__ __forceinline__ void split3(float x, __nv_bfloat16 (&s)[3]) {
@@ -268,22 +268,21 @@ __global__ void __launch_bounds__(128) k_conv_mma(ConvIn in, const uint2* __rest
 // Weights in fragment order, all layers in one launch: entry of layer L's
 // forward product (output channels co, input ci) or of its input gradient
 // (output ci, input co, taps reversed).
-struct PackItem { long long w; int cin, cout, k3, flip; long long at, n; };   // n uint2 from at
+struct PackItem { int w, cin, cout, k3, flip, at, n; };   // weights from w; n elements from at
 struct PackList { PackItem item[14]; int count; };
-__global__ void k_pack_weights(const __nv_bfloat16* __restrict__ w, PackList pl, uint2* __restrict__ out,
-                               long long total) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
+__global__ void k_pack_weights(const __nv_bfloat16* __restrict__ w, const __grid_constant__ PackList pl,
+                               uint2* __restrict__ out, int total) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
     int q = 0;
     while (q + 1 < pl.count && i >= pl.item[q + 1].at) ++q;
     const PackItem& p = pl.item[q];
     const int ni = p.flip ? p.cout : p.cin, no = p.flip ? p.cin : p.cout, ntn = (no + 7) / 8;
-    long long j = i - p.at;
-    const int lane = (int)(j & 31);
+    int j = i - p.at;
+    const int lane = j & 31;
     j >>= 5;
-    const int nt = (int)(j % ntn);
+    const int nt = j % ntn;
     j /= ntn;
-    const int t = (int)(j % p.k3), blk = (int)(j / p.k3);
+    const int t = j % p.k3, blk = j / p.k3;
     const int o = nt * 8 + (lane >> 2);
     unsigned r[2];
 #pragma unroll
@@ -293,8 +292,7 @@ __global__ void k_pack_weights(const __nv_bfloat16* __restrict__ w, PackList pl,
       for (int e = 0; e < 2; ++e) {
         const int c = blk * 16 + b * 8 + (lane & 3) * 2 + e;
         if (c < ni && o < no) {
-          const long long at = p.flip ? ((long long)c * p.cin + o) * p.k3 + (p.k3 - 1 - t)
-                                      : ((long long)o * p.cin + c) * p.k3 + t;
+          const int at = p.flip ? (c * p.cin + o) * p.k3 + (p.k3 - 1 - t) : (o * p.cin + c) * p.k3 + t;
           u |= (unsigned)__bfloat16_as_ushort(w[p.w + at]) << (16 * e);
         }
       }
@@ -320,7 +318,7 @@ cudaError_t conv_mma_t(const ConvIn& in, const uint2* wp, const float* bias, con
   return cudaGetLastError();
 }
 
-// Tile of a convolution (K = 3): of 128 or 64 voxels by 32, 16 or 8 output
+// Tile of a convolution (K = 3): of 128 or 64 voxels by 40, 32, 16 or 8 output
 // channels, the one with the least estimated time: rounds of blocks over the
 // SMs times a block's cost in matrix instructions, which the smaller tiles
 // raise by what they load per instruction (a warp of the largest tile issues
@@ -334,11 +332,12 @@ inline cudaError_t conv_mma(int K, const ConvIn& in, const uint2* wp, const floa
     const long long b = (long long)((d.x + 7) / 8) * ((d.y + 3) / 4) * ((d.z + 2 * mt - 1) / (2 * mt)) * (cout / (8 * nt));
     return (double)((b + num_sms() - 1) / num_sms()) * block;
   };
-  const double c[4] = {cost(2, 4, 24.0), cost(2, 2, 13.5), cost(1, 2, 8.5), cost(1, 1, 6.0)};
-  switch ((int)(std::min_element(c, c + 4) - c)) {
+  const double c[5] = {cost(2, 4, 24.0), cost(2, 5, 30.0), cost(2, 2, 13.5), cost(1, 2, 8.5), cost(1, 1, 6.0)};
+  switch ((int)(std::min_element(c, c + 5) - c)) {
     case 0: return conv_mma_t<3, 2, 4>(in, wp, bias, mask, out, cout, d, relu, st);
-    case 1: return conv_mma_t<3, 2, 2>(in, wp, bias, mask, out, cout, d, relu, st);
-    case 2: return conv_mma_t<3, 1, 2>(in, wp, bias, mask, out, cout, d, relu, st);
+    case 1: return conv_mma_t<3, 2, 5>(in, wp, bias, mask, out, cout, d, relu, st);
+    case 2: return conv_mma_t<3, 2, 2>(in, wp, bias, mask, out, cout, d, relu, st);
+    case 3: return conv_mma_t<3, 1, 2>(in, wp, bias, mask, out, cout, d, relu, st);
   }
   return conv_mma_t<3, 1, 1>(in, wp, bias, mask, out, cout, d, relu, st);
 }
@@ -351,7 +350,7 @@ inline cudaError_t conv_mma(int K, const ConvIn& in, const uint2* wp, const floa
 // Pairs of outputs run in the paired instruction (each half rounds as the
 // scalar one).  On small lattices a sum is one long dependent chain: what
 // helps is every SM busy, operands copied ahead and few instructions per tap.
-// 64 x 45 x 37 ellipsoid: training step 2.60 -> 0.91 ms, same bits.
+// 64 x 45 x 37 ellipsoid: training step 2.60 -> 0.85 ms, same bits.
 
 // a thread's CO outputs at one voxel, pairwise
 __device__ __forceinline__ unsigned long long pair2(float a, float b) {
@@ -425,11 +424,19 @@ __global__ void __launch_bounds__(128) k_conv_f32(ConvIn in, const float* __rest
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
   };
-  unsigned long long acc[CO / 2];
+  // pairs for 8 channels; fewer run the scalar instruction, whose result is
+  // back sooner (with few warps the chain of a sum is what takes the time)
+  constexpr bool PAIRS = CO == 8;
+  unsigned long long acc2[PAIRS ? CO / 2 : 1];
+  float acc[CO];
 #pragma unroll
-  for (int k = 0; k < CO / 2; ++k) {
-    const int co = co0 + cg * CO + 2 * k;
-    acc[k] = pair2(bias && co < cout ? bias[co] : 0.0f, bias && co + 1 < cout ? bias[co + 1] : 0.0f);
+  for (int k = 0; k < CO; ++k) {
+    const int co = co0 + cg * CO + k;
+    acc[k] = bias && co < cout ? bias[co] : 0.0f;
+  }
+  if constexpr (PAIRS) {
+#pragma unroll
+    for (int k = 0; k < CO / 2; ++k) acc2[k] = pair2(acc[2 * k], acc[2 * k + 1]);
   }
   const int hv0 = (wz * T::HY + (lane >> 3)) * T::HX + (lane & 7);
   fetch(0);
@@ -450,49 +457,55 @@ __global__ void __launch_bounds__(128) k_conv_f32(ConvIn in, const float* __rest
 #pragma unroll
       for (int t = 0; t < K3; ++t) {
         const float v = si[((t / (K * K)) * T::HY + (t / K) % K) * T::HX + t % K];
-        const unsigned long long vv = pair2(v, v);
-        const unsigned long long* w = reinterpret_cast<const unsigned long long*>(sw + t * NB);
+        if constexpr (PAIRS) {
+          const unsigned long long vv = pair2(v, v);
+          const unsigned long long* w = reinterpret_cast<const unsigned long long*>(sw + t * NB);
 #pragma unroll
-        for (int k = 0; k < CO / 2; ++k) fma2(acc[k], w[k], vv);
+          for (int k = 0; k < CO / 2; ++k) fma2(acc2[k], w[k], vv);
+        } else {
+#pragma unroll
+          for (int k = 0; k < CO; ++k) acc[k] = fmaf(sw[t * NB + k], v, acc[k]);
+        }
       }
+    }
+  }
+  if constexpr (PAIRS) {
+#pragma unroll
+    for (int k = 0; k < CO / 2; ++k) {
+      const float2 r = unpair2(acc2[k]);
+      acc[2 * k] = r.x;
+      acc[2 * k + 1] = r.y;
     }
   }
   const int x = tx0 + (lane & 7), y = ty0 + (lane >> 3), z = tz0 + wz;
   if (x >= d.x || y >= d.y || z >= d.z) return;
   const long long v = ((long long)z * d.y + y) * d.x + x;
 #pragma unroll
-  for (int k = 0; k < CO / 2; ++k) {
-    const float2 r2 = unpair2(acc[k]);
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int co = co0 + cg * CO + 2 * k + e;
-      if (co < cout) {
-        float r = e ? r2.y : r2.x;
-        if (relu) r = fmaxf(r, 0.0f);
-        if (mask && !(mask[co * nv + v] > 0.0f)) r = 0.0f;
-        out[co * nv + v] = r;
-      }
+  for (int k = 0; k < CO; ++k) {
+    const int co = co0 + cg * CO + k;
+    if (co < cout) {
+      float r = acc[k];
+      if (relu) r = fmaxf(r, 0.0f);
+      if (mask && !(mask[co * nv + v] > 0.0f)) r = 0.0f;
+      out[co * nv + v] = r;
     }
   }
 }
 
 // FP32 weights [ci][t][coutp] of every layer's forward product and of its
 // input gradient (input co, output ci, taps reversed); n floats from at
-__global__ void k_pack_f32(const __nv_bfloat16* __restrict__ w, PackList pl, float* __restrict__ out,
-                           long long total) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
+__global__ void k_pack_f32(const __nv_bfloat16* __restrict__ w, const __grid_constant__ PackList pl,
+                           float* __restrict__ out, int total) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
     int q = 0;
     while (q + 1 < pl.count && i >= pl.item[q + 1].at) ++q;
     const PackItem& p = pl.item[q];
     const int no = p.flip ? p.cin : p.cout, nop = (no + 7) / 8 * 8;
-    const long long j = i - p.at;
-    const int o = (int)(j % nop);
-    const int t = (int)((j / nop) % p.k3), c = (int)(j / nop / p.k3);
+    const int j = i - p.at, r0 = j / nop, o = j - r0 * nop, c = r0 / p.k3, t = r0 - c * p.k3;
     float r = 0.0f;
     if (o < no)
-      r = __bfloat162float(w[p.w + (p.flip ? ((long long)c * p.cin + o) * p.k3 + (p.k3 - 1 - t)
-                                           : ((long long)o * p.cin + c) * p.k3 + t)]);
+      r = __bfloat162float(w[p.w + (p.flip ? (c * p.cin + o) * p.k3 + (p.k3 - 1 - t)
+                                           : (o * p.cin + c) * p.k3 + t)]);
     out[i] = r;
   }
 }
@@ -507,7 +520,9 @@ cudaError_t conv_f32_t(const ConvIn& in, const float* wf, const float* bias, con
 }
 
 // 128, 64 or 32 voxels per block: the least rounds of blocks over the SMs
-// times instructions per tap (8, 5.5 and 4.5 with their loads)
+// times instructions per tap (8, 5.5 and 4.5 with their loads).  Of the layers
+// at 1/4 and 1/8 resolution, 33 us with the 64-voxel tile this picks and 46 with
+// the 32-voxel one (both under one round).
 inline cudaError_t conv_f32(int K, const ConvIn& in, const float* wf, const float* bias, const float* mask,
                             float* out, int cout, Dims d, int relu, cudaStream_t st) {
   if (K == 1) return conv_f32_t<1, 1, 2>(in, wf, bias, mask, out, cout, d, relu, st);
@@ -528,11 +543,15 @@ inline cudaError_t conv_f32(int K, const ConvIn& in, const float* wf, const floa
 // their sums: 2 shared-memory loads for 8 paired multiply-adds.  grid (chunks,
 // output-channel blocks, input-channel blocks), 216 threads.
 constexpr int kWX = 8, kWY = 8, kWZ = 4, kWV = kWX * kWY * kWZ;
+constexpr int kWHX = kWX + 2, kWHY = kWY + 2, kWHV = kWHX * kWHY * (kWZ + 2);
+// halo rows are 11 voxels apart in shared memory: taps t and t + 1 are then an
+// odd number of 64-byte voxels apart, and a quarter warp (two taps) reads all
+// 32 banks
+constexpr int kWPX = kWX + 3, kWPV = kWPX * kWHY * (kWZ + 2);
+constexpr int kWTile = kWPV * 16 + kWV * 8;               // floats of a tile: [halo voxel][16], [voxel][8]
 __global__ void __launch_bounds__(216) k_wgrad_f32(ConvIn in, const float* __restrict__ gout, int cout,
                                                    Dims d, float* __restrict__ part, int tiles_per_chunk) {
-  constexpr int HX = kWX + 2, HY = kWY + 2, HZ = kWZ + 2, HV = HX * HY * HZ;
-  __shared__ __align__(16) float s_in[HV][16];
-  __shared__ __align__(16) float s_g[kWV][8];
+  extern __shared__ __align__(16) float smem_w[];          // two tiles: one arrives while one is summed
   const int ntx = (d.x + kWX - 1) / kWX, nty = (d.y + kWY - 1) / kWY, ntz = (d.z + kWZ - 1) / kWZ;
   const int ntiles = ntx * nty * ntz, co0 = blockIdx.y * 8, c0 = blockIdx.z * 16, cin = in.ca + in.cb;
   const long long nv = d.n(), na = in.up ? in.da.n() : nv;
@@ -541,41 +560,56 @@ __global__ void __launch_bounds__(216) k_wgrad_f32(ConvIn in, const float* __res
   const long long cs = fa ? na : nv;
   const int lim = (fa ? in.ca : cin) - c0;
   const int cig = threadIdx.x & 3, t = (threadIdx.x >> 2) % 27, cog = threadIdx.x / 108;
-  const int hv0 = ((t / 9) * HY + (t / 3) % 3) * HX + t % 3;
+  const int hv0 = ((t / 9) * kWHY + (t / 3) % 3) * kWPX + t % 3;
+  // a quarter warp copies 8 voxels of a channel, the four quarters four channels
+  auto fetch = [&](int tile, float* buf) {
+    const int tx0 = (tile % ntx) * kWX, ty0 = ((tile / ntx) % nty) * kWY, tz0 = (tile / (ntx * nty)) * kWZ;
+    for (int i = threadIdx.x; i < kWHV * 4; i += 216) {
+      const int q = i & 3, hv = i >> 2;
+      const int x = tx0 + hv % kWHX - 1, y = ty0 + (hv / kWHX) % kWHY - 1, z = tz0 + hv / (kWHX * kWHY) - 1;
+      const bool ok = x >= 0 && y >= 0 && z >= 0 && x < d.x && y < d.y && z < d.z;
+      const long long v = up ? ((long long)(z / 2) * in.da.y + y / 2) * in.da.x + x / 2
+                             : ((long long)z * d.y + y) * d.x + x;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int ch = 4 * c + q;
+        const bool k = ok && ch < lim;
+        cp4(buf + (hv / kWHX * kWPX + hv % kWHX) * 16 + ch, k ? src + ch * cs + v : in.a, k);
+      }
+    }
+    float* g = buf + kWPV * 16;
+    for (int i = threadIdx.x; i < kWV * 4; i += 216) {
+      const int q = i & 3, u = i >> 2;
+      const int x = tx0 + u % kWX, y = ty0 + (u / kWX) % kWY, z = tz0 + u / (kWX * kWY);
+      const bool ok = x < d.x && y < d.y && z < d.z;
+      const long long v = ((long long)z * d.y + y) * d.x + x;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int co = 4 * c + q;
+        const bool k = ok && co0 + co < cout;
+        cp4(g + u * 8 + co, k ? gout + (co0 + co) * nv + v : gout, k);
+      }
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
   unsigned long long acc[4][2];                // [output channel][pair of input channels]
 #pragma unroll
   for (int k = 0; k < 4; ++k) acc[k][0] = acc[k][1] = 0ull;
   const int t0 = blockIdx.x * tiles_per_chunk, t1 = min(ntiles, t0 + tiles_per_chunk);
+  if (t0 < t1) fetch(t0, smem_w);
   for (int tile = t0; tile < t1; ++tile) {
-    const int tx0 = (tile % ntx) * kWX, ty0 = ((tile / ntx) % nty) * kWY, tz0 = (tile / (ntx * nty)) * kWZ;
-    __syncthreads();
-    for (int i = threadIdx.x; i < HV * 4; i += 216) {          // 4 channels of a voxel
-      const int q = i / HV, hv = i - q * HV;
-      const int x = tx0 + hv % HX - 1, y = ty0 + (hv / HX) % HY - 1, z = tz0 + hv / (HX * HY) - 1;
-      const bool ok = x >= 0 && y >= 0 && z >= 0 && x < d.x && y < d.y && z < d.z;
-      const long long v = up ? ((long long)(z / 2) * in.da.y + y / 2) * in.da.x + x / 2
-                             : ((long long)z * d.y + y) * d.x + x;
-      float f[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) f[c] = ok && 4 * q + c < lim ? src[(4 * q + c) * cs + v] : 0.0f;
-      *reinterpret_cast<float4*>(&s_in[hv][4 * q]) = make_float4(f[0], f[1], f[2], f[3]);
-    }
-    for (int i = threadIdx.x; i < kWV * 2; i += 216) {
-      const int q = i / kWV, u = i - q * kWV;
-      const int x = tx0 + u % kWX, y = ty0 + (u / kWX) % kWY, z = tz0 + u / (kWX * kWY);
-      const bool ok = x < d.x && y < d.y && z < d.z;
-      float f[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int co = co0 + 4 * q + c;
-        f[c] = ok && co < cout ? gout[co * nv + ((long long)z * d.y + y) * d.x + x] : 0.0f;
-      }
-      *reinterpret_cast<float4*>(&s_g[u][4 * q]) = make_float4(f[0], f[1], f[2], f[3]);
+    const float* buf = smem_w + ((tile - t0) & 1) * kWTile;
+    __syncthreads();                           // the sums over the buffer fetched next are done
+    if (tile + 1 < t1) {
+      fetch(tile + 1, smem_w + ((tile + 1 - t0) & 1) * kWTile);
+      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     }
     __syncthreads();
     for (int r = 0; r < kWY * kWZ; ++r) {
-      const float* a = &s_in[hv0 + ((r / kWY) * HY + r % kWY) * HX][4 * cig];
-      const float* g = &s_g[r * kWX][4 * cog];
+      const float* a = buf + (hv0 + ((r / kWY) * kWHY + r % kWY) * kWPX) * 16 + 4 * cig;
+      const float* g = buf + kWPV * 16 + r * kWX * 8 + 4 * cog;
 #pragma unroll
       for (int u = 0; u < kWX; ++u) {
         const ulonglong2 x2 = *reinterpret_cast<const ulonglong2*>(a + 16 * u);
