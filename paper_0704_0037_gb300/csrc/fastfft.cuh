@@ -256,6 +256,10 @@ __device__ __forceinline__ int fold_axis(int k, int M, int& neg) {
   return k;
 }
 
+// Elements kept for the twiddle table in front of the z pass's tile: an even
+// number, so that the tile takes 16-byte copies whatever the length's parity
+template <int M> constexpr int kTwLen = (M + 1) / 2 * 2;
+
 // Shared-memory rows of one component of the fused z pass: row k1 M2 + j of
 // the two-level split (j < M2) lives in physical row k1 (M2 + 1) + j when a
 // tile row is narrower than the 32 banks (T complex64 < 16 columns), so that
@@ -589,14 +593,14 @@ __device__ __forceinline__ void zc_inverse_b(const cpx<R>* sc, cpx<R>* __restric
 
 template <typename R, int M1, int M2, int T>
 __global__ void __launch_bounds__(T * kQ<M1, M2>,
-                                  kMinB(T * kQ<M1, M2>, 2, (M1 * M2 + 3LL * ZRows<R, M1, M2, T>::rows * T) * sizeof(cpx<R>)))
+                                  kMinB(T * kQ<M1, M2>, 2, (kTwLen<M1 * M2> + 3LL * ZRows<R, M1, M2, T>::rows * T) * sizeof(cpx<R>)))
     fk_zconv(cpx<R>* __restrict__ B2, const cpx<R>* __restrict__ D, int nz, int Mx, int My,
              const cpx<R>* __restrict__ tw, const int* __restrict__ skip) {
   constexpr int M = M1 * M2, NT = T * kQ<M1, M2>, CS = ZRows<R, M1, M2, T>::rows * T;
   B2 += (long long)blockIdx.z * 3 * nz * My * Mx;      // right-hand side blockIdx.z
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* s_tw = reinterpret_cast<cpx<R>*>(smem_raw);
-  cpx<R>* s = s_tw + M;                      // [3][rows][T]
+  cpx<R>* s = s_tw + kTwLen<M>;              // [3][rows][T]
   load_tw(s_tw, tw, M, NT);
   pdl_wait();
   pdl_launch();
@@ -1041,7 +1045,7 @@ struct Passes {
   template <int TC>
   static cudaError_t zconv_t(cpx<R>* B2, const cpx<R>* D, int nz, int Mx, int My, const cpx<R>* tw,
                              int nrhs, const int* skip, cudaStream_t st, bool pdl) {
-    const size_t sm = (size_t)(M + 3 * ZRows<R, M1, M2, TC>::rows * TC) * sizeof(cpx<R>);
+    const size_t sm = (size_t)(kTwLen<M> + 3 * ZRows<R, M1, M2, TC>::rows * TC) * sizeof(cpx<R>);
     cudaError_t e = set_smem(fk_zconv<R, M1, M2, TC>, sm);
     if (e != cudaSuccess) return e;
     // two ~106 KB blocks per SM need the largest shared-memory carveout

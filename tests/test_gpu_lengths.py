@@ -54,3 +54,11 @@ def test_length_on_each_axis(length):
 @pytest.mark.parametrize("box", [(66, 90, 71), (95, 74, 82)])
 def test_three_lengths(box):
     _check(inputs.ellipsoid(*box))
+
+
+@pytest.mark.parametrize("length", [n for n in sorted(LENGTHS) if n % 2])
+def test_odd_z_length_with_16_byte_rows(length):
+    """x padded to an even length: the z pass stages its tile, which follows a
+    table of an odd number of elements, in 16-byte copies."""
+    n = LENGTHS[length][1]
+    _check(inputs.random_occupancy(16, 5, n, fill=0.6, seed=n), 2, length)
