@@ -759,8 +759,9 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, 3, (M1 *
 template <int M> constexpr int kXRow = (M + 1) / 2 < 384 ? (M + 1) / 2 : 384;
 // blocks per SM the x inverse pass's launch bound asks for: four in
 // complex64 (at 270 points 56 registers, no spill: P5 of the 134^3 sphere
-// 59 -> 55 us), three in the wider arithmetic
-template <typename R, int M> constexpr int kXinvB = (sizeof(R) == 4) ? 4 : 3;
+// 59 -> 55 us), three in the wider arithmetic and from 290 points (eight rows,
+// 20 and more elements a thread: 512 points 380 us with three, 475 with two)
+template <typename R, int M> constexpr int kXinvB = (sizeof(R) == 4 && (M < 290 || M >= 1000)) ? 4 : 3;
 
 template <typename R, int M1, int M2, int T, bool CONJ>
 __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, kXinvB<R, M1 * M2>, (M1 * M2 + T * kLD<M1 * M2>) * sizeof(cpx<R>) + T * kXRow<M1 * M2> * sizeof(typename VecOf<R>::type))) fk_xinv(const cpx<R>* __restrict__ B1,
@@ -981,8 +982,6 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, 3, 1)) f
 
 // ---------------------------------------------------------------- launchers
 template <typename R> constexpr int kT = sizeof(R) == 4 ? 16 : 8;
-// rows per block of the x passes (fast_x_rows gives the same on the host)
-template <typename R, int M> constexpr int kTX = (sizeof(R) == 4 && M >= 1000) ? 4 : kT<R>;
 
 template <typename K>
 inline cudaError_t set_smem(K kernel, size_t bytes) {
@@ -994,10 +993,7 @@ inline cudaError_t set_smem(K kernel, size_t bytes) {
 template <typename R, int M1, int M2>
 struct Passes {
   static constexpr int M = M1 * M2, T = kT<R>, NT = T * kQ<M1, M2>;
-  // rows per block of the x passes: 4 for the complex64 lines of 1000 points
-  // and more (four blocks of 4.5 warps per SM; 16 rows of 1080 points would
-  // take 147 KB, one block per SM)
-  static constexpr int TX = kTX<R, M>, NTX = TX * kQ<M1, M2>;
+  static constexpr int TX = fast_x_rows(sizeof(R) == 4, M), NTX = TX * kQ<M1, M2>;
   // columns per block of the fused z pass: the three spectra of TZ columns
   // must fit in shared memory (two blocks per SM where they can)
   static constexpr int TZ = (size_t)(M + 3 * M * T) * sizeof(cpx<R>) <= 113 * 1024 ? T

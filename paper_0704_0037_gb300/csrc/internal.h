@@ -328,9 +328,15 @@ struct FastArgs {
 inline bool fast_pdl(bool fp64, long long Mx, long long My, long long Mz, int nrhs) {
   return !fp64 && Mx * My * Mz * nrhs <= (1LL << 23);
 }
-// rows per block of the x passes: 16 for complex64 lines shorter than 1000
-// points, 4 for the longer ones, 8 for the double-width arithmetic
-inline int fast_x_rows(bool fp32, int Mx) { return fp32 ? (Mx < 1000 ? 16 : 4) : 8; }
+// rows per block of the x passes: 8 for the double-width arithmetic; for
+// complex64 16, 8 where a block of 16 would have more than 288 threads (one or
+// two blocks per SM, idle between their barriers; 256^3 sphere, 512 points: P1
+// 425 -> 315 us, P5 501 -> 380), 4 from 1000 points on
+constexpr int fast_x_rows(bool fp32, int Mx) {
+  if (!fp32) return 8;
+  if (Mx >= 1000) return 4;
+  return Mx >= 290 || Mx == 147 || Mx == 175 || Mx == 189 ? 8 : 16;
+}
 // number of (re, im) partials FP_XINV writes to dotp for nrows rows
 inline int fast_xinv_blocks(int nrows, bool fp32, int Mx) {
   const int t = fast_x_rows(fp32, Mx);
