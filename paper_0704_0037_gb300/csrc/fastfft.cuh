@@ -591,6 +591,167 @@ __device__ __forceinline__ void zc_inverse_b(const cpx<R>* sc, cpx<R>* __restric
   }
 }
 
+// ---- complex64, second phase of up to 8 points: product in registers
+// A thread of the second phase holds its row's M2 values of all three
+// components (6 M2 registers), so the product needs no trip through shared
+// memory (the pass above keeps the shared-memory pipe 80 % busy) and two
+// barriers less.  For each octant entry to be read once, the rows k1 and
+// M1 - k1 run in adjacent halves (or quarters) of a warp, and a row k1 > M1 / 2
+// stands for the frequencies -(m + M1 k2), m = M1 - k1: its twiddles are the
+// conjugates of row m's (one table load for both) and its elements j are kept
+// at (M2 - j) mod M2, so that the same forward codelet gives X(-(m + M1 k2)) at
+// index k2.  Both rows then need the octant at the same fz in the same
+// instruction, with the components odd in z negated in one of them.
+//
+// Above -> this, us (16 right-hand sides where two): 32 points 4.6 -> 4.3 and
+// 40.9 -> 30.2, 48 points 7.1 -> 6.1 and 55.3 -> 42.9, 64 points 8.7 -> 8.2 and
+// 93.5 -> 77.5, 96 points 14.4 -> 11.9 and 155 -> 129, 128 points 26.7 -> 24.0,
+// 147 and 175 points (two right-hand sides) 91.5 -> 72.9 and 106 -> 101.  A
+// second phase of 12 to 16 points takes 128 registers and the gain is lost to
+// the fewer warps: 144 points 93 -> 99, 270 points 246 -> 245 to 254, 512
+// points 1,716 -> 1,712 to 1,830.
+template <int M2> constexpr bool kZReg(int rsize) { return rsize == 4 && M2 <= 8; }
+// row of slot q: 1, M1 - 1, 2, M1 - 2, ..., 0
+template <int M1> __device__ __forceinline__ int zr_row(int q) {
+  if (q == M1 - 1) return 0;
+  const int i = q / 2 + 1;
+  return (q & 1) ? M1 - i : i;
+}
+// Shared-memory rows of a component: row k1's elements from at(k1).  With T = 8
+// a half warp reads the rows k1 and M1 - k1 at once: an odd number of rows
+// apart they fill the 32 banks.
+template <int M1, int M2, int T>
+struct ZRegRows {
+  static constexpr bool pad = T < 16;
+  static constexpr int pitch = pad ? (M2 + 1) / 2 * 2 : M2, rows = M1 * pitch + (pad ? 1 : 0);
+  static __device__ __forceinline__ int at(int k1) { return k1 * pitch + (pad && 2 * k1 > M1 ? 1 : 0); }
+};
+// blocks per SM: as the registers of the held spectra (and of one octant
+// entry, indices and the codelet's temporaries) allow
+constexpr int kZRegB(int nt, int m2, long long smem_bytes) {
+  const int regs = 6 * m2 + 48, w = (nt + 31) / 32 * 32;
+  const int b = 65536 / (w * regs), by_smem = (int)((227LL * 1024) / smem_bytes);
+  const int r = b < by_smem ? b : by_smem;
+  return r >= 1 ? r : 1;
+}
+
+template <int M1, int M2, int T>
+__global__ void __launch_bounds__(T * kQ<M1, M2>,
+                                  kZRegB(T * kQ<M1, M2>, M2, (kTwLen<M1 * M2> + 3LL * ZRegRows<M1, M2, T>::rows * T) * sizeof(c64)))
+    fk_zconv_reg(c64* __restrict__ B2, const c64* __restrict__ D, int nz, int Mx, int My,
+                 const c64* __restrict__ tw, const int* __restrict__ skip) {
+  using Z = ZRegRows<M1, M2, T>;
+  constexpr int M = M1 * M2, NT = T * kQ<M1, M2>, CS = Z::rows * T, kZin = kHalf<M1, M2>;
+  B2 += (long long)blockIdx.z * 3 * nz * My * Mx;      // right-hand side blockIdx.z
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  c64* s_tw = reinterpret_cast<c64*>(smem_raw);
+  c64* s = s_tw + kTwLen<M>;                 // [3][rows][T]
+  load_tw(s_tw, tw, M, NT);
+  pdl_wait();
+  pdl_launch();
+  if (skip && skip[blockIdx.z]) return;
+  const int bx = blockIdx.x, ky = ky_order(blockIdx.y, My);
+  const int t = threadIdx.x % T, q = threadIdx.x / T;
+  const int kx = bx * T + t;
+  const long long plane = (long long)My * Mx;
+  for (int c = 0; c < 3; ++c) zc_stage<float, T, NT>(s + c * CS, B2, c, nz, Mx, My, bx, ky);
+  zc_prefetch<float, M, T, NT>(D, Mx, My, bx, ky);
+  // phase 1 of column j, and where its elements of the rows k1 > M1 / 2 are
+  const int j = q, jr = j ? M2 - j : 0;
+  c64* sj = s + j * T + t;
+  c64* sr = s + jr * T + t;
+  cp_async_wait<0>();
+  __syncthreads();             // the tile (and the twiddles) complete
+  c64 w3[3][kZin];
+  if (q < M2) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int i = 0; i < kZin; ++i) w3[c][i] = j + M2 * i < nz ? sj[c * CS + M2 * i * T] : zero<float>();
+  }
+  __syncthreads();             // every read of the tile before the regions are rewritten
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    c64 v[M1];
+#pragma unroll
+    for (int i = 0; i < M1; ++i) v[i] = i < kZin ? w3[c][i < kZin ? i : 0] : zero<float>();
+    if (q < M2) {
+      dft_padded<float, M1, kZin>(v);
+#pragma unroll
+      for (int k1 = 1; 2 * k1 <= M1; ++k1) {
+        const c64 w = s_tw[j * k1];
+        v[k1] = twiddle<float, false>(v[k1], w);
+        if (2 * k1 < M1) v[M1 - k1] = twiddle<float, true>(v[M1 - k1], w);
+      }
+#pragma unroll
+      for (int k1 = 0; k1 < M1; ++k1) (2 * k1 <= M1 ? sj : sr)[c * CS + Z::at(k1) * T] = v[k1];
+    }
+  }
+  __syncthreads();
+  if (q < M1 && kx < Mx) {
+    const int k1 = zr_row<M1>(q), m = 2 * k1 <= M1 ? k1 : M1 - k1;
+    c64* sc = s + Z::at(k1) * T + t;
+    c64 u[3][M2];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+#pragma unroll
+      for (int r = 0; r < M2; ++r) u[c][r] = sc[c * CS + r * T];
+      cl::Dft<float, false, M2>::run(u[c]);
+    }
+    // octant entry of kz = +-(m + M1 k2), folded at M / 2
+    const int hx = Mx / 2 + 1, hy = My / 2 + 1;
+    int nxs, nys;
+    const int fy = fold_axis(ky, My, nys), fx = fold_axis(kx, Mx, nxs);
+    const float sx = nxs ? -1.0f : 1.0f, sy = nys ? -1.0f : 1.0f, sz = m == k1 ? 1.0f : -1.0f;
+    const float sxy = sx * sy, sxz = sx * sz, syz = sy * sz;
+    const long long zs = 6LL * hy * hx;
+    const c64* Dl = D + 6 * ((long long)fy * hx + fx) + m * zs;      // kz = m
+    const c64* Dh = D + 6 * ((long long)fy * hx + fx) + (M - m) * zs;
+#pragma unroll
+    for (int k2 = 0; k2 < M2; ++k2) {
+      const bool high = 2 * k2 >= M2;
+      const float4* dp = reinterpret_cast<const float4*>(high ? Dh - M1 * k2 * zs : Dl + M1 * k2 * zs);
+      const float4 a = dp[0], b = dp[1], d = dp[2];
+      const c64 dxx = mk<float>(a.x, a.y), dyy = mk<float>(b.z, b.w), dzz = mk<float>(d.z, d.w);
+      const c64 dxy = scale<float>(mk<float>(a.z, a.w), sxy);
+      const c64 dxz = scale<float>(mk<float>(b.x, b.y), high ? -sxz : sxz);
+      const c64 dyz = scale<float>(mk<float>(d.x, d.y), high ? -syz : syz);
+      const c64 vx = u[0][k2], vy = u[1][k2], vz = u[2][k2];
+      u[0][k2] = cmac(cmac(dxx * vx, dxy, vy), dxz, vz);
+      u[1][k2] = cmac(cmac(dxy * vx, dyy, vy), dyz, vz);
+      u[2][k2] = cmac(cmac(dxz * vx, dyz, vy), dzz, vz);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      cl::Dft<float, true, M2>::run(u[c]);
+#pragma unroll
+      for (int r = 0; r < M2; ++r) sc[c * CS + r * T] = u[c][r];
+    }
+  }
+  __syncthreads();
+  if (q < M2 && kx < Mx) {
+    c64* out = B2 + (long long)ky * Mx + kx;
+#pragma unroll 1
+    for (int c = 0; c < 3; ++c, out += nz * plane) {
+      c64 v[M1];
+#pragma unroll
+      for (int k1 = 0; k1 < M1; ++k1) v[k1] = (2 * k1 <= M1 ? sj : sr)[c * CS + Z::at(k1) * T];
+#pragma unroll
+      for (int k1 = 1; 2 * k1 <= M1; ++k1) {
+        const c64 w = s_tw[j * k1];
+        v[k1] = twiddle<float, true>(v[k1], w);
+        if (2 * k1 < M1) v[M1 - k1] = twiddle<float, false>(v[M1 - k1], w);
+      }
+      cl::Dft<float, true, M1>::run(v);
+#pragma unroll
+      for (int i = 0; i < M1; ++i) {
+        const int z = j + M2 * i;
+        if (i < kZin && z < nz) out[z * plane] = v[i];
+      }
+    }
+  }
+}
+
 template <typename R, int M1, int M2, int T>
 __global__ void __launch_bounds__(T * kQ<M1, M2>,
                                   kMinB(T * kQ<M1, M2>, 2, (kTwLen<M1 * M2> + 3LL * ZRows<R, M1, M2, T>::rows * T) * sizeof(cpx<R>)))
@@ -1041,14 +1202,24 @@ struct Passes {
   template <int TC>
   static cudaError_t zconv_t(cpx<R>* B2, const cpx<R>* D, int nz, int Mx, int My, const cpx<R>* tw,
                              int nrhs, const int* skip, cudaStream_t st, bool pdl) {
-    const size_t sm = (size_t)(kTwLen<M> + 3 * ZRows<R, M1, M2, TC>::rows * TC) * sizeof(cpx<R>);
-    cudaError_t e = set_smem(fk_zconv<R, M1, M2, TC>, sm);
+    // the split with the shorter second phase, where its spectra are held in
+    // registers
+    constexpr int ML = M1 > M2 ? M1 : M2, MS = M1 > M2 ? M2 : M1;
+    constexpr bool reg = kZReg<MS>(sizeof(R));
+    constexpr int N1 = reg ? ML : M1, N2 = reg ? MS : M2;
+    auto* kernel = [] {
+      if constexpr (reg) return fk_zconv_reg<N1, N2, TC>;
+      else return fk_zconv<R, N1, N2, TC>;
+    }();
+    using Z = std::conditional_t<reg, ZRegRows<N1, N2, TC>, ZRows<R, N1, N2, TC>>;
+    const size_t sm = (size_t)(kTwLen<M> + 3 * Z::rows * TC) * sizeof(cpx<R>);
+    cudaError_t e = set_smem(kernel, sm);
     if (e != cudaSuccess) return e;
     // two ~106 KB blocks per SM need the largest shared-memory carveout
-    e = ensure_carveout_max((const void*)fk_zconv<R, M1, M2, TC>);
+    e = ensure_carveout_max((const void*)kernel);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(pdl, fk_zconv<R, M1, M2, TC>, dim3((Mx + TC - 1) / TC, My, nrhs), dim3(TC * kQ<M1, M2>),
-                   sm, st, B2, D, nz, Mx, My, tw, skip);
+    e = launch_pdl(pdl, kernel, dim3((Mx + TC - 1) / TC, My, nrhs), dim3(TC * kQ<M1, M2>), sm, st, B2, D, nz, Mx,
+                   My, tw, skip);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
   }
