@@ -498,9 +498,39 @@ __device__ __forceinline__ void zc_forward_product_inva(cpx<R>* s, const cpx<R>*
                                                        const cpx<R>* __restrict__ D, int nz, int Mx,
                                                        int My, int bx, int ky) {
   using Z = ZRows<R, M1, M2, T>;
-  constexpr int M = M1 * M2, CS = Z::rows * T, kZin = kHalf<M1, M2>;
+  constexpr int CS = Z::rows * T, kZin = kHalf<M1, M2>;
   const int t = threadIdx.x % T, q = threadIdx.x / T;
   const int kx = bx * T + t;
+  const int j = q;
+  if constexpr (sizeof(R) == 4) {
+    // all three tiles read before any region is rewritten: two barriers
+    cp_async_wait<0>();
+    __syncthreads();           // the tiles (and the twiddles) complete
+    cpx<R> w[3][kZin];
+    if (q < M2) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int i = 0; i < kZin; ++i) {
+          const int z = j + M2 * i;
+          w[c][i] = z < nz ? s[c * CS + z * T + t] : zero<R>();
+        }
+    }
+    __syncthreads();
+    if (q < M2) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        cpx<R> v[M1];
+#pragma unroll
+        for (int i = 0; i < M1; ++i) v[i] = i < kZin ? w[c][i < kZin ? i : 0] : zero<R>();
+        dft_padded<R, M1, kZin>(v);
+#pragma unroll
+        for (int k1 = 1; k1 < M1; ++k1) v[k1] = twiddle<R, false>(v[k1], s_tw[j * k1]);
+#pragma unroll
+        for (int k1 = 0; k1 < M1; ++k1) s[c * CS + Z::at(k1, j) * T + t] = v[k1];
+      }
+    }
+  } else {
 #pragma unroll 1
   for (int c = 0; c < 3; ++c) {
     if (c == 0) cp_async_wait<2>();
@@ -508,7 +538,6 @@ __device__ __forceinline__ void zc_forward_product_inva(cpx<R>* s, const cpx<R>*
     else cp_async_wait<0>();
     __syncthreads();           // this component's tile (and the twiddles) complete
     cpx<R>* sc = s + c * CS;
-    const int j = q;
     cpx<R> v[M1];
     if (q < M2) {
 #pragma unroll
@@ -525,6 +554,7 @@ __device__ __forceinline__ void zc_forward_product_inva(cpx<R>* s, const cpx<R>*
 #pragma unroll
       for (int k1 = 0; k1 < M1; ++k1) sc[Z::at(k1, j) * T + t] = v[k1];
     }
+  }
   }
   __syncthreads();
   if constexpr (kZOneM2<R>) {
@@ -606,7 +636,7 @@ __device__ __forceinline__ void zc_inverse_b(const cpx<R>* sc, cpx<R>* __restric
 // Above -> this, us (16 right-hand sides where two): 32 points 4.6 -> 4.3 and
 // 40.9 -> 30.2, 48 points 7.1 -> 6.1 and 55.3 -> 42.9, 64 points 8.7 -> 8.2 and
 // 93.5 -> 77.5, 96 points 14.4 -> 11.9 and 155 -> 129, 128 points 26.7 -> 24.0,
-// 147 and 175 points (two right-hand sides) 91.5 -> 72.9 and 106 -> 101.  A
+// 147 and 175 points (two right-hand sides) 91.5 -> 67.0 and 106 -> 104.  A
 // second phase of 12 to 16 points takes 128 registers and the gain is lost to
 // the fewer warps: 144 points 93 -> 99, 270 points 246 -> 245 to 254, 512
 // points 1,716 -> 1,712 to 1,830.
@@ -626,10 +656,11 @@ struct ZRegRows {
   static constexpr int pitch = pad ? (M2 + 1) / 2 * 2 : M2, rows = M1 * pitch + (pad ? 1 : 0);
   static __device__ __forceinline__ int at(int k1) { return k1 * pitch + (pad && 2 * k1 > M1 ? 1 : 0); }
 };
-// blocks per SM: as the registers of the held spectra (and of one octant
-// entry, indices and the codelet's temporaries) allow
-constexpr int kZRegB(int nt, int m2, long long smem_bytes) {
-  const int regs = 6 * m2 + 48, w = (nt + 31) / 32 * 32;
+// blocks per SM: as the registers of the held spectra, or of the first phase's
+// inputs (zin of each component), and of one octant entry, indices and the
+// codelet's temporaries allow
+constexpr int kZRegB(int nt, int zin, int m2, long long smem_bytes) {
+  const int regs = (6 * m2 > 4 * zin ? 6 * m2 : 4 * zin) + 48, w = (nt + 31) / 32 * 32;
   const int b = 65536 / (w * regs), by_smem = (int)((227LL * 1024) / smem_bytes);
   const int r = b < by_smem ? b : by_smem;
   return r >= 1 ? r : 1;
@@ -637,7 +668,7 @@ constexpr int kZRegB(int nt, int m2, long long smem_bytes) {
 
 template <int M1, int M2, int T>
 __global__ void __launch_bounds__(T * kQ<M1, M2>,
-                                  kZRegB(T * kQ<M1, M2>, M2, (kTwLen<M1 * M2> + 3LL * ZRegRows<M1, M2, T>::rows * T) * sizeof(c64)))
+                                  kZRegB(T * kQ<M1, M2>, kHalf<M1, M2>, M2, (kTwLen<M1 * M2> + 3LL * ZRegRows<M1, M2, T>::rows * T) * sizeof(c64)))
     fk_zconv_reg(c64* __restrict__ B2, const c64* __restrict__ D, int nz, int Mx, int My,
                  const c64* __restrict__ tw, const int* __restrict__ skip) {
   using Z = ZRegRows<M1, M2, T>;
@@ -752,9 +783,15 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>,
   }
 }
 
+// blocks per SM the z pass asks for: two; in complex64, whose blocks hold the
+// inputs of all three components in registers, as many as make 640 threads.
+// 512 points 1,716 -> 1,658 us, 336 92 -> 81, 315 88 -> 79, others 1 to 3 % (with
+// two barriers instead of six before the second phase)
+template <typename R> constexpr int kZBlocks(int nt) { return sizeof(R) == 4 && nt <= 320 ? 640 / nt : 2; }
+
 template <typename R, int M1, int M2, int T>
 __global__ void __launch_bounds__(T * kQ<M1, M2>,
-                                  kMinB(T * kQ<M1, M2>, 2, (kTwLen<M1 * M2> + 3LL * ZRows<R, M1, M2, T>::rows * T) * sizeof(cpx<R>)))
+                                  kMinB(T * kQ<M1, M2>, kZBlocks<R>(T * kQ<M1, M2>), (kTwLen<M1 * M2> + 3LL * ZRows<R, M1, M2, T>::rows * T) * sizeof(cpx<R>)))
     fk_zconv(cpx<R>* __restrict__ B2, const cpx<R>* __restrict__ D, int nz, int Mx, int My,
              const cpx<R>* __restrict__ tw, const int* __restrict__ skip) {
   constexpr int M = M1 * M2, NT = T * kQ<M1, M2>, CS = ZRows<R, M1, M2, T>::rows * T;
@@ -1156,8 +1193,10 @@ struct Passes {
   static constexpr int M = M1 * M2, T = kT<R>, NT = T * kQ<M1, M2>;
   static constexpr int TX = fast_x_rows(sizeof(R) == 4, M), NTX = TX * kQ<M1, M2>;
   // columns per block of the fused z pass: the three spectra of TZ columns
-  // must fit in shared memory (two blocks per SM where they can)
-  static constexpr int TZ = (size_t)(M + 3 * M * T) * sizeof(cpx<R>) <= 113 * 1024 ? T
+  // must fit in shared memory (two blocks per SM where they can); half as many
+  // in complex64 where a block would have more than 288 threads (one per SM:
+  // 189 points 121 -> 101 us, 280 80 -> 64, 147 73 -> 67)
+  static constexpr int TZ = (size_t)(M + 3 * M * T) * sizeof(cpx<R>) <= 113 * 1024 && (sizeof(R) > 4 || NT <= 288) ? T
                            : (size_t)(M + 3 * M * (T / 2)) * sizeof(cpx<R>) <= 226 * 1024 ? T / 2
                            : T / 4;
   // Tile variants (lines per block) of the y passes and the z pass: 0 the
