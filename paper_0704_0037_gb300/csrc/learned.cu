@@ -102,6 +102,41 @@ __global__ void k_pool2(const float* __restrict__ in, Dims di, float* __restrict
     out[i] = s / (float)cnt;
   }
 }
+// k_pool2 over split units, a thread per voxel and 8 channels
+__global__ void __launch_bounds__(128) k_pool2_split(const uint4* __restrict__ in, Dims di, uint4* __restrict__ out,
+                                                     Dims dout, int ch) {
+  const long long nin = di.n(), no = dout.n(), n = no * (ch / 8);
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    const int c = (int)(i / no);
+    const long long p = i - c * no;
+    const int X = (int)(p % dout.x), Y = (int)((p / dout.x) % dout.y), Z = (int)(p / ((long long)dout.x * dout.y));
+    float s[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    int cnt = 0;
+    for (int dz = 0; dz < 2; ++dz)
+      for (int dy = 0; dy < 2; ++dy)
+        for (int dx = 0; dx < 2; ++dx) {
+          const int x = 2 * X + dx, y = 2 * Y + dy, z = 2 * Z + dz;
+          if (x < di.x && y < di.y && z < di.z) {
+            const long long v = ((long long)z * di.y + y) * di.x + x;
+            uint4 u[3];
+            float f[8];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) u[k] = in[(3LL * c + k) * nin + v];
+            join_unit(u, f);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) s[k] += f[k];
+            ++cnt;
+          }
+        }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s[k] /= (float)cnt;
+    uint4 u[3];
+    split_unit(s, u);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) out[(3LL * c + k) * no + p] = u[k];
+  }
+}
 // gin[c][v] += gout[c][parent(v)] / children(parent), then zero where the
 // activation act[c][v] <= 0 (gradient behind its relu)
 __global__ void k_pool2_back(const float* __restrict__ gout, Dims dout, float* __restrict__ gin,
@@ -370,6 +405,7 @@ struct Acts {
   Dims d0, d1, d2;
   float *f0, *a0, *a5, *o6, *p1, *a1, *a4, *p2, *a2, *a3;
   float *g6, *ga5, *gcat0, *gcat1, *ga4, *ga3, *ga2, *gp2, *gp1;
+  void* arena_split;                           // split activations of a pass without gradient
 };
 
 size_t acts_floats(Dims d0, Dims d1, Dims d2) {
@@ -396,9 +432,10 @@ int ensure_arena(dda_pcnet_t net, dda_t h, Acts& A) {
   float* p = (float*)net->arena;
   auto take = [&](long long n) { float* r = p; p += n; return r; };
   A.f0 = take(7 * A.d0.n());
+  A.o6 = take(6 * A.d0.n());
+  A.arena_split = (void*)(((size_t)p + 15) & ~(size_t)15);
   A.a0 = take(16 * A.d0.n());
   A.a5 = take(16 * A.d0.n());
-  A.o6 = take(6 * A.d0.n());
   A.g6 = take(6 * A.d0.n());
   A.ga5 = take(16 * A.d0.n());
   A.gcat0 = take(48 * A.d0.n());
@@ -453,14 +490,43 @@ ConvIn layer_input(const Acts& A, int L) {
   }
 }
 
-cudaError_t conv_fwd(dda_pcnet_t net, int L, const Acts& A, float* out, Dims d, bool train, cudaStream_t st) {
+cudaError_t conv_fwd(dda_pcnet_t net, int L, const Acts& A, float* out, Dims d, cudaStream_t st) {
   const LayerSpec& s = kSpec[L];
-  const float* bias = net->w + net->boff[L];
-  if (train)
-    return conv_f32(s.k, layer_input(A, L), net->wf + net->packf.item[L].at, bias, nullptr, out, s.cout, d,
-                    s.relu, st);
-  return conv_mma(s.k, layer_input(A, L), net->wp + net->pack.item[L].at, bias, nullptr, out, s.cout, d,
-                  s.relu, st);
+  return conv_f32(s.k, layer_input(A, L), net->wf + net->packf.item[L].at, net->w + net->boff[L], nullptr, out,
+                  s.cout, d, s.relu, st);
+}
+
+// The seven layers of a pass that keeps nothing for a gradient: features A.f0
+// to A.o6, activations split (244 bytes per voxel of d0, 480 of d1, 2,112 of
+// d2, in the arena of a training pass's 460, 1,280 and 2,816)
+cudaError_t layers_split(dda_pcnet_t net, const Acts& A, cudaStream_t st) {
+  const long long n0 = A.d0.n(), n1 = A.d1.n(), n2 = A.d2.n();
+  uint4* p = (uint4*)(A.arena_split);
+  auto take = [&](int ch, long long n) { uint4* r = p; p += (long long)ch / 8 * 3 * n; return r; };
+  uint4 *a0 = take(16, n0), *a5 = take(16, n0), *p1 = take(16, n1), *a1 = take(32, n1), *a4 = take(32, n1),
+        *p2 = take(32, n2), *a2 = take(160, n2), *a3 = take(160, n2);
+  const Dims no{0, 0, 0};
+  cudaError_t e = cudaSuccess;
+  auto conv = [&](int L, const SplitIn& in, const SplitOut& out, Dims d) {
+    const LayerSpec& s = kSpec[L];
+    if (e == cudaSuccess)
+      e = conv_mma(s.k, in, net->wp + net->pack.item[L].at, net->w + net->boff[L], out, s.cout, d, s.relu, st);
+  };
+  auto pool = [&](const uint4* in, Dims di, uint4* out, Dims dout, int ch) {
+    const long long n = dout.n() * (ch / 8);
+    k_pool2_split<<<(unsigned)std::min<long long>((n + 127) / 128, 1 << 20), 128, 0, st>>>(in, di, out, dout, ch);
+    count_launch();
+  };
+  conv(0, {nullptr, 0, no, false, nullptr, 0, A.f0, 7}, {a0, nullptr}, A.d0);
+  pool(a0, A.d0, p1, A.d1, 16);
+  conv(1, {p1, 16, no, false, nullptr, 0, nullptr, 0}, {a1, nullptr}, A.d1);
+  pool(a1, A.d1, p2, A.d2, 32);
+  conv(2, {p2, 32, no, false, nullptr, 0, nullptr, 0}, {a2, nullptr}, A.d2);
+  conv(3, {a2, 160, no, false, nullptr, 0, nullptr, 0}, {a3, nullptr}, A.d2);
+  conv(4, {a3, 160, A.d2, true, a1, 32, nullptr, 0}, {a4, nullptr}, A.d1);
+  conv(5, {a4, 32, A.d1, true, a0, 16, nullptr, 0}, {a5, nullptr}, A.d0);
+  conv(6, {a5, 16, no, false, nullptr, 0, nullptr, 0}, {nullptr, A.o6}, A.d0);
+  return e;
 }
 
 // input gradient of layer L: gin = conv(gout, wT) (no bias), zero where the
@@ -530,15 +596,20 @@ int forward(dda_pcnet_t net, dda_t h, const c128* v, c128* z, Acts& A, bool trai
   count_launch();
   k_feat_in<<<dim3(gs(A.d0.n()), 3), 256, 0, st>>>(v, h->g.n_occ, net->map, dl, A.d0, net->scal, A.f0);
   count_launch();
-  cudaError_t e = conv_fwd(net, 0, A, A.a0, A.d0, train, st);
-  k_pool2<<<gs(16 * A.d1.n()), 256, 0, st>>>(A.a0, A.d0, A.p1, A.d1, 16); count_launch();
-  if (e == cudaSuccess) e = conv_fwd(net, 1, A, A.a1, A.d1, train, st);
-  k_pool2<<<gs(32 * A.d2.n()), 256, 0, st>>>(A.a1, A.d1, A.p2, A.d2, 32); count_launch();
-  if (e == cudaSuccess) e = conv_fwd(net, 2, A, A.a2, A.d2, train, st);
-  if (e == cudaSuccess) e = conv_fwd(net, 3, A, A.a3, A.d2, train, st);
-  if (e == cudaSuccess) e = conv_fwd(net, 4, A, A.a4, A.d1, train, st);
-  if (e == cudaSuccess) e = conv_fwd(net, 5, A, A.a5, A.d0, train, st);
-  if (e == cudaSuccess) e = conv_fwd(net, 6, A, A.o6, A.d0, train, st);
+  cudaError_t e;
+  if (!train) {
+    e = layers_split(net, A, st);
+  } else {
+    e = conv_fwd(net, 0, A, A.a0, A.d0, st);
+    k_pool2<<<gs(16 * A.d1.n()), 256, 0, st>>>(A.a0, A.d0, A.p1, A.d1, 16); count_launch();
+    if (e == cudaSuccess) e = conv_fwd(net, 1, A, A.a1, A.d1, st);
+    k_pool2<<<gs(32 * A.d2.n()), 256, 0, st>>>(A.a1, A.d1, A.p2, A.d2, 32); count_launch();
+    if (e == cudaSuccess) e = conv_fwd(net, 2, A, A.a2, A.d2, st);
+    if (e == cudaSuccess) e = conv_fwd(net, 3, A, A.a3, A.d2, st);
+    if (e == cudaSuccess) e = conv_fwd(net, 4, A, A.a4, A.d1, st);
+    if (e == cudaSuccess) e = conv_fwd(net, 5, A, A.a5, A.d0, st);
+    if (e == cudaSuccess) e = conv_fwd(net, 6, A, A.o6, A.d0, st);
+  }
   k_feat_out<<<std::min(4096, (h->g.nrows + 7) / 8), 256, 0, st>>>(A.o6, A.d0, h->lat(), h->g.nx, h->g.ny,
                                                                   h->g.nrows, h->g.n_occ, net->scal, v, z);
   count_launch();

@@ -10,23 +10,32 @@
 // products, 256 times smaller, accumulate over the 9 taps of a z plane.
 //
 // The convolution is an implicit matrix product: rows are voxels, columns
-// output channels, the inner dimension is 16 input channels of one tap.  A
-// block stages 16 channels of its voxel tile and halo (FP32 by asynchronous
-// copies, then split) as 16-byte units of 8 channels, [split][half][voxel], so
-// that the rows of a tap are ldmatrix rows at a shifted voxel and eight
-// neighbours in x fill the 32 banks.  The next channels arrive while these are
-// multiplied, the weights, in fragment order (packed when they change), while
-// the channels are split.  Each warp holds MT tiles of 16 voxels (two x rows
-// of 8) by NT tiles of 8 channels.
+// output channels, the inner dimension is 16 input channels of one tap.
+// Activations live in global memory already split, as 16-byte units of 8
+// channels, [8-channel block][part][voxel]: the kernel that produces a value
+// splits it once instead of every tile that reads it (with halos and output
+// blocks about six), and a tile with its halo arrives by 16-byte asynchronous
+// copies in the layout it is used from, [part][half][voxel], where the rows of
+// a tap are ldmatrix rows at a shifted voxel and eight neighbours in x fill
+// the 32 banks.  The weights come in fragment order (packed when they change).
+// Each warp holds MT tiles of 16 voxels (two x rows of 8) by NT tiles of 8
+// channels; several blocks share an SM, so that copies of one run under the
+// matrix instructions of another.  Where the layer has too few tiles for that
+// (1/8 resolution), KG groups of 4 warps in a block take every KG-th 16
+// channels each and their sums are added at the end.
 //
-// 128^3 sphere (31 GFLOP a pass): 2.09 ms of convolutions on the FP32 pipe
-// before, 0.39 ms now (48 to 16 channels at 64^3 voxels 435 -> 130 us); the
-// pass 2.36 -> 0.50 ms; error of N(r) against 64 bits 4.5e-7 before, 1.6e-7 now.
+// 128^3 sphere (31 GFLOP a pass, 93 with the three products): 2.09 ms of
+// convolutions on the FP32 pipe; on the tensor cores 0.38 ms when every tile
+// split the FP32 channels it read, 0.33 ms now (48 to 16 channels at 64^3 voxels
+// 435, 121 and 96 us, 160 to 160 at 16^3 69 and 53 us between the last two);
+// the matrix pipe is 60 to 66 % busy in the large layers.  The pass 2.36, 0.50
+// and 0.45 ms; error of N(r) against 64 bits 4.5e-7 before, 1.4e-7 now.
 #pragma once
 
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "internal.h"
 
@@ -56,6 +65,11 @@ __device__ __forceinline__ void cp4(void* smem, const float* gmem, bool ok) {
   const int n = ok ? 4 : 0;
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(sa), "l"(gmem), "r"(n) : "memory");
 }
+__device__ __forceinline__ void cp16(void* smem, const void* gmem, bool ok) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  const int n = ok ? 16 : 0;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "r"(n) : "memory");
+}
 __device__ __forceinline__ void ldm4(unsigned (&r)[4], const void* smem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
@@ -74,19 +88,54 @@ __device__ __forceinline__ void split3(float x, __nv_bfloat16 (&s)[3]) {
   s[1] = __float2bfloat16_rn(r);
   s[2] = __float2bfloat16_rn(r - __bfloat162float(s[1]));
 }
-// 8 floats p[0], p[stride], ... as three units of 8 bf16
-__device__ __forceinline__ void split_unit(const float* p, int stride, uint4 (&u)[3]) {
+// 8 floats as three units of 8 bf16, and back (exact)
+__device__ __forceinline__ void split_unit(const float (&f)[8], uint4 (&u)[3]) {
   __nv_bfloat16 s[3][8];
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
     __nv_bfloat16 t[3];
-    split3(p[c * stride], t);
+    split3(f[c], t);
 #pragma unroll
     for (int k = 0; k < 3; ++k) s[k][c] = t[k];
   }
 #pragma unroll
   for (int k = 0; k < 3; ++k) u[k] = *reinterpret_cast<const uint4*>(s[k]);
 }
+__device__ __forceinline__ void join_unit(const uint4 (&u)[3], float (&f)[8]) {
+  const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&u[0]);
+  const __nv_bfloat16* m = reinterpret_cast<const __nv_bfloat16*>(&u[1]);
+  const __nv_bfloat16* l = reinterpret_cast<const __nv_bfloat16*>(&u[2]);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) f[c] = (__bfloat162float(h[c]) + __bfloat162float(m[c])) + __bfloat162float(l[c]);
+}
+// 2 floats as three pairs of bf16
+__device__ __forceinline__ void split_pair(float a, float b, unsigned (&u)[3]) {
+  __nv_bfloat16 s[3], t[3];
+  split3(a, s);
+  split3(b, t);
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    u[k] = (unsigned)__bfloat16_as_ushort(s[k]) | (unsigned)__bfloat16_as_ushort(t[k]) << 16;
+}
+
+// Input of a convolution of the apply pass: split units as ConvIn's arrays (ca
+// and cb multiples of 16), or, for the first layer, FP32 channels f (at most
+// 16, split as they are staged).
+struct SplitIn {
+  const uint4* a;
+  int ca;
+  Dims da;
+  bool up;
+  const uint4* b;
+  int cb;
+  const float* f;
+  int cf;
+};
+// Output: split units, or FP32 channels (the last layer)
+struct SplitOut {
+  uint4* s;
+  float* f;
+};
 
 // Voxel tile of 8 x 4 x TZ and its halo for kernels of K^3 taps
 template <int K, int TZ> struct Tile {
@@ -94,66 +143,41 @@ template <int K, int TZ> struct Tile {
 };
 
 // out[co][v] = bias[co] + sum_ci sum_t w[co][ci][t] in[ci][v + t - H], then
-// relu, or zero where mask[co][v] <= 0 (gradient behind a relu).  wp: packed
-// weights [16-channel block][tap][8-channel tile][lane]; grid (voxel tiles,
-// output-channel blocks of 8 NT); 4 warps.
-template <int K, int MT, int NT>
-__global__ void __launch_bounds__(128) k_conv_mma(ConvIn in, const uint2* __restrict__ wp, int ntn,
-                                                  const float* __restrict__ bias,
-                                                  const float* __restrict__ mask,
-                                                  float* __restrict__ out, int cout, Dims d, int relu) {
+// relu.  wp: packed weights [16-channel block][tap][8-channel tile][lane]; grid
+// (voxel tiles, output-channel blocks of 8 NT); 4 KG warps.  FIN: the input is
+// FP32 channels (one block of 16), else split units.
+template <int K, int MT, int NT, int KG, bool FIN>
+__global__ void __launch_bounds__(128 * KG) k_conv_mma(SplitIn in, const uint2* __restrict__ wp, int ntn,
+                                                       const float* __restrict__ bias, SplitOut out,
+                                                       int cout, Dims d, int relu) {
   constexpr int TZ = 2 * MT, K3 = K * K * K;
   using T = Tile<K, TZ>;
   constexpr int NV = (T::HV + 127) / 128;      // halo voxels per thread
+  constexpr int GB = 6 * T::HV * 16 + K3 * NT * 256;       // shared memory of a group
+  static_assert(MT * NT * 4 * 128 * 4 <= GB, "a group's sums fit its buffers");
   extern __shared__ __align__(16) unsigned char smem[];
-  uint4* s_t = reinterpret_cast<uint4*>(smem);                       // [3][2][HV]
-  float* s_f = reinterpret_cast<float*>(smem + (size_t)6 * T::HV * 16);   // [16][HV]
-  uint2* s_w = reinterpret_cast<uint2*>(s_f + 16 * T::HV);           // [K3][NT][32]
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tid = threadIdx.x & 127, grp = threadIdx.x >> 7, lane = threadIdx.x & 31, warp = tid >> 5;
+  uint4* s_t = reinterpret_cast<uint4*>(smem + grp * GB);                 // [3][2][HV]
+  uint2* s_w = reinterpret_cast<uint2*>(s_t + 6 * T::HV);                 // [K3][NT][32]
   const int ntx = (d.x + 7) / 8, nty = (d.y + 3) / 4;
   const int tx0 = (blockIdx.x % ntx) * 8, ty0 = ((blockIdx.x / ntx) % nty) * 4,
             tz0 = (blockIdx.x / (ntx * nty)) * TZ;
   const long long nv = d.n(), na = in.up ? in.da.n() : nv;
-  const int cin = in.ca + in.cb, nblk = (cin + 15) / 16;
+  const int nblk = FIN ? 1 : (in.ca + in.cb) / 16;
   // this thread's halo voxels: index in b (fine) and in a, -1 outside
   int vf[NV], va[NV];
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
-    const int hv = threadIdx.x + 128 * i;
+    const int hv = tid + 128 * i;
     const int x = tx0 + hv % T::HX - T::H, y = ty0 + (hv / T::HX) % T::HY - T::H,
               z = tz0 + hv / (T::HX * T::HY) - T::H;
     const bool ok = hv < T::HV && x >= 0 && y >= 0 && z >= 0 && x < d.x && y < d.y && z < d.z;
     vf[i] = ok ? (z * d.y + y) * d.x + x : -1;
     va[i] = !ok ? -1 : in.up ? ((z / 2) * in.da.y + y / 2) * in.da.x + x / 2 : vf[i];
   }
-  auto fetch = [&](int blk) {
-    const int c0 = blk * 16;
-    const bool fa = c0 < in.ca;
-    const float* src = fa ? in.a + (long long)c0 * na : in.b + (long long)(c0 - in.ca) * nv;
-    const long long cs = fa ? na : nv;
-    const int lim = (fa ? in.ca : cin) - c0;
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      const int hv = threadIdx.x + 128 * i, v = fa ? va[i] : vf[i];
-      if (hv < T::HV) {
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          const bool ok = v >= 0 && c < lim;
-          cp4(s_f + c * T::HV + hv, ok ? src + c * cs + v : in.a, ok);
-        }
-      }
-    }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-  };
-  auto fetch_w = [&](int blk) {
-    const uint2* sw = wp + ((long long)blk * K3 * ntn + blockIdx.y * NT) * 32;
-    for (int i = threadIdx.x; i < K3 * NT * 16; i += 128) {          // 16-byte pieces
-      const int t = i / (NT * 16), r = i - t * NT * 16;
-      const unsigned sa = (unsigned)__cvta_generic_to_shared(s_w + t * NT * 32 + 2 * r);
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(sw + (long long)t * ntn * 32 + 2 * r)
-                   : "memory");
-    }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  auto group_sync = [&] {
+    if constexpr (KG == 1) __syncthreads();
+    else asm volatile("bar.sync %0, 128;" ::"r"(grp + 1) : "memory");
   };
   float acc[MT][NT][4];
 #pragma unroll
@@ -169,31 +193,49 @@ __global__ void __launch_bounds__(128) k_conv_mma(ConvIn in, const uint2* __rest
     const int m = warp * MT + i;               // z = m / 2, rows y = 2 (m % 2) and + 1
     row[i] = ((m >> 1) * T::HY + 2 * (m & 1) + ((lane >> 3) & 1)) * T::HX + (lane & 7) + (lane >> 4) * T::HV;
   }
-  fetch(0);
-  for (int blk = 0; blk < nblk; ++blk) {
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    __syncthreads();                           // the previous channels' products are done
-    fetch_w(blk);
+  for (int blk = grp; blk < nblk; blk += KG) {
+    if (blk >= KG) group_sync();               // the previous channels' products are done
+    const uint2* sw = wp + ((long long)blk * K3 * ntn + blockIdx.y * NT) * 32;
+    for (int i = tid; i < K3 * NT * 16; i += 128) {                  // 16-byte pieces
+      const int t = i / (NT * 16), r = i - t * NT * 16;
+      cp16(s_w + t * NT * 32 + 2 * r, sw + (long long)t * ntn * 32 + 2 * r, true);
+    }
+    if constexpr (FIN) {
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {             // a thread splits the voxels it copied
-      const int hv = threadIdx.x + 128 * i;
-      if (hv < T::HV) {
+      for (int i = 0; i < NV; ++i) {
+        const int hv = tid + 128 * i;
+        if (hv < T::HV) {
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          uint4 u[3];
-          split_unit(s_f + half * 8 * T::HV + hv, T::HV, u);
+          for (int half = 0; half < 2; ++half) {
+            float f[8];
 #pragma unroll
-          for (int k = 0; k < 3; ++k) s_t[(2 * k + half) * T::HV + hv] = u[k];
+            for (int c = 0; c < 8; ++c) f[c] = vf[i] >= 0 && 8 * half + c < in.cf ? in.f[(8 * half + c) * nv + vf[i]] : 0.0f;
+            uint4 u[3];
+            split_unit(f, u);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) s_t[(2 * k + half) * T::HV + hv] = u[k];
+          }
+        }
+      }
+    } else {
+      const bool fa = 16 * blk < in.ca;
+      const long long cs = fa ? na : nv;       // units of a part of 8 channels
+      const uint4* src = fa ? in.a + 6LL * blk * cs : in.b + 6LL * (blk - in.ca / 16) * cs;
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const int hv = tid + 128 * i, v = fa ? va[i] : vf[i];
+        if (hv < T::HV) {
+#pragma unroll
+          for (int half = 0; half < 2; ++half)
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+              cp16(s_t + (2 * k + half) * T::HV + hv, v >= 0 ? src + (3 * half + k) * cs + v : in.a, v >= 0);
         }
       }
     }
-    if (blk + 1 < nblk) {
-      fetch(blk + 1);
-      asm volatile("cp.async.wait_group 1;\n" ::: "memory");        // the weights
-    } else {
-      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    }
-    __syncthreads();
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    group_sync();
     const uint2* wb = s_w + lane;
 #pragma unroll 1
     for (int kz = 0; kz < K; ++kz) {
@@ -240,24 +282,59 @@ __global__ void __launch_bounds__(128) k_conv_mma(ConvIn in, const uint2* __rest
           for (int k = 0; k < 4; ++k) acc[i][n][k] += lo[i][n][k];
     }
   }
-  // accumulator (row r, column c): x = r, output channel c
+  if constexpr (KG > 1) {                      // the groups' sums, in order
+    float* s_a = reinterpret_cast<float*>(smem + grp * GB);
+    group_sync();
+    if (grp > 0) {
+#pragma unroll
+      for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) s_a[((i * NT + n) * 4 + k) * 128 + tid] = acc[i][n][k];
+    }
+    __syncthreads();
+    if (grp > 0) return;
+#pragma unroll
+    for (int g = 1; g < KG; ++g) {
+      const float* p = reinterpret_cast<const float*>(smem + g * GB);
+#pragma unroll
+      for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) acc[i][n][k] += p[((i * NT + n) * 4 + k) * 128 + tid];
+    }
+  }
+  // accumulator (row r, columns c, c + 1): x = r, output channels c, c + 1
 #pragma unroll
   for (int i = 0; i < MT; ++i) {
     const int m = warp * MT + i;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int x = tx0 + (lane >> 2), y = ty0 + 2 * (m & 1) + (k >> 1), z = tz0 + (m >> 1);
+    for (int h = 0; h < 2; ++h) {
+      const int x = tx0 + (lane >> 2), y = ty0 + 2 * (m & 1) + h, z = tz0 + (m >> 1);
       if (x < d.x && y < d.y && z < d.z) {
         const long long v = ((long long)z * d.y + y) * d.x + x;
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
-          const int co = (blockIdx.y * NT + n) * 8 + (lane & 3) * 2 + (k & 1);
-          if (co < cout) {
-            float r = acc[i][n][k];
-            if (bias) r += bias[co];
-            if (relu) r = fmaxf(r, 0.0f);
-            if (mask && !(mask[co * nv + v] > 0.0f)) r = 0.0f;
-            out[co * nv + v] = r;
+          const int cb = blockIdx.y * NT + n, co = cb * 8 + (lane & 3) * 2;
+          if (co < cout) {                     // cout is even
+            float r[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              r[e] = acc[i][n][2 * h + e] + bias[co + e];
+              if (relu) r[e] = fmaxf(r[e], 0.0f);
+            }
+            if (out.s) {
+              unsigned u[3];
+              split_pair(r[0], r[1], u);
+#pragma unroll
+              for (int k = 0; k < 3; ++k)
+                reinterpret_cast<unsigned*>(out.s + (3LL * cb + k) * nv + v)[lane & 3] = u[k];
+            } else {
+              out.f[co * nv + v] = r[0];
+              out.f[(co + 1) * nv + v] = r[1];
+            }
           }
         }
       }
@@ -302,44 +379,50 @@ __global__ void k_pack_weights(const __nv_bfloat16* __restrict__ w, const __grid
   }
 }
 
-template <int K, int MT, int NT>
-cudaError_t conv_mma_t(const ConvIn& in, const uint2* wp, const float* bias, const float* mask, float* out,
-                       int cout, Dims d, int relu, cudaStream_t st) {
+template <int K, int MT, int NT, int KG, bool FIN>
+cudaError_t conv_mma_t(const SplitIn& in, const uint2* wp, const float* bias, const SplitOut& out, int cout, Dims d,
+                       int relu, cudaStream_t st) {
   using T = Tile<K, 2 * MT>;
-  const size_t sm = (size_t)T::HV * (6 * 16 + 16 * 4) + (size_t)K * K * K * NT * 256;
-  cudaError_t e = ensure_smem((const void*)k_conv_mma<K, MT, NT>, sm);
-  if (e == cudaSuccess) e = ensure_carveout_max((const void*)k_conv_mma<K, MT, NT>);
+  const size_t sm = (size_t)KG * (T::HV * 6 * 16 + (size_t)K * K * K * NT * 256);
+  auto kernel = k_conv_mma<K, MT, NT, KG, FIN>;
+  cudaError_t e = ensure_smem((const void*)kernel, sm);
+  if (e == cudaSuccess) e = ensure_carveout_max((const void*)kernel);
   if (e != cudaSuccess) return e;
   const int ntn = (cout + 7) / 8;
   const int tiles = ((d.x + 7) / 8) * ((d.y + 3) / 4) * ((d.z + 2 * MT - 1) / (2 * MT));
-  k_conv_mma<K, MT, NT><<<dim3(tiles, (ntn + NT - 1) / NT), 128, sm, st>>>(in, wp, ntn, bias, mask, out, cout,
-                                                                          d, relu);
+  kernel<<<dim3(tiles, (ntn + NT - 1) / NT), 128 * KG, sm, st>>>(in, wp, ntn, bias, out, cout, d, relu);
   count_launch();
   return cudaGetLastError();
 }
 
-// Tile of a convolution (K = 3): of 128 or 64 voxels by 40, 32, 16 or 8 output
-// channels, the one with the least estimated time: rounds of blocks over the
-// SMs times a block's cost in matrix instructions, which the smaller tiles
-// raise by what they load per instruction (a warp of the largest tile issues
-// 24 instructions for 8 fragment loads, of the smallest 3 for 4).
-inline cudaError_t conv_mma(int K, const ConvIn& in, const uint2* wp, const float* bias, const float* mask,
-                            float* out, int cout, Dims d, int relu, cudaStream_t st) {
-  if (K == 1) return cout <= 8 ? conv_mma_t<1, 2, 1>(in, wp, bias, mask, out, cout, d, relu, st)
-                               : conv_mma_t<1, 2, 2>(in, wp, bias, mask, out, cout, d, relu, st);
-  auto cost = [&](int mt, int nt, double block) {
+// Tile of a convolution (K = 3): 128 or 64 voxels by 40, 32, 16 or 8 output
+// channels, in 1, 2 or 4 groups; the one with the least estimated time.  Per 16
+// channels a block issues 324 MT NT matrix instructions, half a one a clock
+// when several groups share an SM (the small tiles up to twice that long: they
+// load more fragments per instruction); alone a group takes twice as long, and
+// about 1,500 clocks more for its copies.
+inline cudaError_t conv_mma(int K, const SplitIn& in, const uint2* wp, const float* bias, const SplitOut& out,
+                            int cout, Dims d, int relu, cudaStream_t st) {
+  if (K == 1) return conv_mma_t<1, 2, 1, 1, false>(in, wp, bias, out, cout, d, relu, st);
+  if (in.f) return conv_mma_t<3, 2, 2, 1, true>(in, wp, bias, out, cout, d, relu, st);
+  const int nblk = (in.ca + in.cb) / 16;
+  auto cost = [&](int mt, int nt, int kg, int resident, double load) {
     if (cout % (8 * nt) != 0) return 1e30;
     const long long b = (long long)((d.x + 7) / 8) * ((d.y + 3) / 4) * ((d.z + 2 * mt - 1) / (2 * mt)) * (cout / (8 * nt));
-    return (double)((b + num_sms() - 1) / num_sms()) * block;
+    const double per = (double)((b + num_sms() - 1) / num_sms());
+    const double mma = 648.0 * mt * nt * load, alone = (nblk + kg - 1) / kg * (2.0 * mma + 1500.0);
+    return std::max(std::ceil(per / resident) * alone, per * nblk * mma * 1.2);
   };
-  const double c[5] = {cost(2, 4, 24.0), cost(2, 5, 30.0), cost(2, 2, 13.5), cost(1, 2, 8.5), cost(1, 1, 6.0)};
-  switch ((int)(std::min_element(c, c + 5) - c)) {
-    case 0: return conv_mma_t<3, 2, 4>(in, wp, bias, mask, out, cout, d, relu, st);
-    case 1: return conv_mma_t<3, 2, 5>(in, wp, bias, mask, out, cout, d, relu, st);
-    case 2: return conv_mma_t<3, 2, 2>(in, wp, bias, mask, out, cout, d, relu, st);
-    case 3: return conv_mma_t<3, 1, 2>(in, wp, bias, mask, out, cout, d, relu, st);
+  const double c[6] = {cost(2, 4, 1, 2, 1.0), cost(2, 5, 2, 1, 1.0), cost(2, 4, 2, 1, 1.0),
+                       cost(2, 2, 1, 4, 1.1), cost(1, 2, 2, 2, 1.4), cost(1, 1, 4, 1, 2.0)};
+  switch ((int)(std::min_element(c, c + 6) - c)) {
+    case 0: return conv_mma_t<3, 2, 4, 1, false>(in, wp, bias, out, cout, d, relu, st);
+    case 1: return conv_mma_t<3, 2, 5, 2, false>(in, wp, bias, out, cout, d, relu, st);
+    case 2: return conv_mma_t<3, 2, 4, 2, false>(in, wp, bias, out, cout, d, relu, st);
+    case 3: return conv_mma_t<3, 2, 2, 1, false>(in, wp, bias, out, cout, d, relu, st);
+    case 4: return conv_mma_t<3, 1, 2, 2, false>(in, wp, bias, out, cout, d, relu, st);
   }
-  return conv_mma_t<3, 1, 1>(in, wp, bias, mask, out, cout, d, relu, st);
+  return conv_mma_t<3, 1, 1, 4, false>(in, wp, bias, out, cout, d, relu, st);
 }
 
 // ---------------------------------------------------------------- training
@@ -367,7 +450,9 @@ __device__ __forceinline__ float2 unpair2(unsigned long long r) {
   return o;
 }
 
-// out as k_conv_mma, from FP32 copies of the weights wf [ci][t][coutp].  A warp
+// out[co][v] = bias[co] + sum_ci sum_t w[co][ci][t] in[ci][v + t - H], then
+// relu, or zero where mask[co][v] <= 0 (gradient behind a relu), from FP32
+// copies of the weights wf [ci][t][coutp].  A warp
 // takes the 8 x 4 voxels of a z plane and CO channels; 4 warps: ZW planes by
 // 4 / ZW channel groups (8 channels per block).  Eight input channels with
 // their halo and weights are copied while the eight before are summed.
