@@ -11,10 +11,11 @@
 // among codelets compiled into the one kernel (a switch per direction instead
 // of a kernel per pair of lengths); each line is computed with the arithmetic
 // of the separate passes (fastfft.cuh), so the products agree bit for bit.
-// 16^3 sphere: 13.4 -> 11.5 us a product (9.9 with the tables loaded ahead of
-// the wait for the kernel before).  With 16 right-hand sides on a
-// 40 x 29 x 22 ellipsoid the two kernels take what the four took (43.6 against
-// 43.4 us), so the line lies at the lengths whose planes fit an SM twice.
+// 16^3 sphere: 13.4 -> 11.5 us a product, 9.7 with the tables loaded ahead of the
+// wait for the kernel before, 8.8 with the product in registers in the z pass
+// and no division per item here.  With 16 right-hand sides on a 40 x 29 x 22
+// ellipsoid the two kernels took what the four took (43.6 against 43.4 us; 37
+// now), so the line lies at the lengths whose planes fit an SM twice.
 #include "fastfft.cuh"
 
 namespace dda {
@@ -23,12 +24,31 @@ namespace {
 
 constexpr int kXYT = 256;
 
+// A thread's items threadIdx.x, threadIdx.x + kXYT, ... of (q, t), t < n: q = item
+// / n and t = item % n advance by constants (one division, at the start); none
+// when n = 0 (a plane without dipoles)
+struct Items {
+  int q, t, n, dq, dt;
+  __device__ __forceinline__ explicit Items(int n_) : n(max(n_, 1)) {
+    q = threadIdx.x / n;
+    t = threadIdx.x - q * n;
+    dq = kXYT / n;
+    dt = kXYT - dq * n;
+    if (n_ <= 0) q = 1 << 20;
+  }
+  __device__ __forceinline__ void next() {
+    q += dq;
+    t += dt;
+    if (t >= n) { t -= n; ++q; }
+  }
+};
+
 // Row transforms, nrow rows at P + t ld; Q is scratch of the same shape.
 // Forward: P[t][n] (n < kHalf M2 may be nonzero) -> P[t][k].
 template <int M1, int M2>
 __device__ __forceinline__ void rows_fwd(c64* P, c64* Q, int nrow, int ld, const c64* tw) {
-  for (int it = threadIdx.x; it < nrow * M2; it += kXYT) {
-    const int j = it / nrow, t = it - j * nrow;
+  for (Items it(nrow); it.q < M2; it.next()) {
+    const int j = it.q, t = it.t;
     c64 v[M1];
 #pragma unroll
     for (int i = 0; i < M1; ++i) v[i] = i < kHalf<M1, M2> ? P[t * ld + j + M2 * i] : zero<float>();
@@ -39,8 +59,8 @@ __device__ __forceinline__ void rows_fwd(c64* P, c64* Q, int nrow, int ld, const
     for (int k1 = 0; k1 < M1; ++k1) Q[t * ld + k1 * M2 + j] = v[k1];
   }
   __syncthreads();
-  for (int it = threadIdx.x; it < nrow * M1; it += kXYT) {
-    const int k1 = it / nrow, t = it - k1 * nrow;
+  for (Items it(nrow); it.q < M1; it.next()) {
+    const int k1 = it.q, t = it.t;
     c64 u[M2];
 #pragma unroll
     for (int j = 0; j < M2; ++j) u[j] = Q[t * ld + k1 * M2 + j];
@@ -53,8 +73,8 @@ __device__ __forceinline__ void rows_fwd(c64* P, c64* Q, int nrow, int ld, const
 // Inverse: P[t][k] -> P[t][n], n < kHalf M2.
 template <int M1, int M2>
 __device__ __forceinline__ void rows_inv(c64* P, c64* Q, int nrow, int ld, const c64* tw) {
-  for (int it = threadIdx.x; it < nrow * M1; it += kXYT) {
-    const int k1 = it / nrow, t = it - k1 * nrow;
+  for (Items it(nrow); it.q < M1; it.next()) {
+    const int k1 = it.q, t = it.t;
     c64 u[M2];
 #pragma unroll
     for (int k2 = 0; k2 < M2; ++k2) u[k2] = P[t * ld + k1 + M1 * k2];
@@ -65,8 +85,8 @@ __device__ __forceinline__ void rows_inv(c64* P, c64* Q, int nrow, int ld, const
     for (int j = 0; j < M2; ++j) Q[t * ld + k1 * M2 + j] = u[j];
   }
   __syncthreads();
-  for (int it = threadIdx.x; it < nrow * M2; it += kXYT) {
-    const int j = it / nrow, t = it - j * nrow;
+  for (Items it(nrow); it.q < M2; it.next()) {
+    const int j = it.q, t = it.t;
     c64 v[M1];
 #pragma unroll
     for (int k1 = 0; k1 < M1; ++k1) v[k1] = Q[t * ld + k1 * M2 + j];
@@ -76,63 +96,71 @@ __device__ __forceinline__ void rows_inv(c64* P, c64* Q, int nrow, int ld, const
   }
 }
 
-// Column transforms of a plane.  Forward: rows y0 .. y0 + nrow - 1 of the plane
-// are P[t][kx]; out[ky][Mx] in global memory; Q [M][Mx].
+// Column transforms of a plane, cw columns at a time; Q [M][cw].  Forward: rows
+// y0 .. y0 + nrow - 1 of the plane are P[t][kx]; out[ky][Mx] in global memory.
 template <int M1, int M2>
-__device__ __forceinline__ void cols_fwd(const c64* P, c64* Q, int y0, int nrow, int ld, int Mx,
+__device__ __forceinline__ void cols_fwd(const c64* P, c64* Q, int y0, int nrow, int ld, int Mx, int cw,
                                          const c64* tw, c64* __restrict__ out) {
-  for (int it = threadIdx.x; it < Mx * M2; it += kXYT) {
-    const int j = it / Mx, kx = it - j * Mx;
-    c64 v[M1];
+  for (int kx0 = 0; kx0 < Mx; kx0 += cw) {
+    const int w = min(cw, Mx - kx0);
+    if (kx0) __syncthreads();                  // Q has been read
+    for (Items it(w); it.q < M2; it.next()) {
+      const int j = it.q, kx = kx0 + it.t;
+      c64 v[M1];
 #pragma unroll
-    for (int i = 0; i < M1; ++i) {
-      const int t = j + M2 * i - y0;
-      v[i] = (i < kHalf<M1, M2> && t >= 0 && t < nrow) ? P[t * ld + kx] : zero<float>();
+      for (int i = 0; i < M1; ++i) {
+        const int t = j + M2 * i - y0;
+        v[i] = (i < kHalf<M1, M2> && t >= 0 && t < nrow) ? P[t * ld + kx] : zero<float>();
+      }
+      dft_padded<float, M1, kHalf<M1, M2>>(v);
+#pragma unroll
+      for (int k1 = 1; k1 < M1; ++k1) v[k1] = twiddle<float, false>(v[k1], tw[j * k1]);
+#pragma unroll
+      for (int k1 = 0; k1 < M1; ++k1) Q[(k1 * M2 + j) * w + it.t] = v[k1];
     }
-    dft_padded<float, M1, kHalf<M1, M2>>(v);
+    __syncthreads();
+    for (Items it(w); it.q < M1; it.next()) {
+      const int k1 = it.q, kx = kx0 + it.t;
+      c64 u[M2];
 #pragma unroll
-    for (int k1 = 1; k1 < M1; ++k1) v[k1] = twiddle<float, false>(v[k1], tw[j * k1]);
+      for (int j = 0; j < M2; ++j) u[j] = Q[(k1 * M2 + j) * w + it.t];
+      cl::Dft<float, false, M2>::run(u);
 #pragma unroll
-    for (int k1 = 0; k1 < M1; ++k1) Q[(k1 * M2 + j) * Mx + kx] = v[k1];
-  }
-  __syncthreads();
-  for (int it = threadIdx.x; it < Mx * M1; it += kXYT) {
-    const int k1 = it / Mx, kx = it - k1 * Mx;
-    c64 u[M2];
-#pragma unroll
-    for (int j = 0; j < M2; ++j) u[j] = Q[(k1 * M2 + j) * Mx + kx];
-    cl::Dft<float, false, M2>::run(u);
-#pragma unroll
-    for (int k2 = 0; k2 < M2; ++k2) out[(k1 + M1 * k2) * Mx + kx] = u[k2];
+      for (int k2 = 0; k2 < M2; ++k2) out[(k1 + M1 * k2) * Mx + kx] = u[k2];
+    }
   }
 }
 
 // Inverse: in[ky][Mx] in global memory -> P[t][kx] for rows y0 + t, t < nrow.
 template <int M1, int M2>
 __device__ __forceinline__ void cols_inv(const c64* __restrict__ in, c64* P, c64* Q, int y0, int nrow, int ld,
-                                         int Mx, const c64* tw) {
-  for (int it = threadIdx.x; it < Mx * M1; it += kXYT) {
-    const int k1 = it / Mx, kx = it - k1 * Mx;
-    c64 u[M2];
+                                         int Mx, int cw, const c64* tw) {
+  for (int kx0 = 0; kx0 < Mx; kx0 += cw) {
+    const int w = min(cw, Mx - kx0);
+    if (kx0) __syncthreads();                  // Q has been read
+    for (Items it(w); it.q < M1; it.next()) {
+      const int k1 = it.q, kx = kx0 + it.t;
+      c64 u[M2];
 #pragma unroll
-    for (int k2 = 0; k2 < M2; ++k2) u[k2] = in[(k1 + M1 * k2) * Mx + kx];
-    cl::Dft<float, true, M2>::run(u);
+      for (int k2 = 0; k2 < M2; ++k2) u[k2] = in[(k1 + M1 * k2) * Mx + kx];
+      cl::Dft<float, true, M2>::run(u);
 #pragma unroll
-    for (int j = 1; j < M2; ++j) u[j] = twiddle<float, true>(u[j], tw[j * k1]);
+      for (int j = 1; j < M2; ++j) u[j] = twiddle<float, true>(u[j], tw[j * k1]);
 #pragma unroll
-    for (int j = 0; j < M2; ++j) Q[(k1 * M2 + j) * Mx + kx] = u[j];
-  }
-  __syncthreads();
-  for (int it = threadIdx.x; it < Mx * M2; it += kXYT) {
-    const int j = it / Mx, kx = it - j * Mx;
-    c64 v[M1];
+      for (int j = 0; j < M2; ++j) Q[(k1 * M2 + j) * w + it.t] = u[j];
+    }
+    __syncthreads();
+    for (Items it(w); it.q < M2; it.next()) {
+      const int j = it.q, kx = kx0 + it.t;
+      c64 v[M1];
 #pragma unroll
-    for (int k1 = 0; k1 < M1; ++k1) v[k1] = Q[(k1 * M2 + j) * Mx + kx];
-    cl::Dft<float, true, M1>::run(v);
+      for (int k1 = 0; k1 < M1; ++k1) v[k1] = Q[(k1 * M2 + j) * w + it.t];
+      cl::Dft<float, true, M1>::run(v);
 #pragma unroll
-    for (int i = 0; i < kHalf<M1, M2>; ++i) {
-      const int t = j + M2 * i - y0;
-      if (t >= 0 && t < nrow) P[t * ld + kx] = v[i];
+      for (int i = 0; i < kHalf<M1, M2>; ++i) {
+        const int t = j + M2 * i - y0;
+        if (t >= 0 && t < nrow) P[t * ld + kx] = v[i];
+      }
     }
   }
 }
@@ -148,7 +176,7 @@ __device__ __forceinline__ void cols_inv(const c64* __restrict__ in, c64* P, c64
   }
 
 // Shared memory of a plane: twiddles of both axes, P [nrow][ld], Q (the larger
-// of P's shape and [My][Mx]), and the row offsets (ny + 1).
+// of P's shape and [My][cw]), and the row offsets (ny + 1).
 struct PlaneMem {
   c64 *twx, *twy, *P, *Q;
   long long* off;
@@ -169,9 +197,18 @@ __device__ __forceinline__ PlaneMem plane_mem(unsigned char* smem, const c64* __
   m.nrow = lat.yr ? lat.yr[2 * z + 1] - m.y0 + 1 : ny;
   return m;
 }
-size_t plane_bytes(int ny, int Mx, int My) {
-  const size_t p = (size_t)ny * (Mx + 1), q = (size_t)Mx * My;
+size_t plane_bytes(int ny, int Mx, int My, int cw) {
+  const size_t p = (size_t)ny * (Mx + 1), q = (size_t)cw * My;
   return 16 * ((ny + 2) / 2) + (Mx + My + p + (p > q ? p : q)) * sizeof(c64);
+}
+// Columns transformed at a time: all, or half of them where whole planes let no
+// more than `few` blocks share an SM and the launch fills those (96 x 96 points
+// with 8 right-hand sides, two planes an SM: 35.1 -> 32.4 us forward, 42.0 -> 40.4
+// inverse; 80 x 64 with 16, three: 18.3 -> 18.6 and 20.0 -> 18.9; 64 x 64, four:
+// 19.4 -> 20.3 and 19.7 -> 20.5).
+int plane_columns(const FastArgs& a, int few) {
+  const long long fit = (227LL << 10) / (long long)(plane_bytes(a.ny, a.Mx, a.My, a.Mx) + 1024);
+  return fit <= few && 3LL * a.nz * a.nrhs > fit * num_sms() ? a.Mx / 2 : a.Mx;
 }
 // row (of ny) of dipole i: the last one whose offset is <= i
 __device__ __forceinline__ int row_in_plane(const long long* off, int ny, long long i) {
@@ -184,9 +221,9 @@ __device__ __forceinline__ int row_in_plane(const long long* off, int ny, long l
 
 // grid (nz, 3 nrhs)
 template <bool CONJ>
-__global__ void __launch_bounds__(kXYT) fk_xy_fwd(const c64* __restrict__ x, c64* __restrict__ B2,
+__global__ void __launch_bounds__(kXYT, 4) fk_xy_fwd(const c64* __restrict__ x, c64* __restrict__ B2,
                                                   LatticeDev lat, const c64* __restrict__ beta,
-                                                  long long n_occ, int ny, int Mx, int My,
+                                                  long long n_occ, int ny, int Mx, int My, int cw,
                                                   const c64* __restrict__ tw, int bstride,
                                                   const int* __restrict__ skip) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -224,17 +261,17 @@ __global__ void __launch_bounds__(kXYT) fk_xy_fwd(const c64* __restrict__ x, c64
 #undef ROWS
   __syncthreads();
   c64* out = B2 + ((long long)cc * gridDim.x + z) * My * Mx;
-#define COLS(A, B) cols_fwd<A, B>(m.P, m.Q, m.y0, m.nrow, m.ld, Mx, m.twy, out)
+#define COLS(A, B) cols_fwd<A, B>(m.P, m.Q, m.y0, m.nrow, m.ld, Mx, cw, m.twy, out)
   DDA_XY_LENGTHS(My, COLS)
 #undef COLS
 }
 
 // grid (nz, 3 nrhs); dotp (or null): the block's partial of x^T y
 template <bool CONJ>
-__global__ void __launch_bounds__(kXYT) fk_yx_inv(const c64* __restrict__ B2, const c64* __restrict__ x,
+__global__ void __launch_bounds__(kXYT, 4) fk_yx_inv(const c64* __restrict__ B2, const c64* __restrict__ x,
                                                   c64* __restrict__ y, LatticeDev lat,
                                                   const c64* __restrict__ beta, long long n_occ, int ny,
-                                                  int Mx, int My, const c64* __restrict__ tw,
+                                                  int Mx, int My, int cw, const c64* __restrict__ tw,
                                                   double* __restrict__ dotp, int bstride,
                                                   const int* __restrict__ skip) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -246,7 +283,7 @@ __global__ void __launch_bounds__(kXYT) fk_yx_inv(const c64* __restrict__ B2, co
   pdl_launch();
   if (skip && skip[cc / 3]) return;
   const c64* in = B2 + ((long long)cc * gridDim.x + z) * My * Mx;
-#define COLS(A, B) cols_inv<A, B>(in, m.P, m.Q, m.y0, m.nrow, m.ld, Mx, m.twy)
+#define COLS(A, B) cols_inv<A, B>(in, m.P, m.Q, m.y0, m.nrow, m.ld, Mx, cw, m.twy)
   DDA_XY_LENGTHS(My, COLS)
 #undef COLS
   __syncthreads();
@@ -302,8 +339,8 @@ __global__ void __launch_bounds__(kXYT) fk_yx_inv(const c64* __restrict__ B2, co
 bool xy_length(int M) { return M == 32 || M == 40 || M == 48 || M == 64 || M == 80 || M == 96; }
 
 template <typename K, typename... Args>
-cudaError_t launch_plane(K kernel, const FastArgs& a, Args... args) {
-  const size_t sm = plane_bytes(a.ny, a.Mx, a.My);
+cudaError_t launch_plane(K kernel, const FastArgs& a, int cw, Args... args) {
+  const size_t sm = plane_bytes(a.ny, a.Mx, a.My, cw);
   cudaError_t e = ensure_smem((const void*)kernel, sm);
   if (e == cudaSuccess) e = ensure_carveout_max((const void*)kernel);
   if (e != cudaSuccess) return e;
@@ -321,9 +358,10 @@ bool fast_xy_supported(int Mx, int My) { return fast::xy_length(Mx) && fast::xy_
 cudaError_t fast_xy_fwd_c64(const FastArgs& a) {
   const c64 *x = (const c64*)a.in, *beta = (const c64*)a.beta, *tw = (const c64*)a.tw;
   c64* out = (c64*)a.out;
-  return a.adj ? fast::launch_plane(fast::fk_xy_fwd<true>, a, x, out, a.lat, beta, a.n_occ, a.ny, a.Mx, a.My, tw,
+  const int cw = fast::plane_columns(a, 2);
+  return a.adj ? fast::launch_plane(fast::fk_xy_fwd<true>, a, cw, x, out, a.lat, beta, a.n_occ, a.ny, a.Mx, a.My, cw, tw,
                                     a.bstride, a.skip)
-               : fast::launch_plane(fast::fk_xy_fwd<false>, a, x, out, a.lat, beta, a.n_occ, a.ny, a.Mx, a.My, tw,
+               : fast::launch_plane(fast::fk_xy_fwd<false>, a, cw, x, out, a.lat, beta, a.n_occ, a.ny, a.Mx, a.My, cw, tw,
                                     a.bstride, a.skip);
 }
 
@@ -331,9 +369,10 @@ cudaError_t fast_xy_fwd_c64(const FastArgs& a) {
 cudaError_t fast_yx_inv_c64(const FastArgs& a) {
   const c64 *in = (const c64*)a.in, *x = (const c64*)a.x, *beta = (const c64*)a.beta, *tw = (const c64*)a.tw;
   c64* out = (c64*)a.out;
-  return a.adj ? fast::launch_plane(fast::fk_yx_inv<true>, a, in, x, out, a.lat, beta, a.n_occ, a.ny, a.Mx, a.My,
+  const int cw = fast::plane_columns(a, 3);
+  return a.adj ? fast::launch_plane(fast::fk_yx_inv<true>, a, cw, in, x, out, a.lat, beta, a.n_occ, a.ny, a.Mx, a.My, cw,
                                     tw, a.dotp, a.bstride, a.skip)
-               : fast::launch_plane(fast::fk_yx_inv<false>, a, in, x, out, a.lat, beta, a.n_occ, a.ny, a.Mx, a.My,
+               : fast::launch_plane(fast::fk_yx_inv<false>, a, cw, in, x, out, a.lat, beta, a.n_occ, a.ny, a.Mx, a.My, cw,
                                     tw, a.dotp, a.bstride, a.skip);
 }
 
