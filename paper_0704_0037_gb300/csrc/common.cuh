@@ -183,6 +183,11 @@ using cdf = cpx<df>;
 // words form one f32x2 register pair and the low words another, so each step
 // of the double-float algorithms above runs once for both parts (the same
 // roundings per part as the scalar form).
+// The pair (0, 0) as a value the compiler cannot see (a constant it does not
+// know to stay unwritten): a product's rounded high word is an fma with this
+// addend.  A paired multiply followed by a paired add may be contracted into
+// one fused operation, which adds the product's rounding error a second time.
+[[maybe_unused]] static __constant__ unsigned long long g_nul2;
 #ifdef DDA_F32X2
 struct df2 { unsigned long long h, l; };   // (re.hi, im.hi), (re.lo, im.lo)
 __device__ __forceinline__ unsigned long long f2add(unsigned long long a, unsigned long long b) {
@@ -240,12 +245,7 @@ __device__ __forceinline__ df2 dsub2(df2 a, df2 b) {
 // Product without the final renormalisation: (p, e), p the rounded product of
 // the high words and e its error plus the cross terms (within 2 ulp of p)
 __device__ __forceinline__ df2 dmul2_raw(df2 a, df2 b) {
-  // The rounded product comes from an fma with a zero addend the compiler
-  // cannot see through (a - a): a paired multiply followed by the paired add
-  // below may otherwise be contracted into one fused operation, which adds
-  // the product's rounding error a second time.
-  const unsigned long long z = f2sub(a.h, a.h);
-  const unsigned long long p = f2fma(a.h, b.h, z);
+  const unsigned long long p = f2fma(a.h, b.h, g_nul2);
   unsigned long long e = f2fma(a.h, b.h, f2sub(0ull, p));
   e = f2fma(a.h, b.l, e);
   e = f2fma(a.l, b.h, e);
@@ -258,21 +258,13 @@ __device__ __forceinline__ df2 drenorm2(df2 a) {
 __device__ __forceinline__ df2 dmul2(df2 a, df2 b) { return drenorm2(dmul2_raw(a, b)); }
 // the pair (v, v) of a double-float scalar
 __device__ __forceinline__ df2 dsplat(df v) { return df2{pk2(v.hi, v.hi), pk2(v.lo, v.lo)}; }
-// multiply the first part by -1 (exact)
-__device__ __forceinline__ df2 dneg_re(df2 a) {
-  const unsigned long long m = pk2(-1.0f, 1.0f);
-  return df2{f2mul(a.h, m), f2mul(a.l, m)};
-}
-// (a + ib)(c + id) = (ac - bd) + i(ad + bc): (ac, ad) + (-bd, bc), renormalised
-// once, after the sum (25 paired instructions; with both products
-// renormalised before it 28, at the same error bound: what the sum loses is
-// 2^-48 of the products)
+// (a + ib)(c + id) = (ac - bd) + i(ad + bc): a (c, d) + b (-d, c), renormalised
+// once, after the sum (21 paired instructions; with both products renormalised
+// before it 24, at the same error bound: what the sum loses is 2^-48 of the
+// products)
 __device__ __forceinline__ cpx<df> dcmul(const cpx<df>& z, const cpx<df>& w) {
-  const df2 wp = dpack(w);
-  const df2 ws{pk2(w.y.hi, w.x.hi), pk2(w.y.lo, w.x.lo)};
-  const df2 p1 = dmul2_raw(dsplat(z.x), wp);
-  const df2 p2 = dmul2_raw(dsplat(z.y), ws);
-  return dunpack(drenorm2(dadd2(p1, dneg_re(p2))));
+  const df2 ws{pk2(-w.y.hi, w.x.hi), pk2(-w.y.lo, w.x.lo)};
+  return dunpack(drenorm2(dadd2(dmul2_raw(dsplat(z.x), dpack(w)), dmul2_raw(dsplat(z.y), ws))));
 }
 #endif
 

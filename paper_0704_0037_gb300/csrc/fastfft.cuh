@@ -372,6 +372,45 @@ __device__ __forceinline__ void zc_prefetch(const cpx<R>* D, int Mx, int My, int
   }
 }
 
+#ifdef DDA_F32X2
+// A double-float complex factor w as the two pairs its products take:
+// (c + id) w = c (w.x, w.y) + d (-w.y, w.x)
+struct DfFactor {
+  df2 p, q;
+  __device__ __forceinline__ explicit DfFactor(const cpx<df>& w) : p(dpack(w)), q{pk2(-w.y.hi, w.x.hi), pk2(-w.y.lo, w.x.lo)} {}
+};
+// A real double-float operand of df_dot3 and its negative, in both halves
+struct DfSplat {
+  df2 p, n;
+  __device__ __forceinline__ explicit DfSplat(df v) : p(dsplat(v)), n(dsplat(df(-v.hi, -v.lo))) {}
+};
+// r + a b: the product's high word is rounded, the negative of its error and cross terms comes from a's
+// negative, and the two-sum of the high words adds both
+__device__ __forceinline__ df2 df_macc(df2 r, const DfSplat& a, df2 b) {
+  const unsigned long long p = f2fma(a.p.h, b.h, g_nul2);
+  const unsigned long long ne = f2fma(a.n.l, b.h, f2fma(a.n.h, b.l, f2fma(a.n.h, b.h, p)));
+  const unsigned long long s = f2add(r.h, p), bb = f2sub(s, r.h);
+  const unsigned long long e = f2add(f2sub(r.h, f2sub(s, bb)), f2sub(p, bb));
+  return df2{s, f2add(e, f2sub(r.l, ne))};
+}
+// a v0 + b v1 + c v2 (vx[k], vy[k]: real and imaginary part of v_k): six
+// real-by-complex products whose error terms stay beside them, summed as they
+// are and renormalised once (75 paired instructions; renormalised product by
+// product 91).
+// 16 pairs of 46^3 cubes: z pass 1,324 -> 942 us, product 1,898 -> 1,514.
+__device__ __forceinline__ cpx<df> df_dot3(const DfFactor& a, const DfFactor& b, const DfFactor& c,
+                                           const DfSplat (&vx)[3], const DfSplat (&vy)[3]) {
+  df2 r{0ull, 0ull};
+  r = df_macc(r, vx[0], a.p);
+  r = df_macc(r, vy[0], a.q);
+  r = df_macc(r, vx[1], b.p);
+  r = df_macc(r, vy[1], b.q);
+  r = df_macc(r, vx[2], c.p);
+  r = df_macc(r, vy[2], c.q);
+  return dunpack(drenorm2(r));
+}
+#endif
+
 // Fourier-space product with the octant of FFT(G).  Work item (t, fz): the
 // six octant values at (fx, fy, fz) are loaded once and applied to both
 // kz = fz and kz = M - fz (sign flips for the components odd in z); the
@@ -400,29 +439,57 @@ __device__ __forceinline__ void zc_product(cpx<R>* s, const cpx<R>* __restrict__
   long long o = ((long long)fz * hy + fy) * hx + fx;
   int a1 = fz % M1, a2 = fz / M1;                // kz = fz
   int b1 = (M - fz) % M1, b2 = (M - fz) / M1;    // kz = M - fz
-#pragma unroll 2
+  constexpr int kUnroll = std::is_same<R, df>::value ? 1 : 2;
+#pragma unroll kUnroll
   for (; fz < hz; fz += FS, o += ostep) {
     cpx<R> d6[6];
     load_oct<R>(D, o, octs, d6);
-    const cpx<R> dxx = d6[0], dyy = d6[3], dzz = d6[5];
-    cpx<R> dxy = d6[1], ez = d6[2], fzz = d6[4];
-    if (nxs ^ nys) dxy = mk<R>(-dxy.x, -dxy.y);
-    if (nxs) ez = mk<R>(-ez.x, -ez.y);           // xz and yz at kz = fz
-    if (nys) fzz = mk<R>(-fzz.x, -fzz.y);
+#ifdef DDA_F32X2
+    if constexpr (std::is_same<R, df>::value) {
+      if (nxs ^ nys) d6[1] = mk<R>(-d6[1].x, -d6[1].y);
+      if (nxs) d6[2] = mk<R>(-d6[2].x, -d6[2].y);          // xz and yz at kz = fz
+      if (nys) d6[4] = mk<R>(-d6[4].x, -d6[4].y);
+      const int two = fz != 0 && 2 * fz != M;
+      // one copy of the code for kz = fz and kz = M - fz (where xz and yz, odd in
+      // z, change sign): the pass misses the instruction cache
+#pragma unroll 1
+      for (int h = 0; h <= two; ++h) {
+        const int e = (h ? Z::at(b1, b2) : Z::at(a1, a2)) * T + t2;
+        if (h) {
+          d6[2] = mk<R>(-d6[2].x, -d6[2].y);
+          d6[4] = mk<R>(-d6[4].x, -d6[4].y);
+        }
+        const DfFactor xx(d6[0]), xy(d6[1]), xz(d6[2]), yy(d6[3]), yz(d6[4]), zz(d6[5]);
+        const cpx<R> x = s[e], y = s[CS + e], z = s[2 * CS + e];
+        const DfSplat vx[3] = {DfSplat(x.x), DfSplat(y.x), DfSplat(z.x)};
+        const DfSplat vy[3] = {DfSplat(x.y), DfSplat(y.y), DfSplat(z.y)};
+        s[e] = df_dot3(xx, xy, xz, vx, vy);
+        s[CS + e] = df_dot3(xy, yy, yz, vx, vy);
+        s[2 * CS + e] = df_dot3(xz, yz, zz, vx, vy);
+      }
+    } else
+#endif
     {
-      const int e = Z::at(a1, a2) * T + t2;
-      const cpx<R> vx = s[e], vy = s[CS + e], vz = s[2 * CS + e];
-      s[e] = cmac(cmac(dxx * vx, dxy, vy), ez, vz);
-      s[CS + e] = cmac(cmac(dxy * vx, dyy, vy), fzz, vz);
-      s[2 * CS + e] = cmac(cmac(ez * vx, fzz, vy), dzz, vz);
-    }
-    if (fz != 0 && 2 * fz != M) {
-      // kz = M - fz: xz and yz change sign (odd in z): their terms are subtracted
-      const int e = Z::at(b1, b2) * T + t2;
-      const cpx<R> vx = s[e], vy = s[CS + e], vz = s[2 * CS + e];
-      s[e] = cnmac(cmac(dxx * vx, dxy, vy), ez, vz);
-      s[CS + e] = cnmac(cmac(dxy * vx, dyy, vy), fzz, vz);
-      s[2 * CS + e] = cnmac(cnmac(dzz * vz, ez, vx), fzz, vy);
+      const cpx<R> dxx = d6[0], dyy = d6[3], dzz = d6[5];
+      cpx<R> dxy = d6[1], ez = d6[2], fzz = d6[4];
+      if (nxs ^ nys) dxy = mk<R>(-dxy.x, -dxy.y);
+      if (nxs) ez = mk<R>(-ez.x, -ez.y);           // xz and yz at kz = fz
+      if (nys) fzz = mk<R>(-fzz.x, -fzz.y);
+      {
+        const int e = Z::at(a1, a2) * T + t2;
+        const cpx<R> vx = s[e], vy = s[CS + e], vz = s[2 * CS + e];
+        s[e] = cmac(cmac(dxx * vx, dxy, vy), ez, vz);
+        s[CS + e] = cmac(cmac(dxy * vx, dyy, vy), fzz, vz);
+        s[2 * CS + e] = cmac(cmac(ez * vx, fzz, vy), dzz, vz);
+      }
+      if (fz != 0 && 2 * fz != M) {
+        // kz = M - fz: xz and yz change sign (odd in z): their terms are subtracted
+        const int e = Z::at(b1, b2) * T + t2;
+        const cpx<R> vx = s[e], vy = s[CS + e], vz = s[2 * CS + e];
+        s[e] = cnmac(cmac(dxx * vx, dxy, vy), ez, vz);
+        s[CS + e] = cnmac(cmac(dxy * vx, dyy, vy), fzz, vz);
+        s[2 * CS + e] = cnmac(cnmac(dzz * vz, ez, vx), fzz, vy);
+      }
     }
     a1 += S1;
     a2 += S2;
@@ -456,7 +523,7 @@ __device__ __forceinline__ void zc_m2_one_codelet(cpx<R>* s, const cpx<R>* s_tw,
                                                   const cpx<R>* __restrict__ D, int Mx, int My,
                                                   int bx, int ky) {
   using Z = ZRows<R, M1, M2, T>;
-  constexpr int M = M1 * M2, CS = Z::rows * T;
+  constexpr int CS = Z::rows * T;
   const int t = threadIdx.x % T, q = threadIdx.x / T;
   const int kx = bx * T + t;
 #pragma unroll 1
