@@ -37,7 +37,9 @@ cudaError_t run_pass(int pass, const FastArgs& a) {
 }
 
 // The product passes alone, default tiles only (lengths without whole-line
-// passes and tile variants)
+// passes and tile variants).  P4 of the lengths with a 21-point phase takes 8
+// columns: blocks of 16 have 336 threads (147 points 20.0 -> 17.0 us, 189 48.3 ->
+// 44.4; 320 threads, 280 points, 13.9 -> 15.2).
 template <typename R, int M1, int M2>
 cudaError_t run_product_pass(int pass, const FastArgs& a) {
   using P = Passes<R, M1, M2>;
@@ -53,7 +55,7 @@ cudaError_t run_product_pass(int pass, const FastArgs& a) {
       return P::template zconv_t<P::TZ>((cpx<R>*)a.out, (const cpx<R>*)a.D, a.nz, a.Mx, a.My, tw, a.nrhs,
                                         a.skip, a.st, a.pdl);
     case FP_YINV:
-      return P::template yinv_t<P::T>((const cpx<R>*)a.in, (cpx<R>*)a.out, a.ny, a.nz, a.Mx, tw, a.nrhs,
+      return P::template yinv_t<P::NT == 336 ? P::T / 2 : P::T>((const cpx<R>*)a.in, (cpx<R>*)a.out, a.ny, a.nz, a.Mx, tw, a.nrhs,
                                       a.skip, a.st, a.pdl);
     case FP_XINV:
       return P::xinv((const cpx<R>*)a.in, (const typename P::V*)a.x, (typename P::V*)a.out, a.lat,

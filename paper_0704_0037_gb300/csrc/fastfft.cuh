@@ -889,6 +889,11 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>,
 // B1 [3][nrows][M]; grid (ceil(nrows/T), 3)
 template <int M> constexpr int kLD = (M % 2 == 1) ? M : M + 1;
 
+// blocks per SM the x passes' launch bounds ask for: four in
+// complex64 (at 270 points 56 registers, no spill: P5 of the 134^3 sphere
+// 59 -> 55 us), three in the wider arithmetic and from 290 points (eight rows,
+// 20 and more elements a thread: 512 points 380 us with three, 475 with two)
+template <typename R, int M> constexpr int kXB = (sizeof(R) == 4 && (M < 290 || M >= 1000)) ? 4 : 3;
 // Row t (0 <= t < T) of the block holding dipole i: the last t with
 // off[t] <= i, for the non-decreasing offsets off[0..T] of the block's rows
 // (off[0] <= i < off[T]; empty rows are skipped over).
@@ -902,22 +907,29 @@ __device__ __forceinline__ int row_of(const long long* off, long long i) {
   return t;
 }
 
-// Loads per thread issued together in the gather and scatter loops over a
-// block's dipoles
-// in the x forward and x inverse passes: more for the long lines, whose
-// blocks of few rows hold many dipoles, as far as the registers of the
-// blocks an SM holds allow
-template <int M> constexpr int kGUF = M >= 1000 ? 8 : 4;
-template <int M> constexpr int kGUI = M >= 1000 ? 16 : 4;
+// Outside their transforms the complex64 x passes of 256 points (P1) and 128
+// points (P5) and more work row by row, a warp to a row: no division of an
+// element's index, no search for a dipole's row (134^3 sphere P1 39.1 -> 33.8 us,
+// P5 51.3 -> 44.3; 256^3 314 -> 267, 379 -> 337; 50 x 110 x 100 P1 12.2 -> 12.9,
+// P5 15.9 -> 15.5).  Over shorter rows, and in the wider arithmetic, whose
+// instructions take as long for a warp half of whose lanes are past a row's end,
+// a block's threads run over its dipoles (12 x 100 x 100 by rows P1 5.0 -> 7.1
+// us; double-float 96 points 88 -> 108).
+template <typename R, int M> constexpr bool kRowsF = sizeof(R) == 4 && M >= 256;
+template <typename R, int M> constexpr bool kRowsI = sizeof(R) == 4 && M >= 128;
+// Dipoles per lane (by rows) whose loads are issued together: all of a row's
+// where the registers of the blocks an SM holds allow, and more for the long
+// lines, whose blocks of few rows hold many dipoles
+template <int M> constexpr int kGR = M >= 1000 ? 8 : (M / 2 + 32) / 32 < 5 ? (M / 2 + 32) / 32 : 5;
 
 template <typename R, int M1, int M2, int T, bool CONJ>
-__global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, 3, (M1 * M2 + T * kLD<M1 * M2>) * sizeof(cpx<R>))) fk_xfwd(const typename VecOf<R>::type* __restrict__ x,
+__global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, kRowsF<R, M1 * M2> ? kXB<R, M1 * M2> : 3, (M1 * M2 + T * kLD<M1 * M2>) * sizeof(cpx<R>))) fk_xfwd(const typename VecOf<R>::type* __restrict__ x,
                                                           cpx<R>* __restrict__ B1, LatticeDev lat,
                                                           const cpx<R>* __restrict__ beta,
                                                           long long n_occ, int nrows,
                                                           const cpx<R>* __restrict__ tw,
                                                           int bstride, const int* __restrict__ skip) {
-  constexpr int M = M1 * M2, NT = T * kQ<M1, M2>, LD = kLD<M>, kGU = kGUF<M1 * M2>;
+  constexpr int M = M1 * M2, NT = T * kQ<M1, M2>, LD = kLD<M>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ long long s_off[T + 1];
   cpx<R>* s_tw = reinterpret_cast<cpx<R>*>(smem_raw);
@@ -936,40 +948,53 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, 3, (M1 *
     if (threadIdx.x < T) s_row[threadIdx.x] = lat.arow ? lat.arow[min(i, nr - 1)] : i;
   }
   load_tw(s_tw, tw, M, NT);
-  for (int i = threadIdx.x; i < T * LD; i += NT) a[i] = zero<R>();
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if constexpr (kRowsF<R, M>) {
+    for (int r = wid; r < T && wid < NT / 32; r += NT / 32)          // the inputs of the first phase
+      for (int m = lane; m < kHalf<M1, M2> * M2; m += 32) a[r * LD + m] = zero<R>();
+  } else {
+    for (int i = threadIdx.x; i < T * LD; i += NT) a[i] = zero<R>();
+  }
   pdl_wait();
   pdl_launch();
   if (skip && skip[cc / 3]) return;
   __syncthreads();
   {
-    // all threads over the block's dipoles (contiguous in x: rows r0..r0+T-1),
-    // kGU independent loads of x, xi and mat in flight per thread
     const typename VecOf<R>::type* __restrict__ xc = x + (long long)cc * n_occ;
     const uint16_t* __restrict__ xi = lat.xi;
     const uint8_t* __restrict__ mt = lat.mat;
-    const long long S0 = s_off[0];
-    const int span = (int)(s_off[T] - S0);
-    for (int k0 = threadIdx.x; k0 < span; k0 += kGU * NT) {
-      typename VecOf<R>::type xv[kGU];
-      int xk[kGU], mk_[kGU];
+    // GU independent loads of x, xi and mat in flight: of dipoles k0, k0 + step, ...
+    // below n of the run that starts at S0, in row r (searched for when r < 0)
+    auto gather = [&](auto gu, long long S0, int n, int k0, int step, int r) {
+      constexpr int GU = decltype(gu)::value;
+      for (; k0 < n; k0 += GU * step) {
+        typename VecOf<R>::type xv[GU];
+        int xk[GU], mk_[GU];
 #pragma unroll
-      for (int u = 0; u < kGU; ++u) {
-        const int k = k0 + u * NT;
-        if (k < span) {
-          xv[u] = xc[S0 + k];
-          xk[u] = xi[S0 + k];
-          mk_[u] = mt[S0 + k];
+        for (int u = 0; u < GU; ++u) {
+          const int k = k0 + u * step;
+          if (k < n) {
+            xv[u] = xc[S0 + k];
+            xk[u] = xi[S0 + k];
+            mk_[u] = mt[S0 + k];
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < GU; ++u) {
+          const int k = k0 + u * step;
+          if (k < n) {
+            cpx<R> v = vin<R>(xv[u]);
+            if (CONJ) v = conjg(v);
+            a[(r < 0 ? row_of<T>(s_off, S0 + k) : r) * LD + xk[u]] = beta[mk_[u] * 3 + c] * v;
+          }
         }
       }
-#pragma unroll
-      for (int u = 0; u < kGU; ++u) {
-        const int k = k0 + u * NT;
-        if (k < span) {
-          cpx<R> v = vin<R>(xv[u]);
-          if (CONJ) v = conjg(v);
-          a[row_of<T>(s_off, S0 + k) * LD + xk[u]] = beta[mk_[u] * 3 + c] * v;
-        }
-      }
+    };
+    if constexpr (kRowsF<R, M>) {
+      for (int r = wid; r < T && wid < NT / 32; r += NT / 32)
+        gather(std::integral_constant<int, kGR<M>>(), s_off[r], (int)(s_off[r + 1] - s_off[r]), lane, 32, r);
+    } else {
+      gather(std::integral_constant<int, 4>(), s_off[0], (int)(s_off[T] - s_off[0]), threadIdx.x, NT, -1);
     }
   }
   __syncthreads();
@@ -1001,12 +1026,20 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, 3, (M1 *
     for (int k2 = 0; k2 < M2; ++k2) at[k1 + M1 * k2] = u[k2];
   }
   __syncthreads();
-  // row tt of the block is row s_row[tt] of B1
-  cpx<R>* out = B1 + (long long)cc * nrows * M;
-  const int nel = min(T, nr - r0) * M;
-  for (int idx = threadIdx.x; idx < nel; idx += NT) {
-    const int tt = idx / M, m = idx - tt * M;
-    out[(long long)s_row[tt] * M + m] = a[tt * LD + m];
+  // row r of the block is row s_row[r] of B1
+  if constexpr (kRowsF<R, M>) {
+    for (int r = wid; r < min(T, nr - r0) && wid < NT / 32; r += NT / 32) {
+      cpx<R>* out = B1 + ((long long)cc * nrows + s_row[r]) * M;
+#pragma unroll 4
+      for (int m = lane; m < M; m += 32) out[m] = a[r * LD + m];
+    }
+  } else {
+    cpx<R>* out = B1 + (long long)cc * nrows * M;
+    const int nel = min(T, nr - r0) * M;
+    for (int idx = threadIdx.x; idx < nel; idx += NT) {
+      const int r = idx / M, m = idx - r * M;
+      out[(long long)s_row[r] * M + m] = a[r * LD + m];
+    }
   }
 }
 
@@ -1022,14 +1055,9 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, 3, (M1 *
 // dipoles; the long lines stage up to 384 (about the mean of the 536^3
 // sphere's 4-row tiles) and read the rest directly
 template <int M> constexpr int kXRow = (M + 1) / 2 < 384 ? (M + 1) / 2 : 384;
-// blocks per SM the x inverse pass's launch bound asks for: four in
-// complex64 (at 270 points 56 registers, no spill: P5 of the 134^3 sphere
-// 59 -> 55 us), three in the wider arithmetic and from 290 points (eight rows,
-// 20 and more elements a thread: 512 points 380 us with three, 475 with two)
-template <typename R, int M> constexpr int kXinvB = (sizeof(R) == 4 && (M < 290 || M >= 1000)) ? 4 : 3;
 
 template <typename R, int M1, int M2, int T, bool CONJ>
-__global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, kXinvB<R, M1 * M2>, (M1 * M2 + T * kLD<M1 * M2>) * sizeof(cpx<R>) + T * kXRow<M1 * M2> * sizeof(typename VecOf<R>::type))) fk_xinv(const cpx<R>* __restrict__ B1,
+__global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, kXB<R, M1 * M2>, (M1 * M2 + T * kLD<M1 * M2>) * sizeof(cpx<R>) + T * kXRow<M1 * M2> * sizeof(typename VecOf<R>::type))) fk_xinv(const cpx<R>* __restrict__ B1,
                                                           const typename VecOf<R>::type* __restrict__ x,
                                                           typename VecOf<R>::type* __restrict__ y,
                                                           LatticeDev lat,
@@ -1038,7 +1066,7 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, kXinvB<R
                                                           const cpx<R>* __restrict__ tw,
                                                           double* __restrict__ dotp, int bstride,
                                                           const int* __restrict__ skip) {
-  constexpr int M = M1 * M2, NT = T * kQ<M1, M2>, LD = kLD<M>, kXS = T * kXRow<M>, kGU = kGUI<M1 * M2>;
+  constexpr int M = M1 * M2, NT = T * kQ<M1, M2>, LD = kLD<M>, kXS = T * kXRow<M>;
   using V = typename VecOf<R>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ long long s_off[T + 1];
@@ -1065,12 +1093,12 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, kXinvB<R
     runs = lat.arow[r0 + rows - 1] - rb != rows - 1;
   }
   const cpx<R>* in = B1 + (long long)cc * nrows * M;
-  for (int idx = threadIdx.x; idx < T * M; idx += NT) {
-    const int tt = idx / M, m = idx - tt * M;
-    const bool ok = tt < rows;
-    const long long row = runs ? (ok ? lat.arow[r0 + tt] : 0) : rb + tt;
-    cp_async_elem<sizeof(cpx<R>)>(a + tt * LD + m, ok ? (const void*)(in + row * M + m) : (const void*)B1,
-                                  ok);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int r = wid; r < T && wid < NT / 32; r += NT / 32) {
+    const bool ok = r < rows;
+    const cpx<R>* src = in + (runs ? (ok ? lat.arow[r0 + r] : 0) : (long long)(ok ? rb + r : 0)) * M;
+#pragma unroll 4
+    for (int m = lane; m < M; m += 32) cp_async_elem<sizeof(cpx<R>)>(a + r * LD + m, src + m, ok);
   }
   const V* xc = x + (long long)cc * n_occ;
   V* yc = y + (long long)cc * n_occ;
@@ -1111,7 +1139,6 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, kXinvB<R
   }
   __syncthreads();
   constexpr int NW = (NT + 31) / 32;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   // partial x^T y (bilinear) when dotp is set: per thread and per warp in
   // the arithmetic's precision (FP32 for complex64: no FP64 work per
   // element), across warps in FP64
@@ -1119,32 +1146,43 @@ __global__ void __launch_bounds__(T * kQ<M1, M2>, kMinB(T * kQ<M1, M2>, kXinvB<R
   {
     const uint16_t* __restrict__ xi = lat.xi;
     const uint8_t* __restrict__ mt = lat.mat;
-    for (int k0 = threadIdx.x; k0 < span; k0 += kGU * NT) {
-      int xk[kGU], mk_[kGU];
+    // dipoles k0, k0 + step, ... below e of the block, in row r (searched for when
+    // r < 0)
+    auto scatter = [&](auto gu, int e, int k0, int step, int r) {
+      constexpr int GU = decltype(gu)::value;
+      for (; k0 < e; k0 += GU * step) {
+        int xk[GU], mk_[GU];
 #pragma unroll
-      for (int u2 = 0; u2 < kGU; ++u2) {
-        const int k = k0 + u2 * NT;
-        if (k < span) {
-          xk[u2] = xi[S0 + k];
-          mk_[u2] = mt[S0 + k];
+        for (int u2 = 0; u2 < GU; ++u2) {
+          const int k = k0 + u2 * step;
+          if (k < e) {
+            xk[u2] = xi[S0 + k];
+            mk_[u2] = mt[S0 + k];
+          }
         }
-      }
 #pragma unroll
-      for (int u2 = 0; u2 < kGU; ++u2) {
-        const int k = k0 + u2 * NT;
-        if (k < span) {
-          const cpx<R> xv = vin<R>(k < kXS ? s_x[k] : xc[S0 + k]);
-          cpx<R> v = xv;
-          if (CONJ) v = conjg(v);
-          cpx<R> o = cnmac(v, beta[mk_[u2] * 3 + c], a[row_of<T>(s_off, S0 + k) * LD + xk[u2]]);
-          if (CONJ) o = conjg(o);
-          yc[S0 + k] = vstore(o);
-          if (dotp) {
-            tr = tr + (xv.x * o.x - xv.y * o.y);
-            ti = ti + (xv.x * o.y + xv.y * o.x);
+        for (int u2 = 0; u2 < GU; ++u2) {
+          const int k = k0 + u2 * step;
+          if (k < e) {
+            const cpx<R> xv = vin<R>(k < kXS ? s_x[k] : xc[S0 + k]);
+            cpx<R> v = xv;
+            if (CONJ) v = conjg(v);
+            cpx<R> o = cnmac(v, beta[mk_[u2] * 3 + c], a[(r < 0 ? row_of<T>(s_off, S0 + k) : r) * LD + xk[u2]]);
+            if (CONJ) o = conjg(o);
+            yc[S0 + k] = vstore(o);
+            if (dotp) {
+              tr = tr + (xv.x * o.x - xv.y * o.y);
+              ti = ti + (xv.x * o.y + xv.y * o.x);
+            }
           }
         }
       }
+    };
+    if constexpr (kRowsI<R, M>) {
+      for (int r = wid; r < T && wid < NT / 32; r += NT / 32)
+        scatter(std::integral_constant<int, kGR<M>>(), (int)(s_off[r + 1] - S0), (int)(s_off[r] - S0) + lane, 32, r);
+    } else {
+      scatter(std::integral_constant<int, 4>(), span, threadIdx.x, NT, -1);
     }
   }
   if (dotp) {
