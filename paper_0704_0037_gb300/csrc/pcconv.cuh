@@ -464,8 +464,12 @@ __global__ void __launch_bounds__(128) k_conv_f32(ConvIn in, const float* __rest
   using T = Tile<K, ZW>;
   constexpr int K3 = K * K * K, CB = 8, NB = 8, NV = (T::HV + 127) / 128;
   static_assert(CO * (4 / ZW) == NB, "8 channels per block");
-  __shared__ __align__(16) float s_in[2][CB][T::HV];
-  __shared__ __align__(16) float s_w[2][CB][K3][NB];
+  // rows in x are 24 floats apart, two channels to a row: the four rows of a warp
+  // fill the 32 banks.  The weights of a warp's CO channels lie together, tap by
+  // tap, so that 16 bytes are one tap of 4 channels or two taps of 2.
+  constexpr int P = 24, PV = T::HY * T::HZ * P, KP = K3 + 1;
+  __shared__ __align__(16) float s_in[2][CB / 2][PV];
+  __shared__ __align__(16) float s_w[2][CB][NB / CO][KP * CO];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int wz = warp % ZW, cg = warp / ZW;
   const int ntx = (d.x + 7) / 8, nty = (d.y + 3) / 4;
@@ -497,15 +501,24 @@ __global__ void __launch_bounds__(128) k_conv_f32(ConvIn in, const float* __rest
 #pragma unroll
         for (int c = 0; c < CB; ++c) {
           const bool ok = v >= 0 && c < lim;
-          cp4(&s_in[b][c][hv], ok ? src + c * cs + v : in.a, ok);
+          cp4(&s_in[b][c >> 1][(hv / T::HX) * P + hv % T::HX + (c & 1) * (P / 2)], ok ? src + c * cs + v : in.a, ok);
         }
       }
     }
     const int nc = min(CB, cin - c0);
     for (int i = threadIdx.x; i < nc * K3 * 2; i += 128) {           // 16-byte pieces
-      const unsigned sa = (unsigned)__cvta_generic_to_shared(&s_w[b][0][0][0] + 4 * i);
-      const float* g = wf + ((long long)c0 * K3 + (i >> 1)) * coutp + co0 + 4 * (i & 1);
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(g) : "memory");
+      const int h = i & 1, c = (i >> 1) / K3, t = (i >> 1) - c * K3;
+      const float* g = wf + ((long long)c0 * K3 + (i >> 1)) * coutp + co0 + 4 * h;
+      if constexpr (CO == 2) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const unsigned sa = (unsigned)__cvta_generic_to_shared(&s_w[b][c][2 * h + e][t * CO]);
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(g + 2 * e) : "memory");
+        }
+      } else {
+        const unsigned sa = (unsigned)__cvta_generic_to_shared(CO == 4 ? &s_w[b][c][h][t * CO] : &s_w[b][c][0][t * CO + 4 * h]);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(g) : "memory");
+      }
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
   };
@@ -523,7 +536,7 @@ __global__ void __launch_bounds__(128) k_conv_f32(ConvIn in, const float* __rest
 #pragma unroll
     for (int k = 0; k < CO / 2; ++k) acc2[k] = pair2(acc[2 * k], acc[2 * k + 1]);
   }
-  const int hv0 = (wz * T::HY + (lane >> 3)) * T::HX + (lane & 7);
+  const int hv0 = (wz * T::HY + (lane >> 3)) * P + (lane & 7);
   fetch(0);
   for (int blk = 0; blk < nblk; ++blk) {
     __syncthreads();                         // the sums over the buffer fetched next are done
@@ -537,19 +550,22 @@ __global__ void __launch_bounds__(128) k_conv_f32(ConvIn in, const float* __rest
     const int nc = min(CB, cin - blk * CB), b = blk & 1;
 #pragma unroll 1
     for (int c = 0; c < nc; ++c) {
-      const float* si = &s_in[b][c][hv0];
-      const float* sw = &s_w[b][c][0][cg * CO];
+      const float* si = &s_in[b][c >> 1][hv0 + (c & 1) * (P / 2)];
+      const float* sw = &s_w[b][c][cg][0];
+      float4 w2 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
       for (int t = 0; t < K3; ++t) {
-        const float v = si[((t / (K * K)) * T::HY + (t / K) % K) * T::HX + t % K];
+        const float v = si[((t / (K * K)) * T::HY + (t / K) % K) * P + t % K];
         if constexpr (PAIRS) {
           const unsigned long long vv = pair2(v, v);
-          const unsigned long long* w = reinterpret_cast<const unsigned long long*>(sw + t * NB);
+          const unsigned long long* w = reinterpret_cast<const unsigned long long*>(sw + t * CO);
 #pragma unroll
           for (int k = 0; k < CO / 2; ++k) fma2(acc2[k], w[k], vv);
         } else {
+          if (CO == 4 || t % 2 == 0) w2 = *reinterpret_cast<const float4*>(sw + t * CO);
+          const float w[4] = {w2.x, w2.y, w2.z, w2.w};
 #pragma unroll
-          for (int k = 0; k < CO; ++k) acc[k] = fmaf(sw[t * NB + k], v, acc[k]);
+          for (int k = 0; k < CO; ++k) acc[k] = fmaf(w[CO == 2 && t % 2 ? 2 + k : k], v, acc[k]);
         }
       }
     }
