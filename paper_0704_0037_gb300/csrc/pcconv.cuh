@@ -433,7 +433,7 @@ inline cudaError_t conv_mma(int K, const SplitIn& in, const uint2* wp, const flo
 // Pairs of outputs run in the paired instruction (each half rounds as the
 // scalar one).  On small lattices a sum is one long dependent chain: what
 // helps is every SM busy, operands copied ahead and few instructions per tap.
-// 64 x 45 x 37 ellipsoid: training step 2.60 -> 0.85 ms, same bits.
+// 64 x 45 x 37 ellipsoid: training step 2.60 -> 0.82 ms, same bits.
 
 // a thread's CO outputs at one voxel, pairwise
 __device__ __forceinline__ unsigned long long pair2(float a, float b) {
@@ -622,8 +622,8 @@ cudaError_t conv_f32_t(const ConvIn& in, const float* wf, const float* bias, con
 
 // 128, 64 or 32 voxels per block: the least rounds of blocks over the SMs
 // times instructions per tap (8, 5.5 and 4.5 with their loads).  Of the layers
-// at 1/4 and 1/8 resolution, 33 us with the 64-voxel tile this picks and 46 with
-// the 32-voxel one (both under one round).
+// at 1/4 and 1/8 resolution, 31 us with the 64-voxel tile this picks and 42 with
+// the 32-voxel one (one round of blocks against two).
 inline cudaError_t conv_f32(int K, const ConvIn& in, const float* wf, const float* bias, const float* mask,
                             float* out, int cout, Dims d, int relu, cudaStream_t st) {
   if (K == 1) return conv_f32_t<1, 1, 2>(in, wf, bias, mask, out, cout, d, relu, st);
