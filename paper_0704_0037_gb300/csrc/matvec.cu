@@ -540,9 +540,12 @@ cudaError_t tune_tiles(Geom& g, const LatticeDev& lat, Work<R>& w, cudaStream_t 
   std::array<int, 3> best{0, 0, 0};
   for (int pass = 0; pass < 3 && e == cudaSuccess; ++pass) {
     if (!has(pass == 1 ? g.Mz : g.My)) continue;       // one variant, or the Stockham passes
-    // the variants in turn, the least of three times two launches: a clock that
-    // still rises while the first is timed would favour the second (half tiles
-    // were chosen for double-float y passes that take 1.4 times as long on them)
+    // the variants in turn, the least of three times two launches (six where a
+    // launch is a few microseconds, not far from an event's own time): a clock
+    // that still rises while the first is timed would favour the second (half
+    // tiles were chosen for double-float y passes that take 1.4 times as long on
+    // them)
+    const int reps = (long long)g.Mx * g.My * g.Mz <= (1LL << 20) ? 6 : 2;
     float least[2] = {0.f, 0.f};
     for (int round = 0; round < 4 && e == cudaSuccess; ++round) {
       for (int var = 0; var < 2 && e == cudaSuccess; ++var) {
@@ -556,7 +559,7 @@ cudaError_t tune_tiles(Geom& g, const LatticeDev& lat, Work<R>& w, cudaStream_t 
           continue;
         }
         if ((e = cudaEventRecord(e0, st)) != cudaSuccess) break;
-        for (int r = 0; r < 2 && e == cudaSuccess; ++r) e = fast_pass<R>(M, op, a);
+        for (int r = 0; r < reps && e == cudaSuccess; ++r) e = fast_pass<R>(M, op, a);
         if (e != cudaSuccess) break;
         if ((e = cudaEventRecord(e1, st)) != cudaSuccess) break;
         if ((e = cudaEventSynchronize(e1)) != cudaSuccess) break;
