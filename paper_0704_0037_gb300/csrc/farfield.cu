@@ -54,7 +54,6 @@ constexpr int kDirs = 32;         // directions per tile
 constexpr int kJMax = 72;         // folded cells per chunk: 2 * 72 = 144 inner columns
 constexpr int kNT = 128;          // threads
 constexpr int kBBlk = kSl * 1024; // bytes of one 16-column step of a direction tile
-constexpr int kFix = 54;          // |value| <= 2^54 in fixed point
 
 // inner dimension: H = ceil(nx / 2) folded cells in nchunk chunks of J, each
 // ks steps of 16 columns (2 J padded with zeros)
@@ -74,7 +73,7 @@ __device__ __forceinline__ unsigned pack2(int a, int b) {
   const __nv_bfloat162 v = __floats2bfloat162_rn((float)a, (float)b);
   return *reinterpret_cast<const unsigned*>(&v);
 }
-// v 2^(kFix - e) rounded to an integer, for |v| <= 2^e and e >= -900, in integer
+// v 2^(54 - e) rounded to an integer, for |v| <= 2^e and e >= -900, in integer
 // instructions (the FP64 pipe is the busiest one): the mantissa shifted by the
 // difference of the exponents
 __device__ __forceinline__ long long to_fixed(double v, int e) {
