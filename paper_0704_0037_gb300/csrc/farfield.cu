@@ -48,16 +48,8 @@
 namespace dda {
 namespace {
 
-constexpr int kSl = 7;            // digits per number
-constexpr int kRows = 8;          // lattice rows per block
-constexpr int kDirs = 32;         // directions per tile
-constexpr int kJMax = 72;         // folded cells per chunk: 2 * 72 = 144 inner columns
+constexpr int kSl = kFfSl, kRows = kFfRows, kDirs = kFfDirs, kJMax = kFfJMax, kBBlk = kFfBBlk;
 constexpr int kNT = 128;          // threads
-constexpr int kBBlk = kSl * 1024; // bytes of one 16-column step of a direction tile
-
-// inner dimension: H = ceil(nx / 2) folded cells in nchunk chunks of J, each
-// ks steps of 16 columns (2 J padded with zeros)
-struct FfShape { int H, J, nchunk, ks; };
 
 // t = sum of dg[i] 256^(6 - i), -128 <= dg[i] <= 127 for i > 0
 __device__ __forceinline__ void digits(long long t, int (&dg)[kSl]) {
@@ -368,41 +360,13 @@ __global__ void __launch_bounds__(384) k_ff_fin(const double* __restrict__ part,
   }
 }
 
-FfShape ff_shape(int nx) {
-  FfShape s;
-  s.H = (nx + 1) / 2;
-  s.nchunk = (s.H + kJMax - 1) / kJMax;
-  s.J = (s.H + s.nchunk - 1) / s.nchunk;
-  s.ks = (2 * s.J + 15) / 16;
-  return s;
-}
-
-// row blocks in flight: two blocks per SM, no more than there are units, and
-// partial sums of at most 64 MB
-int ff_groups(int units, int n_dir) {
-  const long long fit = std::max(1LL, (64LL << 20) / (48LL * n_dir));
-  return (int)std::min<long long>(std::min(units, 2 * num_sms()), fit);
-}
-
-size_t up256(size_t b) { return (b + 255) / 256 * 256; }
-
 }  // namespace
-
-FarfieldPlan farfield_plan(int n_dir, int nx, int ny, int nz, int nr) {
-  const FfShape s = ff_shape(nx);
-  const int nt = (n_dir + kDirs - 1) / kDirs;
-  const int units = ((nr + kRows - 1) / kRows) * s.nchunk;
-  FarfieldPlan p;
-  p.tab = up256((size_t)n_dir * (nx + ny + nz) * sizeof(c128));
-  p.pack = (size_t)s.nchunk * nt * s.ks * kBBlk;
-  p.part = up256((size_t)ff_groups(units, n_dir) * n_dir * 6 * sizeof(double));
-  return p;
-}
 
 cudaError_t farfield_tables(void* ws, const double* dirs, int n_dir, double kd, int nx, int ny, int nz,
                             const FarfieldPlan& p, cudaStream_t st) {
+  if (n_dir > p.cap) return cudaErrorInvalidValue;         // the workspace is p's
   const FfShape s = ff_shape(nx);
-  const int nt = (n_dir + kDirs - 1) / kDirs;
+  const int nt = ff_tiles(n_dir);
   c128* tab = (c128*)ws;
   unsigned* pack = (unsigned*)((unsigned char*)ws + p.tab);
   const long long tt = (long long)n_dir * ((nx + 1) / 2 + (ny + 1) / 2 + (nz + 1) / 2), tp = (long long)s.nchunk * nt * s.ks * 256;
@@ -417,9 +381,8 @@ cudaError_t farfield_sums(void* ws, const c128* P, const LatticeDev& lat, const 
                           double kd, int nx, int ny, int nr, long long n_occ, const FarfieldPlan& p,
                           double* F, cudaStream_t st) {
   const FfShape s = ff_shape(nx);
-  const int nt = (n_dir + kDirs - 1) / kDirs;
-  const int units = ((nr + kRows - 1) / kRows) * s.nchunk;
-  const int G = ff_groups(units, n_dir);
+  const int nt = ff_tiles(n_dir), units = ff_units(s, nr), G = p.groups;
+  if (n_dir > p.cap || G > units) return cudaErrorInvalidValue;
   const c128* tab = (const c128*)ws;
   const unsigned char* pack = (const unsigned char*)ws + p.tab;
   double* part = (double*)((unsigned char*)ws + p.tab + p.pack);

@@ -9,6 +9,7 @@
 
 #include "../../include/dda.h"
 #include "common.cuh"
+#include "farfield_plan.h"
 #include "fft.cuh"
 
 namespace dda {
@@ -255,15 +256,9 @@ long long launch_total();
 }  // namespace dda
 
 namespace dda {
-// Far-field sums of dda_scatter (farfield.cu): workspace of one call for n_dir
-// directions on a lattice of nx x ny x nz cells with nr rows (phase tables,
-// their digits, partial sums), the direction tables, and the amplitudes F
-// [n_dir][6] of one polarization P from them.
-struct FarfieldPlan {
-  size_t tab, pack, part;
-  size_t bytes() const { return tab + pack + part; }
-};
-FarfieldPlan farfield_plan(int n_dir, int nx, int ny, int nz, int nr);
+// Far-field sums of dda_scatter (farfield.cu) in a workspace of plan p: the
+// tables of n_dir <= p.cap directions, and from them the amplitudes F [n_dir][6]
+// of one polarization P.
 cudaError_t farfield_tables(void* ws, const double* dirs, int n_dir, double kd, int nx, int ny, int nz,
                             const FarfieldPlan& p, cudaStream_t st);
 cudaError_t farfield_sums(void* ws, const c128* P, const LatticeDev& lat, const double* dirs, int n_dir,

@@ -288,7 +288,7 @@ int dda_scatter_internal(dda_t h, int presc, const void* P_dev, int nrhs, const 
   const int fnr = flat.arow ? flat.nact : fnrows;
   const int nblk = n_dir > 0 ? (n_dir + kDirBlock - 1) / kDirBlock : 0;
   FarfieldPlan plan{};
-  if (n_dir > 0) plan = farfield_plan(std::min(n_dir, kDirBlock), fnx, fny, fnz, fnr);
+  if (n_dir > 0) plan = farfield_plan(std::min(n_dir, kDirBlock), fnx, fny, fnz, fnr, num_sms());
   const size_t tab_b = plan.bytes() + (size_t)Lq * sizeof(c128);
   const size_t fp_b = (size_t)2 * qblocks * sizeof(double) + (size_t)n_dir * 9 * sizeof(double) +
                       3 * sizeof(double);
@@ -310,8 +310,7 @@ int dda_scatter_internal(dda_t h, int presc, const void* P_dev, int nrhs, const 
   double* d_qdir = d_dirs + 3 * (size_t)n_dir;
   auto tables = [&](int b) -> cudaError_t {
     const int d0 = b * kDirBlock, nd = std::min(n_dir - d0, kDirBlock);
-    return farfield_tables(ws, d_dirs + 3 * (size_t)d0, nd, h->kd, fnx, fny, fnz,
-                           farfield_plan(nd, fnx, fny, fnz, fnr), st);
+    return farfield_tables(ws, d_dirs + 3 * (size_t)d0, nd, h->kd, fnx, fny, fnz, plan, st);
   };
   if (n_dir > 0) {
     DDA_CK(h, cudaMemcpyAsync(d_dirs, dirs, (size_t)n_dir * 3 * sizeof(double), cudaMemcpyHostToDevice, st));
@@ -335,8 +334,8 @@ int dda_scatter_internal(dda_t h, int presc, const void* P_dev, int nrhs, const 
       for (int b = 0; b < nblk; ++b) {
         const int d0 = b * kDirBlock, nd = std::min(n_dir - d0, kDirBlock);
         if (nblk > 1) DDA_CK(h, tables(b));
-        DDA_CK(h, farfield_sums(ws, Pf, flat, d_dirs + 3 * (size_t)d0, nd, h->kd, fnx, fny, fnr, fnocc,
-                                farfield_plan(nd, fnx, fny, fnz, fnr), d_F + 6 * (size_t)d0, st));
+        DDA_CK(h, farfield_sums(ws, Pf, flat, d_dirs + 3 * (size_t)d0, nd, h->kd, fnx, fny, fnr, fnocc, plan,
+                                d_F + 6 * (size_t)d0, st));
       }
       tr_end(g.tr, st, TR_FARFIELD);
       DDA_CK(h, cudaMemcpyAsync(F_out + (size_t)r * n_dir * 6, d_F, (size_t)n_dir * 6 * sizeof(double),

@@ -1,7 +1,9 @@
 """GPU parity of the far-field sums (exact digit products on the tensor cores)
 with the oracle's direct sum, at the edges of their tiles: folded rows of one
 cell, odd and even lengths, one and several inner chunks (72 folded cells
-each), row blocks of 16 that are partly filled, and direction tiles of 32.
+each), row blocks of 8 that are partly filled, lattices with more row blocks
+than run at once, direction tiles of 32, and calls whose directions are taken in
+several blocks of 8,192.
 
 Tolerance: both sides evaluate the phases in FP64 (|phase| <= kd n: relative
 error of a sum a few 1e-16 times kd n) and sum at FP64 accuracy: 1e-13 of the
@@ -20,6 +22,9 @@ CASES = [  # nx, ny, nz, fill (0: full box), directions
     (1, 1, 1, 0, 1), (2, 1, 3, 0, 31), (5, 4, 4, 0, 32), (16, 3, 6, 0.4, 33), (15, 7, 5, 0.5, 64),
     (143, 3, 2, 0.7, 40), (144, 2, 3, 0, 5), (145, 3, 3, 0.3, 70), (300, 2, 2, 0.6, 45),
     (9, 33, 17, 0.2, 130),
+    # more than 2 x 152 row blocks: a block's sums carried over several of them,
+    # with one inner chunk and with two
+    (6, 70, 70, 0, 34), (150, 50, 50, 0, 36),
 ]
 
 
@@ -56,3 +61,27 @@ def test_farfield_nonfinite_input_stays_nonfinite():
         F, q = dda.dda_scatter(p.h, dda.DDA_LDR, torch.from_numpy(x).cuda(), [[0.0, 0.0, 1.0]],
                                [[1.0, 0.0, 0.0]], inputs.random_unit_vectors(1, 9))
         assert not np.isfinite(F).any() and not np.isfinite(q[0, 0])
+
+
+def test_farfield_of_several_direction_blocks():
+    """16,368 directions (8,192 + 8,176: a last block for which a plan of its own
+    would not have fitted the first one's workspace) against the oracle at
+    directions of both blocks, and against calls of one block."""
+    torch, dda = need_gpu()
+    nx, ny, nz, n_dir = 6, 70, 70, 16368
+    occ = inputs.cube(nx, ny, nz)
+    pos = lattice.positions(occ > 0)
+    prop, pol = [[0.0, 0.0, 1.0]] * 2, [[1.0, 0.0, 0.0], [0.0, 1.0, 0.0]]
+    dirs = inputs.random_unit_vectors(7, n_dir)
+    with dda.Particle(occ, [1.4 + 0.05j], 0.2) as p:
+        x = inputs.random_vectors(3, 2, p.n_occ)
+        P = torch.from_numpy(x).cuda()
+        F, q = dda.dda_scatter(p.h, dda.DDA_LDR, P, prop, pol, dirs)
+        pick = [0, 31, 4095, 8191, 8192, 8193, 12000, n_dir - 1]
+        for r in range(2):
+            ref = observables.farfield(x[r], pos, p.kd, dirs[pick])
+            assert np.abs(F[r][pick] - ref).max() <= 1e-13 * np.abs(ref).max()
+        for d0, d1 in ((0, 8192), (8192, n_dir), (5000, 9000)):
+            part, q1 = dda.dda_scatter(p.h, dda.DDA_LDR, P, prop, pol, dirs[d0:d1])
+            assert np.abs(part - F[:, d0:d1]).max() <= 1e-13 * np.abs(F).max()
+            assert np.array_equal(q[:, :2], q1[:, :2])      # Q sums: their table lies behind the plan
