@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(kXYT, 4) fk_yx_inv(const c64* __restrict__ B2,
         const int k = k0 + u * kRL;
         if (k < n) {
           const c64 v = CONJ ? conjg(xv[u]) : xv[u];
-          c64 o = cnmac(v, beta[mk_[u] * 3 + c], m.P[r * m.ld + xk[u]]);
+          c64 o = v - beta[mk_[u] * 3 + c] * m.P[r * m.ld + xk[u]];
           if (CONJ) o = conjg(o);
           yc[S0 + k] = o;
           tr = tr + (xv[u].x * o.x - xv[u].y * o.y);
