@@ -18,18 +18,21 @@
 // numbers of 55 bits, relative to the largest entry of their (lattice row,
 // component) and to 1, cut into seven signed 8-bit digits that bf16 holds
 // exactly; the products of digits i and j with i + j = g go to accumulator g
-// (28 of the 49 pairs, g <= 6: what is left out lies below 2^-53 of the
-// row's scale).  A product of two digits is at most 2^14 and accumulator g
-// adds at most (g + 1) K <= 7 * 144 of them, below 2^24: every FP32 sum of the
-// tensor cores is exact.  The seven accumulators are put together in 64-bit
-// integers; FP64 work is left only for the (y, z) phase of each row.
+// (34 of the 49 pairs, g <= 7).  What is left out is 2^-59 of the row's scale
+// for digits of any value, 2^-52.5 if all were largest and of one sign; without
+// g = 7 (28 pairs) it was 2^-51 and 2^-44, as large as the roundings of the
+// phases (error on random fields 1.1 to 1.25 times the direct sums').  A product
+// of two digits is at most 2^14 and an accumulator adds at most 7 K <= 7 * 144 of
+// them, below 2^24: every FP32 sum of the tensor cores is exact.  The eight
+// accumulators are put together in 64-bit integers; FP64 work is left only for
+// the (y, z) phase of each row.
 //
 // One block holds the digits of 8 lattice rows (48 matrix rows, up to 144
 // inner columns: 97 KB) in shared memory, in the order the tensor-core
 // fragments are loaded, and runs all directions past them in tiles of 32.  Each
 // of 4 warps takes 8 directions, whose digits it streams from L2 in fragment
 // order, against the three tiles of 16 matrix rows (8 lattice rows, real and
-// imaginary part, of one component): 84 matrix instructions for 28 fragment
+// imaginary part, of one component): 102 matrix instructions for 28 fragment
 // loads.  The warps meet only when the digits of the next rows are made, and
 // two blocks share an SM, so that one warp's sums (FP64 and integer pipes)
 // overlap another's products (tensor pipe).
@@ -37,8 +40,7 @@
 // 128^3 sphere, 1,152 directions, per right-hand side: direct FP64 sums 65.4 ms;
 // this product with 16 rows and 12 warps in one block per SM 3.26 ms, with two
 // blocks and integer scaling 2.58 ms; digits made in integer instructions 2.31 ms;
-// warps that meet only once per row block 2.0 ms; error
-// against 64-bit sums 2.0e-15 before, 1.9e-15 now.
+// warps that meet only once per row block 2.0 ms; with the pairs i + j = 7 2.2 ms.
 #include <algorithm>
 
 #include "internal.h"
@@ -259,11 +261,11 @@ __global__ void __launch_bounds__(kNT, 2)
       const bool mine = (lane & 4) == 0 && d < n_dir;
       double old[3] = {0.0, 0.0, 0.0};
       if (mine && u != (int)blockIdx.x) { old[0] = o[0]; old[1] = o[2]; old[2] = o[4]; }
-      float acc[3][kSl][4];
+      float acc[3][kSl + 1][4];
 #pragma unroll
       for (int n = 0; n < 3; ++n)
 #pragma unroll
-        for (int k = 0; k < kSl; ++k)
+        for (int k = 0; k <= kSl; ++k)
 #pragma unroll
           for (int v = 0; v < 4; ++v) acc[n][k][v] = 0.0f;
       for (int s = 0; s < sh.ks; ++s, ++q) {
@@ -283,7 +285,7 @@ __global__ void __launch_bounds__(kNT, 2)
 #pragma unroll
         for (int i = 0; i < kSl; ++i)
 #pragma unroll
-          for (int j = 0; j < kSl - i; ++j)
+          for (int j = 0; j < (i ? kSl + 1 - i : kSl); ++j)
 #pragma unroll
             for (int c = 0; c < 3; ++c) mma(acc[c][i + j], af[c][i], bf[j].x, bf[j].y);
       }
@@ -301,7 +303,9 @@ __global__ void __launch_bounds__(kNT, 2)
             long long t = __float2int_rn(acc[c][0][2 * im + col]);
 #pragma unroll
             for (int k = 1; k < kSl - 1; ++k) t = t * 256 + __float2int_rn(acc[c][k][2 * im + col]);
-            t = t * 16 + (__float2int_rn(acc[c][kSl - 1][2 * im + col]) >> 4);
+            const int last = __float2int_rn(acc[c][kSl - 1][2 * im + col]) +
+                             (__float2int_rn(acc[c][kSl][2 * im + col]) >> 8);
+            t = t * 16 + ((last + 8) >> 4);
             z[im] = e3[c] == kBad ? nan("") : scaled(t, e3[c]);
           }
           v[c][col][0] = z[0] * w.x - z[1] * w.y;

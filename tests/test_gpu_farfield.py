@@ -85,3 +85,25 @@ def test_farfield_of_several_direction_blocks():
             part, q1 = dda.dda_scatter(p.h, dda.DDA_LDR, P, prop, pol, dirs[d0:d1])
             assert np.abs(part - F[:, d0:d1]).max() <= 1e-13 * np.abs(F).max()
             assert np.array_equal(q[:, :2], q1[:, :2])      # Q sums: their table lies behind the plan
+
+
+@pytest.mark.parametrize("nx", [31, 100, 144])
+def test_farfield_row_is_as_exact_as_its_phases(nx):
+    """One lattice row and directions whose phase arguments are exact in FP64: the
+    error of a sum is that of its cosines and sines, each rounded to at most half
+    a unit of 2^-53 (0.41 2^-53 rms per complex entry), in nx terms of random
+    sign, and of the final roundings: below 0.55 2^-53 sqrt(nx) of the largest
+    entry.  Digit products left out of the sum must not show."""
+    torch, dda = need_gpu()
+    kd, n_dir = 0.125, 96
+    c = np.arange(1, n_dir + 1) / 128.0
+    dirs = np.stack([c, np.zeros(n_dir), np.sqrt(1.0 - c * c)], axis=1)
+    rng = np.random.default_rng(1)
+    x = rng.uniform(-1, 1, (1, 3, nx)) + 1j * rng.uniform(-1, 1, (1, 3, nx))
+    with dda.Particle(inputs.cube(nx, 1, 1), [1.4], kd) as p:
+        F, _ = dda.dda_scatter(p.h, dda.DDA_LDR, torch.from_numpy(x).cuda(), [[0.0, 0.0, 1.0]],
+                               [[1.0, 0.0, 0.0]], dirs)
+    ph = np.outer(kd * c, np.arange(nx) - 0.5 * (nx - 1)).astype(np.longdouble)
+    ref = -1j * np.longdouble(kd) ** 3 * ((np.cos(ph) - 1j * np.sin(ph)) @ x[0, 1].astype(np.clongdouble))
+    err = np.abs(F.reshape(n_dir, 3)[:, 1] - ref).astype(float) / kd ** 3      # y: no projection
+    assert np.sqrt((err ** 2).mean()) <= 0.55 * 2.0 ** -53 * np.sqrt(nx) * np.abs(x).max()
