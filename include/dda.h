@@ -329,7 +329,7 @@ int dda_residual(dda_t h, int pol_prescription, int nrhs, const double* prop_hos
                  const double* pol_host, const void* P_dev, double* res_out_host);
 
 /*
- * dda_scatter -- scattering quantities of Sec. 3.1 from P (FP64 sums).
+ * dda_scatter -- scattering quantities of Sec. 3.1 from P, at FP64 accuracy.
  *   pol_prescription : the prescription P was computed with (Q_abs needs alpha).
  *   P_dev     : device [nrhs][3][N_occ] complex128.
  *   prop_host, pol_host : as in dda_solve (E_inc for Q_ext, alpha for Q_abs).
@@ -340,6 +340,11 @@ int dda_residual(dda_t h, int pol_prescription, int nrhs, const double* prop_hos
  *                F(n) = -i kd^3 (I - n n) sum_j P_j exp(-i kd n.r_j).
  *   q_out_host : host [nrhs][3] = (Q_ext, Q_abs, Q_sca); Q_sca is NaN without
  *                weights.  x = kd (3 N_occ / (4 pi))^(1/3) normalises Q.
+ * Device memory kept by the handle, for D = min(n_dir, 8192): about
+ * 16 D (nx + ny + nz) + 14 D nx bytes of phase tables and up to 64 MB of partial
+ * sums.  Where that cannot be had (dda_set_memory_limit), D is 512; where that
+ * cannot either, the sums run directly, some 30 times slower at many directions,
+ * in 16 n_dir (nx + ny + nz) bytes and less than 1 MB besides.
  * Synchronises the stream.
  */
 int dda_scatter(dda_t h, int pol_prescription, const void* P_dev, int nrhs,

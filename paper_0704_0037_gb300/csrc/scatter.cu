@@ -166,6 +166,7 @@ struct Wave2 { double a[3]; double e[6]; };
 
 constexpr int kCollapseG = 8;   // y groups of the collapse (partials per (x, z))
 constexpr int kDirBlock = 8192; // directions whose phase tables are held at once
+constexpr int kDirBlockMin = 512;   // and where memory is short
 
 // per-row-chunk partials of sum Im(E_inc^* . P) and sum w |P|^2.  ptab holds
 // exp(-i kd a_mu r_mu) along x, then y, then z (k_phase_tab for the incidence
@@ -283,38 +284,74 @@ int dda_scatter_internal(dda_t h, int presc, const void* P_dev, int nrhs, const 
   }
   const int qblocks = (int)std::min<long long>((g.nrows + 7) / 8, 1024);
   const int Lq = g.nx + g.ny + g.nz;   // incidence phase table of the Q sums
-  // rows of the far-field lattice that can hold dipoles, and its directions
-  // in blocks of at most kDirBlock (bounded phase tables)
+  // rows of the far-field lattice that can hold dipoles; directions go in blocks
+  // of at most kDirBlock (bounded phase tables)
   const int fnr = flat.arow ? flat.nact : fnrows;
-  const int nblk = n_dir > 0 ? (n_dir + kDirBlock - 1) / kDirBlock : 0;
+  // Workspace of the digit products; where it cannot be had (a memory limit, a
+  // full device), that of 512 directions at a time, then that of the direct sums
+  // (phase tables of all directions and partial sums of n_chunks groups of rows)
+  const int dblocks = (n_dir + kDB - 1) / kDB;
+  int n_chunks = 1, rows_per_chunk = fnrows;
+  if (n_dir > 0) {
+    n_chunks = std::max(1, std::min((4 * num_sms() + dblocks - 1) / dblocks, (fnrows + 31) / 32));
+    rows_per_chunk = (fnrows + n_chunks - 1) / n_chunks;
+    n_chunks = (fnrows + rows_per_chunk - 1) / rows_per_chunk;
+  }
   FarfieldPlan plan{};
-  if (n_dir > 0) plan = farfield_plan(std::min(n_dir, kDirBlock), fnx, fny, fnz, fnr, num_sms());
-  const size_t tab_b = plan.bytes() + (size_t)Lq * sizeof(c128);
-  const size_t fp_b = (size_t)2 * qblocks * sizeof(double) + (size_t)n_dir * 9 * sizeof(double) +
-                      3 * sizeof(double);
-  if (h->tab_bytes < tab_b) {
-    dev_free(h->d_tab, h->stream); h->d_tab = nullptr; h->tab_bytes = 0;
-    if (dev_malloc(&h->d_tab, tab_b) != cudaSuccess) { cudaGetLastError(); return dda_fail(h, DDA_ERR_OOM, "scatter tables"); }
-    h->tab_bytes = tab_b;
+  size_t ws_b = 0, part_b = 0;
+  auto reserve = [&](void** buf, size_t* have, size_t need) {
+    if (*have >= need) return true;
+    dev_free(*buf, h->stream);
+    *buf = nullptr;
+    *have = 0;
+    if (dev_malloc(buf, need) != cudaSuccess) { cudaGetLastError(); return false; }
+    *have = need;
+    return true;
+  };
+  auto get = [&](size_t ws, size_t pt) {
+    ws_b = ws;
+    part_b = std::max(pt, (size_t)2 * qblocks * sizeof(double));
+    const size_t tab_b = ws_b + (size_t)Lq * sizeof(c128);
+    const size_t fp_b = part_b + (size_t)n_dir * 9 * sizeof(double) + 3 * sizeof(double);
+    if (!reserve((void**)&h->d_tab, &h->tab_bytes, tab_b)) return false;
+    if (reserve((void**)&h->d_fpart, &h->fpart_bytes, fp_b)) return true;
+    dev_free(h->d_tab, h->stream);             // a smaller plan starts from nothing
+    h->d_tab = nullptr;
+    h->tab_bytes = 0;
+    return false;
+  };
+  auto get_plan = [&](int cap) {
+    plan = farfield_plan(std::min(n_dir, cap), fnx, fny, fnz, fnr, num_sms());
+    return get(plan.bytes(), 0);
+  };
+  bool direct = false;
+  if (n_dir == 0) {
+    if (!get(0, 0)) return dda_fail(h, DDA_ERR_OOM, "scatter tables");
+  } else if (!get_plan(kDirBlock) && !(n_dir > kDirBlockMin && get_plan(kDirBlockMin))) {
+    direct = true;
+    if (!get((size_t)n_dir * (fnx + fny + fnz) * sizeof(c128), (size_t)n_chunks * n_dir * 6 * sizeof(double)))
+      return dda_fail(h, DDA_ERR_OOM, "scatter tables");
   }
-  if (h->fpart_bytes < fp_b) {
-    dev_free(h->d_fpart, h->stream); h->d_fpart = nullptr; h->fpart_bytes = 0;
-    if (dev_malloc(&h->d_fpart, fp_b) != cudaSuccess) { cudaGetLastError(); return dda_fail(h, DDA_ERR_OOM, "scatter partials"); }
-    h->fpart_bytes = fp_b;
-  }
+  const int nblk = direct || n_dir == 0 ? 0 : (n_dir + plan.cap - 1) / plan.cap;
   void* ws = h->d_tab;
-  c128* qtab = (c128*)((unsigned char*)ws + plan.bytes());
+  c128* qtab = (c128*)((unsigned char*)ws + ws_b);
   double* part = h->d_fpart;
-  double* d_F = part + 2 * qblocks;
+  double* d_F = part + part_b / sizeof(double);
   double* d_dirs = d_F + 6 * (size_t)n_dir;
   double* d_qdir = d_dirs + 3 * (size_t)n_dir;
   auto tables = [&](int b) -> cudaError_t {
-    const int d0 = b * kDirBlock, nd = std::min(n_dir - d0, kDirBlock);
+    const int d0 = b * plan.cap, nd = std::min(n_dir - d0, plan.cap);
     return farfield_tables(ws, d_dirs + 3 * (size_t)d0, nd, h->kd, fnx, fny, fnz, plan, st);
   };
   if (n_dir > 0) {
     DDA_CK(h, cudaMemcpyAsync(d_dirs, dirs, (size_t)n_dir * 3 * sizeof(double), cudaMemcpyHostToDevice, st));
-    if (nblk == 1) DDA_CK(h, tables(0));
+    if (direct) {
+      const long long tt = (long long)n_dir * (fnx + fny + fnz);
+      k_phase_tab<<<(int)std::min<long long>((tt + 255) / 256, 4096), 256, 0, st>>>(d_dirs, n_dir, h->kd, fnx, fny, fnz, (c128*)ws); count_launch();
+      DDA_CK(h, cudaGetLastError());
+    } else if (nblk == 1) {
+      DDA_CK(h, tables(0));
+    }
   }
   std::vector<double> qp(2 * qblocks);
   for (int r = 0; r < nrhs; ++r) {
@@ -331,8 +368,14 @@ int dda_scatter_internal(dda_t h, int presc, const void* P_dev, int nrhs, const 
         k_collapse_fin<<<(int)std::min<long long>((3 * fnocc + 255) / 256, 2048), 256, 0, st>>>(Qpart, G, fnocc, Qc); count_launch();
         Pf = Qc;
       }
+      if (direct) {
+        k_farfield<<<dim3(dblocks, n_chunks), 256, 0, st>>>(Pf, flat, (const c128*)ws, n_dir, fnx, fny, fnz, fnrows,
+                                                            fnocc, rows_per_chunk, part); count_launch();
+        k_farfield_fin<<<(n_dir + 127) / 128, 128, 0, st>>>(part, n_chunks, n_dir, d_dirs, h->kd, d_F); count_launch();
+        DDA_CK(h, cudaGetLastError());
+      }
       for (int b = 0; b < nblk; ++b) {
-        const int d0 = b * kDirBlock, nd = std::min(n_dir - d0, kDirBlock);
+        const int d0 = b * plan.cap, nd = std::min(n_dir - d0, plan.cap);
         if (nblk > 1) DDA_CK(h, tables(b));
         DDA_CK(h, farfield_sums(ws, Pf, flat, d_dirs + 3 * (size_t)d0, nd, h->kd, fnx, fny, fnr, fnocc, plan,
                                 d_F + 6 * (size_t)d0, st));
