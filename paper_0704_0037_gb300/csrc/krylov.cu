@@ -345,23 +345,28 @@ __global__ void k_rhs(c128* __restrict__ b, LatticeDev lat, const c128* __restri
 int launch_rhs(dda_t h, c128* b, const c128* beta, int nrhs, const double* prop, const double* pol,
                cudaStream_t st) {
   const Geom& g = h->g;
-  const int L = g.nx + g.ny + g.nz, cap = nrhs < kWaves ? nrhs : kWaves;
-  const size_t need = (size_t)L * cap * sizeof(c128);
-  if (h->ptab_bytes < need) {
+  const int L = g.nx + g.ny + g.nz;
+  const size_t one = (size_t)L * sizeof(c128);
+  int cap = nrhs < kWaves ? nrhs : kWaves;      // right-hand sides in one launch
+  if (h->ptab_bytes < cap * one) {
     dev_free(h->d_ptab, h->stream);
     h->d_ptab = nullptr;
     h->ptab_bytes = 0;
-    if (dev_malloc(&h->d_ptab, need) != cudaSuccess) {
-      h->d_ptab = nullptr;
+    if (dev_malloc(&h->d_ptab, cap * one) != cudaSuccess) {
       cudaGetLastError();
-      return dda_fail(h, DDA_ERR_OOM, "incident phase table");
+      cap = 1;                                  // memory is short: one after the other
+      if (dev_malloc(&h->d_ptab, one) != cudaSuccess) {
+        h->d_ptab = nullptr;
+        cudaGetLastError();
+        return dda_fail(h, DDA_ERR_OOM, "incident phase table");
+      }
     }
-    h->ptab_bytes = need;
+    h->ptab_bytes = cap * one;
   }
   c128* ptab = (c128*)h->d_ptab;
   const int rows_grid = (int)std::min<long long>((g.nrows + 7) / 8, 32LL * num_sms());
-  for (int r0 = 0; r0 < nrhs; r0 += kWaves) {
-    const int cnt = nrhs - r0 < kWaves ? nrhs - r0 : kWaves;
+  for (int r0 = 0; r0 < nrhs; r0 += cap) {
+    const int cnt = nrhs - r0 < cap ? nrhs - r0 : cap;
     WaveList wl{};
     for (int r = 0; r < cnt; ++r) {
       std::memcpy(wl.w[r].a, prop + 3 * (r0 + r), 3 * sizeof(double));
