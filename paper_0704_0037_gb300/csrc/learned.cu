@@ -182,65 +182,35 @@ __global__ void k_idx_map(LatticeDev lat, int nx, int ny, int nrows, int* __rest
     for (long long i = lat.row_off[row] + lane; i < lat.row_off[row + 1]; i += 32)
       map[(long long)row * nx + lat.xi[i]] = (int)i;
 }
-// A number as the unevaluated sum of two floats, and its running sum: 48 bits,
-// of which a feature keeps 24
-struct Pair {
-  float h, l;
-  __device__ __forceinline__ void add(Pair a) {
-    const float t = __fadd_rn(h, a.h), bb = __fsub_rn(t, h);
-    const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(t, bb)), __fsub_rn(a.h, bb));
-    h = t;
-    l = __fadd_rn(l, __fadd_rn(e, a.l));
-  }
-};
-// v 2^-es in integer and FP32 instructions (below 2^-126: zero)
-__device__ __forceinline__ Pair to_pair(double v, int es) {
-  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-  const int E = (int)(hi >> 20) & 0x7ff, e = E - 1023 - es;
-  const unsigned sign = hi & 0x80000000u;
-  if (E == 0x7ff || e > 127) return {__fmul_rn(__uint_as_float(sign | 0x7f800000u), (hi & 0xfffffu) | lo ? 0.0f : 1.0f), 0.0f};
-  if (E == 0 || e < -126) return {0.0f, 0.0f};
-  const float h = __uint_as_float(sign | (unsigned)(e + 127) << 23 | (hi & 0xfffffu) << 3 | lo >> 29);
-  const float u = e < -74 ? 0.0f : __uint_as_float(sign | (unsigned)(e + 75) << 23);      // 2^(e - 52)
-  return {h, __fmul_rn(__uint2float_rn(lo & 0x1fffffffu), u)};
-}
 // features at s0: channel 2c / 2c+1 = mean of Re / Im of v_c / rms over the
 // cell's children (void children count as zero), channel 6 = occupied
-// fraction; a thread per cell and component.  In FP64 the sums took 20
-// operations a thread, on the pipe that bounds the kernel (128^3 sphere: 36 us); as
-// pairs of floats, scaled by the power of two of rms, it takes 23 us, issue 80 %
-// busy, and gives the same 24 bits but for sums within 2^-22 of a rounding tie.
+// fraction; a thread per cell and component
 __global__ void __launch_bounds__(256) k_feat_in(const c128* __restrict__ v, long long n_occ,
                                                  const int* __restrict__ map, Dims dl, Dims d0,
                                                  const double* __restrict__ scl, float* __restrict__ f) {
-  const int es = (int)((unsigned)__double2hiint(scl[0]) >> 20) - 1023;       // rms = 2^es (1 to 2)
-  const Pair g = to_pair(scl[5], 3 - es);                                    // 2^es / (8 rms)
+  const double inv = scl[5] * 0.125;           // exact: a power of two
   const int c = blockIdx.y;
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < d0.n();
        p += (long long)gridDim.x * blockDim.x) {
-    const unsigned q = (unsigned)p / d0.x, X = (unsigned)p - q * d0.x, Z = q / d0.y, Y = q - Z * d0.y;   // fewer than 2^31 cells
+    const int X = (int)(p % d0.x), Y = (int)((p / d0.x) % d0.y), Z = (int)(p / ((long long)d0.x * d0.y));
     int id[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const int x = 2 * (int)X + (k & 1), y = 2 * (int)Y + ((k >> 1) & 1), z = 2 * (int)Z + (k >> 2);
+      const int x = 2 * X + (k & 1), y = 2 * Y + ((k >> 1) & 1), z = 2 * Z + (k >> 2);
       id[k] = x < dl.x && y < dl.y && z < dl.z ? map[((long long)z * dl.y + y) * dl.x + x] : -1;
     }
-    Pair re{0.0f, 0.0f}, im{0.0f, 0.0f};
+    double re = 0.0, im = 0.0;
     int occ = 0;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      if (id[k] < 0) continue;
+      if (id[k] < 0) continue;               // FP64 additions only where there are dipoles
       const c128 a = v[c * n_occ + id[k]];
       ++occ;
-      re.add(to_pair(a.x, es));
-      im.add(to_pair(a.y, es));
+      re += a.x;
+      im += a.y;
     }
-    auto mean = [&](Pair a) {
-      const float t = __fmul_rn(a.h, g.h);
-      return __fadd_rn(t, __fmaf_rn(a.l, g.h, __fmaf_rn(a.h, g.l, __fmaf_rn(a.h, g.h, -t))));
-    };
-    f[(2 * c) * d0.n() + p] = mean(re);
-    f[(2 * c + 1) * d0.n() + p] = mean(im);
+    f[(2 * c) * d0.n() + p] = (float)(re * inv);
+    f[(2 * c + 1) * d0.n() + p] = (float)(im * inv);
     if (c == 0) f[6 * d0.n() + p] = occ * 0.125f;
   }
 }

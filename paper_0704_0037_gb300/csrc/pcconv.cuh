@@ -29,7 +29,7 @@
 // split the FP32 channels it read, 0.33 ms now (48 to 16 channels at 64^3 voxels
 // 435, 121 and 96 us, 160 to 160 at 16^3 69 and 53 us between the last two);
 // the matrix pipe is 60 to 66 % busy in the large layers.  The pass 2.36, 0.50
-// and 0.44 ms; error of N(r) against 64 bits 4.5e-7 before, 1.4e-7 now.
+// and 0.45 ms; error of N(r) against 64 bits 4.5e-7 before, 1.4e-7 now.
 #pragma once
 
 #include <cuda_bf16.h>
