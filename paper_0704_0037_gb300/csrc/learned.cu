@@ -214,13 +214,13 @@ __global__ void __launch_bounds__(256) k_feat_in(const c128* __restrict__ v, lon
     if (c == 0) f[6 * d0.n() + p] = occ * 0.125f;
   }
 }
-// (double)x in integer instructions (zero for subnormal x): the sweep below is
+// (double)x, in integer instructions for zero and normal x: the sweep below is
 // bound by the FP64 pipe, which also does the conversions
 __device__ __forceinline__ double widen(float x) {
   const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
-  if (m >= 0x7f800000u) return (double)x;                      // infinity, NaN
-  const unsigned hi = m < 0x00800000u ? 0u : (m >> 3) + 0x38000000u;
-  return __hiloint2double((int)(hi | (u & 0x80000000u)), m < 0x00800000u ? 0 : (int)(u << 29));
+  if (m >= 0x7f800000u || (m < 0x00800000u && m)) return (double)x;      // infinity, NaN, subnormal
+  const unsigned hi = m ? (m >> 3) + 0x38000000u : 0u;
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
 }
 // z_i = v_i + rms * out6[.][cell(i)] for every dipole (complex128): the
 // identity plus the learned correction

@@ -74,3 +74,18 @@ def test_cell_sums_keep_the_bits_of_their_fields():
     got = (_apply(dda, torch, occ, _field_weights(2.0 ** 52), v) - v) / rms * (8 * rms)
     ref = (_apply(dda, torch, occ, _field_weights(), one) - one) / rms1 * rms1
     assert rel_l2(got, ref) <= 1e-5
+
+
+@pytest.mark.parametrize("value", [1e-40, -3e-45, 2e-38, 0.0, 1.5, np.float32(3.4e38)])
+def test_output_of_any_size_reaches_z(value):
+    """The last layer's bias alone: z = v + rms value, subnormal floats included."""
+    torch, dda = need_gpu()
+    occ = inputs.cube(5, 4, 6)
+    v = np.zeros((3, occ.size), complex)
+    v[1, 7] = 2.0
+    w = _zeros()
+    w[6][1][:] = value
+    z = _apply(dda, torch, occ, _pack(w), v)
+    rms = np.sqrt((np.abs(v) ** 2).mean())
+    b = float(np.float32(value))
+    assert (np.abs(z - (v + rms * b * (1 + 1j))) <= 1e-14 * (np.abs(v) + rms * abs(b))).all()
