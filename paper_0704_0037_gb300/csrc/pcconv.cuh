@@ -81,10 +81,16 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const unsigned (&a)[4], 
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// x = hi + mid + lo, exact for every normal float whose parts stay normal
+// x = hi + mid + lo, exact for floats of 2^-110 and more (below, mid and lo are
+// subnormal bf16: to within 2^-134).  What rounds beyond bf16's largest number is
+// truncated; infinity is hi alone (its remainder would be NaN, which the relu of
+// the next layer turns into 0).
 __device__ __forceinline__ void split3(float x, __nv_bfloat16 (&s)[3]) {
-  s[0] = __float2bfloat16_rn(x);
-  const float r = x - __bfloat162float(s[0]);
+  const unsigned u = __float_as_uint(x);
+  const unsigned m = u & 0x7fffffffu;
+  const bool inf = m == 0x7f800000u;
+  s[0] = m >= 0x7f7f8000u && m <= 0x7f800000u ? __ushort_as_bfloat16((unsigned short)(u >> 16)) : __float2bfloat16_rn(x);
+  const float r = inf ? 0.0f : x - __bfloat162float(s[0]);
   s[1] = __float2bfloat16_rn(r);
   s[2] = __float2bfloat16_rn(r - __bfloat162float(s[1]));
 }

@@ -89,3 +89,32 @@ def test_output_of_any_size_reaches_z(value):
     rms = np.sqrt((np.abs(v) ** 2).mean())
     b = float(np.float32(value))
     assert (np.abs(z - (v + rms * b * (1 + 1j))) <= 1e-14 * (np.abs(v) + rms * abs(b))).all()
+
+
+def test_infinite_activation_stays_non_finite():
+    """An overflow in the first layer, all weights positive: the output is infinite
+    (a NaN on the way would come out of the next relu as 0)."""
+    torch, dda = need_gpu()
+    occ = inputs.cube(9, 8, 10)
+    w = [(np.full_like(W, 0.01), b) for W, b in _zeros()]
+    w[0][1][3] = np.inf
+    v = inputs.random_vectors(3, 1, occ.size)[0]
+    assert not np.isfinite(_apply(dda, torch, occ, _pack(w), v)).any()
+
+
+@pytest.mark.parametrize("value", [3.4e38, 3.3895e38, 3.3e38, 1.2345678e20, 7.7e-30])
+def test_activation_up_to_the_largest_float_is_kept(value):
+    """One channel of the first layer through the skip connection, a power of two
+    and a one: values that bf16 would round to infinity keep their 24 bits."""
+    torch, dda = need_gpu()
+    occ = inputs.cube(7, 6, 5)
+    w = _zeros()
+    w[0][1][0] = value
+    scale = 2.0 ** -min(120, round(np.log2(value)))
+    w[5][0][0, 32, 1, 1, 1] = scale
+    w[6][0][:, 0] = 1.0
+    v = inputs.random_vectors(3, 1, occ.size)[0]
+    rms = np.sqrt((np.abs(v) ** 2).mean())
+    got = (_apply(dda, torch, occ, _pack(w), v) - v) / rms
+    ref = float(np.float32(value)) * scale * (1 + 1j)
+    assert np.abs(got - ref).max() <= 1e-6 * abs(ref)
