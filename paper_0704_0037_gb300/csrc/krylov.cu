@@ -870,10 +870,13 @@ __global__ void __launch_bounds__(kVT) k_bs_ts(const cpx<R>* __restrict__ t, con
   if (last_block(&s->cnt)) bs_c_fin(s, part, gridDim.x);
 }
 
-__device__ void bs_d_fin(Scal* s, const double* part, int nb) {
+// the step's end: stop test and the next direction's coefficient; *skip stays set
+// when the solve ends here (the second product of a step queued behind it)
+__device__ void bs_d_fin(Scal* s, const double* part, int nb, int* skip) {
   double f[3];
   fin_k<3>(part, kNB, 1, nb, f);
   if (threadIdx.x) return;
+  *skip = 1;
   const double r2 = f[0];
   const c128 rho = mk<double>(f[1], f[2]);
   const double res = s->half ? s->sres : sqrt(r2) / s->bnorm;
@@ -891,7 +894,7 @@ template <typename R>
 __global__ void __launch_bounds__(kVT) k_bs_xr(cpx<R>* __restrict__ x, cpx<R>* __restrict__ r,
                                                const cpx<R>* __restrict__ p, const cpx<R>* __restrict__ sv,
                                                const cpx<R>* __restrict__ t, const cpx<R>* __restrict__ rh,
-                                               long long n, Scal* s, double* part) {
+                                               long long n, Scal* s, double* part, int* skip) {
   if (s->done) return;
   const cpx<R> al = cs<R>(s->alpha), om = cs<R>(s->omega);
   double acc[3] = {0.0, 0.0, 0.0};
@@ -906,7 +909,7 @@ __global__ void __launch_bounds__(kVT) k_bs_xr(cpx<R>* __restrict__ x, cpx<R>* _
     acc[2] = fma(hx, b, fma(-hy, a, acc[2]));
   }
   block_store<3>(acc, part, 0);
-  if (last_block(&s->cnt)) bs_d_fin(s, part, gridDim.x);
+  if (last_block(&s->cnt)) bs_d_fin(s, part, gridDim.x, skip);
 }
 
 // ---------------------------------------------------------------- CGNR
@@ -1167,7 +1170,7 @@ int run_solver(Run& ru, int solver, const cpx<R>* b, cpx<R>* x, cpx<R>** vec, do
       k_bs_s<R><<<nb, kVT, 0, st>>>(r, v, sv, n, s, part, skip); count_launch();
       RK(product<R>(ru, sv, t, false, skip));
       k_bs_ts<R><<<nb, kVT, 0, st>>>(t, sv, n, s, part); count_launch();
-      k_bs_xr<R><<<nb, kVT, 0, st>>>(x, r, p, sv, t, rh, n, s, part); count_launch();
+      k_bs_xr<R><<<nb, kVT, 0, st>>>(x, r, p, sv, t, rh, n, s, part, skip); count_launch();
       return DDA_OK;
     }, [&]() {
       count_products<R>(ru, 1 + ru.hs->iters - second);
