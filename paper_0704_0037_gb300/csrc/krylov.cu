@@ -580,11 +580,15 @@ __global__ void __launch_bounds__(kVT) k_qmr_k1(const cpx<R>* __restrict__ pt, c
   pdl_launch();
   const int rr = blockIdx.y;
   pt += rr * n; v += rr * n; part += rr * kPS; s += rr;
-  if (s->done) return;
   c128 eps_new, beta;
   if (dotp) {
+    // block 0 may end the solve below while others start: one thread reads the
+    // flag, so that a block's threads go the same way
     __shared__ c128 s_eb[2];
-    __shared__ int s_status;
+    __shared__ int s_status, s_done;
+    if (threadIdx.x == 0) s_done = *(volatile int*)&s->done;
+    __syncthreads();
+    if (s_done) return;
     double a[2];
     fin_k<2>(dotp + 2LL * rr * dnb, 1, 2, dnb, a);
     if (threadIdx.x < 32) {
@@ -600,6 +604,7 @@ __global__ void __launch_bounds__(kVT) k_qmr_k1(const cpx<R>* __restrict__ pt, c
     eps_new = s_eb[0];
     beta = s_eb[1];
   } else {
+    if (s->done) return;
     eps_new = s->q.eps_new;
     beta = s->q.beta;
   }

@@ -107,3 +107,29 @@ def test_resume_refuses_another_incidence_or_a_short_buffer(sphere):
     with pytest.raises(dda.DDAError) as ei:
         dda.dda_solve(p.h, dict(opts, resume=False, checkpoint_every=8), PROP, POLS, P, 8)
     assert ei.value.status == dda.DDA_ERR_ARG
+
+
+def test_one_right_hand_side_fails_the_others_go_on(sphere):
+    """A NaN in the saved vectors of one right-hand side (in the host's image): its
+    solve ends as non-finite, the others resume bit for bit; repeatedly, since the
+    block that ends a solve does so while others of it start."""
+    torch, dda = need_gpu()
+    p = sphere
+    n = 3 * p.n_occ * 16
+    nbytes = dda.dda_checkpoint_bytes(p.h, dda.DDA_FP64, 2)
+    buf = np.zeros(nbytes, dtype=np.uint8)
+    _, info_a, P_a = _solve(p, dda.DDA_FP64, maxiter=24)
+    _solve(p, dda.DDA_FP64, maxiter=24, checkpoint_every=8, checkpoint=buf, checkpoint_stop=True)
+    head = 18 * 8 + 48                                  # incidences and the fixed header
+    bad = buf.copy()
+    vec = bad[head:head + 16 * n].view(np.float64).reshape(8, 2, 3, p.n_occ, 2)
+    vec[:6, 1, 0, 5, 0] = np.nan
+    for _ in range(10):
+        P = torch.zeros((2, 3, p.n_occ), dtype=torch.complex128, device="cuda")
+        with pytest.raises(dda.DDAError) as ei:
+            dda.dda_solve(p.h, dict(solver=dda.DDA_QMR_CS, pol=dda.DDA_LDR, prec=dda.DDA_FP64, tol=1e-16, maxiter=24,
+                                    checkpoint=bad, resume=True), PROP, POLS, P)
+        assert ei.value.status == dda.DDA_ERR_NONFINITE
+        assert torch.equal(P[0], P_a[0])
+        _, info, P = _solve(p, dda.DDA_FP64, maxiter=24, checkpoint=buf, resume=True)
+        assert torch.equal(P, P_a) and info[1]["iters"] == 24
