@@ -15,7 +15,15 @@
 // wait for the kernel before, 8.7 with the product in registers in the z pass
 // and no division per item here.  With 16 right-hand sides on a 40 x 29 x 22
 // ellipsoid the two kernels took what the four took (43.6 against 43.4 us; 37
-// now), so the line lies at the lengths whose planes fit an SM twice.
+// now), so the line lies at the lengths whose planes fit an SM twice.  A plane is
+// one block's work, and few planes with long columns leave the chip idle where the
+// passes per axis spread over it: from 64 points in y and more than 3,072 in a
+// plane, (My - 32) / 3 planes (of all right-hand sides) are fused and fewer are
+// not.  Fused against not, us: 96 x 96 points 20.6 and 16.4 (1 plane), 18.1 and
+// 15.6 (16), 19.6 and 21.6 (24); 80 x 80 15.6 and 14.3 (12), 17.4 and 16.7 (24),
+// 17.3 and 18.3 (32); 64 x 64 20.6 and 19.1 (4), 12.1 and 12.6 (12); 40 x 96 13.1
+// and 12.6 (12), 13.8 and 14.3 (20); 96 x 40 12.1 and 12.8 (12); 48 x 64 12.5 and
+// 12.8 (1); 32 x 32 10.5 and 12.5 (1).
 #include "fastfft.cuh"
 
 namespace dda {
@@ -352,7 +360,10 @@ cudaError_t launch_plane(K kernel, const FastArgs& a, int cw, Args... args) {
 }  // namespace
 }  // namespace fast
 
-bool fast_xy_supported(int Mx, int My) { return fast::xy_length(Mx) && fast::xy_length(My); }
+bool fast_xy_supported(int Mx, int My, long long planes) {
+  if (!fast::xy_length(Mx) || !fast::xy_length(My)) return false;
+  return My <= 48 || Mx * My <= 3072 || 3 * planes >= My - 32;
+}
 
 // a.in x, a.out B2, a.tw the twiddles of x, then y
 cudaError_t fast_xy_fwd_c64(const FastArgs& a) {

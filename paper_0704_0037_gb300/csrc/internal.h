@@ -357,7 +357,7 @@ cudaError_t fast_pass_c64_h(int M, int pass, const FastArgs& a);
 // x and y passes fused per z plane (fast_xy.cu, complex64): P1 and P2 (in: x,
 // out: B2), P4 and P5 (in: B2, x: x, out: y, dotp: nz partials per component);
 // tw: the twiddles of x followed by those of y
-bool fast_xy_supported(int Mx, int My);
+bool fast_xy_supported(int Mx, int My, long long planes);     // planes: nz x right-hand sides
 cudaError_t fast_xy_fwd_c64(const FastArgs& a);
 cudaError_t fast_yx_inv_c64(const FastArgs& a);
 template <typename R> cudaError_t fast_pass(int M, int pass, const FastArgs& a);

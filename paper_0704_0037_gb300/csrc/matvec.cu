@@ -344,7 +344,7 @@ cudaError_t launch_matvec(const Geom& g, const LatticeDev& lat, Work<R>& w, cons
     la.nact = 0;
   }
   // small complex64 grids: x and y passes fused per z plane
-  const bool xy = sizeof(R) == 4 && g.engine == 0 && fast_xy_supported(g.Mx, g.My);
+  const bool xy = sizeof(R) == 4 && g.engine == 0 && fast_xy_supported(g.Mx, g.My, (long long)g.nz * nrhs);
   const int dnb = xy ? 3 * g.nz : fast_xinv_blocks(la.arow ? la.nact : g.nrows, sizeof(R) == 4, g.Mx);
   if (dotp && dot_nb && fx) *dot_nb = dnb;
   // right-hand sides in chunks of the work buffers' capacity, each chunk in

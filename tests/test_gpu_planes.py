@@ -64,3 +64,32 @@ def test_planes_and_rows_without_dipoles(nrhs):
     occ[-1, :, :] = 0
     occ[-1, -1, -1] = 1
     _check(occ, nrhs)
+
+
+@pytest.mark.parametrize("mx", sorted(CELLS))
+@pytest.mark.parametrize("my", sorted(CELLS))
+def test_every_pair_of_plane_lengths_with_planes_to_fuse(mx, my):
+    """25 planes: fused whatever the lengths (7, above, are for the shorter ones)."""
+    _check(inputs.random_occupancy(CELLS[mx], CELLS[my], 25, fill=0.4, seed=mx + 2 * my), 1, (mx, my))
+
+
+@pytest.mark.parametrize("box,nrhs,fused", [((47, 45, 21), 1, False), ((47, 45, 22), 1, True), ((47, 45, 10), 2, False),
+                                            ((47, 45, 11), 2, True), ((30, 31, 10), 1, False),
+                                            ((47, 23, 1), 1, True), ((16, 46, 2), 1, True)])
+def test_line_between_fused_and_separate_passes(box, nrhs, fused):
+    """The traced passes say which way a solve's products went; the products and
+    their sums (x^T y) come from either."""
+    torch, dda = need_gpu()
+    occ = inputs.cube(*box)
+    _check(occ, nrhs)
+    with dda.Particle(occ, [1.3], 0.5) as p:
+        dda.dda_build_Dmatrix(p.h, dda.DDA_FP32_REFINED)
+        P = torch.zeros((nrhs, 3, p.n_occ), dtype=torch.complex128, device="cuda")
+        dda.dda_trace(p.h, 1)
+        st, info = dda.dda_solve_batch(p.h, dict(solver=dda.DDA_QMR_CS, pol=dda.DDA_LDR, prec=dda.DDA_FP32_REFINED,
+                                                 tol=1e-6, maxiter=200, inner_tol=1e-4), [[0.0, 0.0, 1.0]] * nrhs,
+                                       [[1.0, 0.0, 0.0]] * nrhs, P)
+        names = set(dda.dda_trace_read(p.h))
+        dda.dda_trace(p.h, 0)
+        assert st == dda.DDA_OK and all(i["rel_res_true"] < 1e-6 for i in info)
+        assert any(k.startswith("p2_") and k.endswith("c64") for k in names) != fused, names
