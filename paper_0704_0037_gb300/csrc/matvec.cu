@@ -540,6 +540,8 @@ cudaError_t tune_tiles(Geom& g, const LatticeDev& lat, Work<R>& w, cudaStream_t 
   std::array<int, 3> best{0, 0, 0};
   for (int pass = 0; pass < 3 && e == cudaSuccess; ++pass) {
     if (!has(pass == 1 ? g.Mz : g.My)) continue;       // one variant, or the Stockham passes
+    // y passes of planes that are fused for any number of right-hand sides never run
+    if (pass != 1 && std::is_same<R, float>::value && fast_xy_supported(g.Mx, g.My, g.nz)) continue;
     // the variants in turn, the least of three times two launches (six where a
     // launch is a few microseconds, not far from an event's own time): a clock
     // that still rises while the first is timed would favour the second (half

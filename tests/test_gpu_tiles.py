@@ -102,3 +102,20 @@ def test_pinned_tiles_survive_a_rebuild_and_bad_values_are_refused():
         # back to the autotuner
         dda.dda_set_pass_tiles(p.h, dda.DDA_FP32_REFINED, None)
         assert dda.dda_get_pass_tiles(p.h, dda.DDA_FP32_REFINED) == (-1, -1, -1)
+
+
+@pytest.mark.parametrize("box,passes", [((17, 33, 26), 3 + 1), ((34, 41, 3), 2)])
+def test_autotuner_times_the_passes_that_run(box, passes):
+    """Launches of a grid's first build over those of its second (choices cached):
+    2 variants x (1 + 3 x 6) launches for each pass timed: three passes in
+    double-float and in complex64 z alone, where the x and y passes are fused; the
+    two y passes in complex64, where z has no register-resident passes."""
+    torch, dda = need_gpu()
+    occ = inputs.cube(*box)
+    counts = []
+    for _ in range(2):
+        with dda.Particle(occ, [1.4], 0.3) as p:
+            dda.dda_trace(p.h, 1)
+            dda.dda_build_Dmatrix(p.h, dda.DDA_FP32_REFINED)
+            counts.append(dda.dda_trace_read(p.h)["all_launches"][1])
+    assert counts[0] - counts[1] == 38 * passes
