@@ -132,9 +132,12 @@ int dda_set_fft_engine(dda_t h, int engine);
  *        where the z pass's spectra would not fit in shared memory);
  *   1  : half as many lines per block (twice the blocks);
  *   -1 : chosen by dda_build_Dmatrix, which times both variants of each pass
- *        on the handle's own buffers (CUDA events, three launches) and takes
- *        the half tiles when they are at least 3 % faster (cached per device
- *        and grid shape).  The default.
+ *        on the handle's own buffers (in turn, the least of three times two
+ *        launches, six on small grids; CUDA events) and takes the half tiles
+ *        when they are at least 3 % faster (cached per device and grid shape).
+ *        The default.  (Where the complex64 x and y passes run fused per z
+ *        plane, on grids of up to 96 points in x and y, the y entries have no
+ *        effect.)
  * Every variant computes each line with the same arithmetic: the products
  * agree bit for bit.  dda_set_pass_tiles with tiles == NULL sets -1 for all
  * three; an entry set to 0 or 1 is kept by later builds.  dda_get_pass_tiles
@@ -492,7 +495,9 @@ int dda_farfield_noalloc(dda_t h, const void* P_dev, int n_dir, const double* di
  * reads from its half-resolution cell, times rms(r), and adds to r
  * (N(r) = r + correction: identity plus what was learned).  Training, inference
  * and the solver run in the library's own kernels; every reduction has a
- * fixed order (deterministic).
+ * fixed order (deterministic).  A network holds about 30 MB of device memory
+ * (parameters, moments, gradients, and copies of the weights in the orders the
+ * kernels read), and the activations of the largest lattice it has seen.
  */
 typedef struct dda_pcnet* dda_pcnet_t;
 
@@ -561,6 +566,8 @@ int dda_solve_pc(dda_t h, dda_pcnet_t net, const dda_solve_opts* opts, const dou
  * CUDA event pair around each launch of the product passes P1..P5, the
  * D-matrix build and the far-field kernels on the handle's stream, and
  * resets the totals; 0 stops.  Adds two event records per traced launch.
+ * Complex64 products whose x and y passes run fused per z plane record P1 and
+ * P2 as P1, P4 and P5 as P5.
  */
 int dda_trace(dda_t h, int enable);
 

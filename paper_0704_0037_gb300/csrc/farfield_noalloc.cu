@@ -1,14 +1,15 @@
 // dda_farfield_noalloc: the far-field amplitude of dda_scatter for callers
 // that must not allocate device memory.
 //
-// dda_scatter allocates its working memory (per-direction phase tables and
-// per-chunk partial sums) with cudaMalloc on first use.  Some callers cannot
+// dda_scatter allocates its working memory (phase tables of the directions, their
+// digits, partial sums) with cudaMalloc on first use.  Some callers cannot
 // let a library do that: code that runs while a CUDA stream is being
 // captured into a graph, processes whose device memory is handed out by their
 // own allocator or reserved up front, and long-running services that forbid
-// allocation after start-up.  This entry point runs the same far-field
-// kernels, but keeps their working memory in one fixed array in device
-// global memory, kFarfieldScratchBytes long, that is part of the library
+// allocation after start-up.  This entry point runs the direct FP64 sums
+// (k_farfield in scatter.cu; dda_scatter takes digit products on the tensor
+// cores, some 30 times faster at many directions), and keeps their working memory
+// in one fixed array in device global memory, kFarfieldScratchBytes long, that is part of the library
 // image: every GPU that loads the library holds it until the process exits.
 //
 // Rules of use:

@@ -1,6 +1,8 @@
 // Scattering quantities from the dipole polarizations (arXiv:0704.0037,
 // Sec. 3.1: extinction, and the Mueller matrix in one scattering plane).
-// FP64 sums throughout.  Units d = 1, kappa = kd, dimensionless P = beta x:
+// FP64 sums, but for the amplitudes, whose sums are exact digit products
+// (farfield.cu; the direct FP64 sums of k_farfield where memory is short and in
+// dda_farfield_noalloc).  Units d = 1, kappa = kd, dimensionless P = beta x:
 //   F(n)  = -i kappa^3 (I - n n) sum_j P_j exp(-i kappa n . r_j)
 //   Q_ext = (4 kappa^3 / x^2) sum_j Im(E_inc,j^* . P_j)
 //   Q_abs = (4 kappa^3 / x^2) sum_j sum_mu [-Im(1/alpha_mu) - (2/3) kappa^3] |P_mu,j|^2

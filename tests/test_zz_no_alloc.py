@@ -32,7 +32,7 @@ def test_farfield_noalloc_matches_scatter_twice():
         free = []
         for call, seed in enumerate((1, 2, 3)):
             P = torch.from_numpy(inputs.random_vectors(seed, 1, p.n_occ)).cuda()
-            # general directions (non-zero y components): dda_scatter's direct sum
+            # general directions (non-zero y components): no collapse over y in dda_scatter
             dirs = inputs.random_unit_vectors(10 + seed, 37 + 50 * call)
             F_ref, _ = dda.dda_scatter(p.h, dda.DDA_LDR, P, prop, pol, dirs)
             d_dev = torch.from_numpy(np.ascontiguousarray(dirs)).cuda()
